@@ -113,10 +113,70 @@ void host_pipe_free(hubbard_sector* H) {
     H->host_pipe = nullptr;
 }
 
+// Page-locked buffers for the a_j, b_{j+1} of the two chunks a device-resident
+// Lanczos run keeps in flight, with the events that mark them.  Page-locking
+// costs far more than a small solve and releasing it waits for the device, so
+// handles take them from a process-wide pool (by device, at most kLzPool kept)
+// and return them when they are destroyed.
+struct LzHost {
+    int device = 0;
+    double* ab[2] = {nullptr, nullptr};
+    cudaEvent_t ev[2] = {nullptr, nullptr};
+};
+
 namespace {
+
+constexpr size_t kLzPool = 64;
+std::mutex g_lz_mu;
+std::vector<LzHost*> g_lz_pool;
+
+void lz_host_delete(LzHost* p) {
+    if (p->ab[0]) cudaFreeHost(p->ab[0]);
+    for (cudaEvent_t e : p->ev)
+        if (e) cudaEventDestroy(e);
+    delete p;
+}
+
+LzHost* lz_host_take(int device) {
+    {
+        std::lock_guard<std::mutex> lk(g_lz_mu);
+        for (size_t i = 0; i < g_lz_pool.size(); ++i)
+            if (g_lz_pool[i]->device == device) {
+                LzHost* p = g_lz_pool[i];
+                g_lz_pool.erase(g_lz_pool.begin() + (ptrdiff_t)i);
+                return p;
+            }
+    }
+    LzHost* p = new (std::nothrow) LzHost;
+    if (p == nullptr) return nullptr;
+    p->device = device;
+    bool ok = cudaMallocHost((void**)&p->ab[0], 2 * 256) == cudaSuccess;
+    if (ok) p->ab[1] = p->ab[0] + 32;
+    for (cudaEvent_t& e : p->ev) ok = ok && cudaEventCreateWithFlags(&e, cudaEventDisableTiming) == cudaSuccess;
+    if (!ok) {
+        lz_host_delete(p);
+        cudaGetLastError();
+        return nullptr;
+    }
+    return p;
+}
+
+void lz_host_return(LzHost* p) {
+    if (p == nullptr) return;
+    {
+        std::lock_guard<std::mutex> lk(g_lz_mu);
+        if (g_lz_pool.size() < kLzPool) {
+            g_lz_pool.push_back(p);
+            return;
+        }
+    }
+    lz_host_delete(p);
+}
 
 void free_dev(hubbard_sector* H) {
     host_pipe_free(H);
+    lz_host_return(H->lz_host);                // no run is in flight: every run ends with its stream synchronised
+    H->lz_host = nullptr;
     for (int s = 0; s < 2; ++s) {
         H->dev[s] = DevSpin{};                 // owned by the shared entry
         H->spin_owner[s].reset();
@@ -952,8 +1012,13 @@ static int lanczos_core_host(hubbard_t H, const void* v0, int v0_dtype, int max_
                              size_t store_stride, int store_cap, const LanczosStop* stop);
 
 // The handle's device-resident Lanczos control block and a/b history for
-// cap steps (grown on demand; freed with the handle).
+// cap steps (grown on demand; freed with the handle), and its page-locked
+// buffers (returned to the pool with the handle).
 static int ensure_lz(hubbard_sector* H, int cap) {
+    if (H->lz_host == nullptr) {
+        H->lz_host = lz_host_take(H->device);
+        if (H->lz_host == nullptr) return fail(HUB_ENOMEM, "page-locked Lanczos history");
+    }
     if (H->lz != nullptr && H->lz_cap >= cap) return HUB_OK;
     dev_free(H->lz, H->mem_stream);
     H->lz = nullptr;
@@ -1001,139 +1066,113 @@ static bool lanczos_record_step(LanczosRun& R, double aj, double bn, double tol,
 //
 // Device-resident: every step's scalars (beta_j for the H*v, the deferred
 // update's coefficients, a_j and b_{j+1}) are formed and consumed on the
-// device (k_lz_finish, k_lz_finish2), so steps are enqueued in chunks with no
-// host round trip inside a chunk; after each chunk the recorded a_j, b_{j+1}
-// come back and the host runs the tridiagonal stop test on every step of it,
-// in order.  A chunk can run a few steps past the one that stops the run:
-// those steps only overwrite f, g (and stored vectors past it), never the
-// recorded values of the steps before.  The kernels and roundings are those of
-// the host-driven step, so the a_j, b_{j+1} are the same bit for bit.
-// Chunks are longer for small sectors (where a round trip costs more than a
-// step); sectors of more than 2.7e6 elements (one step per chunk) and those
-// whose H*v kernels do not fuse the reductions take the host-driven loop.
-// steps per chunk of the device-resident loop: about 4e6 / D (a round trip is
-// worth a few steps of a small sector)
+// device (close_sums3), so steps are enqueued in chunks with no host round
+// trip, and while the host runs the tridiagonal stop test on the recorded a_j,
+// b_{j+1} of one chunk, step by step and in order, the next one is already
+// enqueued.  A run can go up to two chunks past the step that stops it: those
+// steps only overwrite vectors past it, never the recorded values of the steps
+// before.  The kernels and roundings are those of the host-driven step, so the
+// a_j, b_{j+1} are the same bit for bit.  A step whose fused sums cancel
+// (near breakdown) stalls the ones behind it; the host then runs the explicit
+// branch and enqueues them again.
+// Steps per chunk: two chunks cover the host's test of one (a few us a step),
+// and the steps past the end stay few.
 static int lanczos_chunk(hubbard_t H) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(16, (int64_t)(4e6 / (double)H->D)));
+    return (int)std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(4e6 / (double)H->D)));
 }
 
-// whether lanczos_core takes the host-driven loop: one step per round trip
-// gains nothing over it (its explicit branch costs no launches when unused;
-// same results either way), and it needs fused reductions and the scratch
+// whether lanczos_core takes the host-driven loop: above 2.5e7 elements a step
+// takes half a millisecond, and the round trip it would save less than the one
+// or two steps run past the end; and it needs fused reductions and the scratch
 static bool lanczos_host_driven(hubbard_t H, int dtype) {
-    return lanczos_chunk(H) == 1 || !hv_phases_fuse(H, dtype) || H->fx_bytes < (size_t)H->D * 16;
+    return H->D > 25000000 || !hv_phases_fuse(H, dtype) || H->fx_bytes < (size_t)H->D * 16;
 }
 
 static int lanczos_core(hubbard_t H, const void* v0, int v0_dtype, int max_iters, double tol, int dtype, void* f,
                         void* g, cudaStream_t s, LanczosRun& R, double rel_tol = 0.0, char* store = nullptr,
                         size_t store_stride = 0, int store_cap = 0, const LanczosStop* stop = nullptr) {
-    const int chunk = lanczos_chunk(H);
     if (lanczos_host_driven(H, dtype))
         return lanczos_core_host(H, v0, v0_dtype, max_iters, tol, dtype, f, g, s, R, rel_tol, store, store_stride,
                                  store_cap, stop);
     int rc;
+    const int chunk = lanczos_chunk(H);
     const int m_cap = (int)std::min<int64_t>(max_iters, H->D);
     if ((rc = ensure_lz(H, m_cap))) return rc;
     LzDev* dv = reinterpret_cast<LzDev*>(H->lz);
-    double* ha = reinterpret_cast<double*>((char*)H->lz + 256);
-    double* hb = ha + H->lz_cap;
+    double* hist = reinterpret_cast<double*>((char*)H->lz + 256);
+    LzHost* pin = H->lz_host;
     double n0 = 0.0;
     if ((rc = launch_dot(H, v0, v0, H->D, v0_dtype, H->red, s)) || (rc = reduce_partials_host(H->red, s, &n0))) return rc;
     n0 = std::sqrt(n0);
     if (!(n0 > 0.0) || !std::isfinite(n0)) return fail(HUB_EINVAL, "start vector has zero or non-finite norm");
-    if (v0_dtype == dtype) rc = launch_copy_normalise(v0, f, H->D, dtype, 1.0 / n0, s);
-    else rc = launch_f64_to_f32_scaled((const double*)v0, (float*)f, H->D, 1.0 / n0, s);
+    // f_j lives in its slot of the store, past the last slot in f and g by turns;
+    // step j writes H f_j - b_j f_{j-1} where f_{j+1} will be completed
+    auto vec = [&](int j) -> void* {
+        if (j < store_cap) return store + (size_t)j * store_stride;
+        return (j & 1) ? g : f;
+    };
+    if (v0_dtype == dtype) rc = launch_copy_normalise(v0, vec(0), H->D, dtype, 1.0 / n0, s);
+    else rc = launch_f64_to_f32_scaled((const double*)v0, (float*)vec(0), H->D, 1.0 / n0, s);
     if (rc) return rc;
-    const size_t vbytes = (size_t)H->D * elem_size(dtype);
-    if (store_cap > 0 && cudaMemcpyAsync(store, f, vbytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-        return fail(HUB_ECUDA, "store f_0");
-    if (cudaMemsetAsync(g, 0, vbytes, s) != cudaSuccess) return fail(HUB_ECUDA, "memset");
-    const LzDev init{0.0, 0.0, 1.0, 0.0, 0, 1, {0, 0}};
+    if (cudaMemsetAsync(vec(1), 0, (size_t)H->D * elem_size(dtype), s) != cudaSuccess) return fail(HUB_ECUDA, "memset");
+    const LzDev init{0.0, 0.0, 1.0, 0.0, 0, 1, 0, 0};
     if (cudaMemcpyAsync(dv, &init, sizeof(init), cudaMemcpyHostToDevice, s) != cudaSuccess)
         return fail(HUB_ECUDA, "Lanczos control upload");
-    std::vector<double> ab(2 * (size_t)chunk);
-    // one Lanczos step: g <- H f_j - b_j g with f_j completed from the previous
-    // step inside the row phase, then the explicit branch (a no-op when fused)
-    auto step = [&](void* fj, void* gj, bool first, uint64_t& launches, cudaStream_t st) -> int {
-        const uint64_t c0 = hubbard_kernel_launches();
-        RowUpdate upd{gj, 0.0, 1.0, dv};
+    // one Lanczos step: f_j is completed from the previous step on the way
+    auto step = [&](int j) -> int {
+        RowUpdate upd{j > 0 ? vec(j - 1) : nullptr, 0.0, 1.0, dv};
         bool fused = false;
-        int r = launch_hv_fast(H, fj, gj, dtype, 0.0, gj, 1023, st, H->red, &fused, first ? nullptr : &upd, dv, ha, hb);
+        int r = launch_hv_fast(H, vec(j), vec(j + 1), dtype, 0.0, j > 0 ? vec(j - 1) : vec(1), 1023, s, H->red, &fused,
+                               j > 0 ? &upd : nullptr, dv, hist);
         if (r == HUB_OK && !fused) r = fail(HUB_ECUDA, "device-resident Lanczos: fused reductions unavailable");
-        if (r == HUB_OK) r = launch_lz_explicit(dv, fj, gj, H->D, dtype, H->red, hb, st);
-        launches = hubbard_kernel_launches() - c0;
         return r;
     };
-    // Small sectors are bound by kernel launches: with no vectors to store, the
-    // steps of either parity (f, g or g, f) are the same launches every time, so
-    // each is captured once as a CUDA graph (after one step run directly, which
-    // also settles every kernel attribute) and replayed on the caller's stream.
-    // Capture runs on a private stream (the legacy default stream cannot be
-    // captured); nothing executes during capture.
-    bool graphs = chunk > 1 && store_cap == 0 && m_cap > 4 && hv_phases_capturable(H, dtype);
-    cudaGraphExec_t gx[2] = {nullptr, nullptr};
-    uint64_t glaunch[2] = {0, 0};
-    cudaStream_t cap = nullptr;
-    if (graphs && cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking) != cudaSuccess) {
-        cudaGetLastError();
-        graphs = false;
-    }
-    struct GraphGuard {
-        cudaGraphExec_t* g;
-        cudaStream_t cap;
-        ~GraphGuard() {
-            for (int i = 0; i < 2; ++i)
-                if (g[i]) cudaGraphExecDestroy(g[i]);
-            if (cap) cudaStreamDestroy(cap);
-        }
-    } gguard{gx, cap};
-    int j = 0;
-    bool done = false;
-    while (!done && j < m_cap) {
-        const int j0 = j;
-        const int j1 = std::min(m_cap, j0 + chunk);
-        for (; j < j1; ++j) {
-            const int par = j & 1;
-            if (graphs && j >= 1 && gx[par] == nullptr) {
-                cudaGraph_t gr = nullptr;
-                const cudaError_t e0 = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-                if (e0 != cudaSuccess) return cuda_fail(e0, "Lanczos step capture");
-                uint64_t n = 0;
-                const int r = step(f, g, false, n, cap);
-                const cudaError_t e = cudaStreamEndCapture(cap, &gr);
-                if (r != HUB_OK) {
-                    if (gr) cudaGraphDestroy(gr);
-                    return r;
-                }
-                if (e != cudaSuccess) return cuda_fail(e, "Lanczos step capture");
-                const cudaError_t e2 = cudaGraphInstantiate(&gx[par], gr, 0);
-                cudaGraphDestroy(gr);
-                if (e2 != cudaSuccess) return cuda_fail(e2, "Lanczos step graph");
-                glaunch[par] = n;
-                count_launches(-(int)n);              // captured, not run: counted at each replay
-            }
-            if (graphs && j >= 1) {
-                if (cudaGraphLaunch(gx[par], s) != cudaSuccess) return fail(HUB_ECUDA, "Lanczos step graph launch");
-                count_launches((int)glaunch[par]);
-            } else {
-                uint64_t n = 0;
-                if ((rc = step(f, g, j == 0, n, s))) return rc;
-            }
-            // f holds the final f_j from here on
-            if (j >= 1 && j < store_cap &&
-                cudaMemcpyAsync(store + (size_t)j * store_stride, f, vbytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
-                return fail(HUB_ECUDA, "store f_j");
-            std::swap(f, g);
-        }
-        // the recorded a_j, b_{j+1} of the chunk, then the stop tests step by step
-        if (cudaMemcpyAsync(ab.data(), ha + j0, (size_t)(j1 - j0) * sizeof(double), cudaMemcpyDeviceToHost, s) !=
-                cudaSuccess ||
-            cudaMemcpyAsync(ab.data() + chunk, hb + j0, (size_t)(j1 - j0) * sizeof(double), cudaMemcpyDeviceToHost,
-                            s) != cudaSuccess)
+    struct Drain {                                   // no copy into the pooled buffers outlives the run
+        cudaStream_t s;
+        ~Drain() { cudaStreamSynchronize(s); }
+    } drain{s};
+    struct Chunk { int j0, j1; } inflight[2];
+    int n_in = 0, next = 0, slot = 0;                // chunks in flight, next step to enqueue, their buffer
+    // enqueues a chunk and the copy of its history
+    auto enqueue = [&]() -> int {
+        const int j0 = next, j1 = std::min(m_cap, j0 + chunk);
+        for (int j = j0; j < j1; ++j)
+            if (int r = step(j)) return r;
+        const int b = (slot + n_in) & 1;
+        if (cudaMemcpyAsync(pin->ab[b], hist + 2 * j0, 2 * (size_t)(j1 - j0) * sizeof(double), cudaMemcpyDeviceToHost,
+                            s) != cudaSuccess ||
+            cudaEventRecord(pin->ev[b], s) != cudaSuccess)
             return fail(HUB_ECUDA, "Lanczos history download");
-        if (cudaStreamSynchronize(s) != cudaSuccess) return fail(HUB_ECUDA, "lanczos synchronise");
-        for (int q = 0; q < j1 - j0 && !done; ++q)
-            done = lanczos_record_step(R, ab[(size_t)q], ab[(size_t)chunk + q], tol, rel_tol, stop);
+        inflight[b] = Chunk{j0, j1};
+        ++n_in;
+        next = j1;
+        return HUB_OK;
+    };
+    bool done = false;
+    while (!done) {
+        while (n_in < 2 && next < m_cap)
+            if ((rc = enqueue())) return rc;
+        if (n_in == 0) break;
+        if (cudaEventSynchronize(pin->ev[slot]) != cudaSuccess) return fail(HUB_ECUDA, "lanczos synchronise");
+        const Chunk c = inflight[slot];
+        const double* ab = pin->ab[slot];
+        for (int j = c.j0; j < c.j1 && !done; ++j) {
+            double aj = ab[2 * (j - c.j0)], bn = ab[2 * (j - c.j0) + 1];
+            if (bn < 0.0) {
+                // stalled: nothing behind step j has run
+                if ((rc = launch_lz_explicit(dv, vec(j), vec(j + 1), H->D, dtype, H->red, hist, s))) return rc;
+                if (cudaMemcpyAsync(&bn, hist + 2 * j + 1, sizeof(double), cudaMemcpyDeviceToHost, s) != cudaSuccess ||
+                    cudaStreamSynchronize(s) != cudaSuccess)
+                    return fail(HUB_ECUDA, "lanczos synchronise");
+                next = j + 1;
+                n_in = 1;                            // the chunk behind is enqueued again
+                done = lanczos_record_step(R, aj, bn, tol, rel_tol, stop);
+                break;
+            }
+            done = lanczos_record_step(R, aj, bn, tol, rel_tol, stop);
+        }
+        slot ^= 1;
+        --n_in;
     }
     if (tol <= 0.0 && rel_tol <= 0.0) R.converged = true;
     if (cudaStreamSynchronize(s) != cudaSuccess) return fail(HUB_ECUDA, "lanczos synchronise");

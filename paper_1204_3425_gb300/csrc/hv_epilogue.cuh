@@ -135,6 +135,26 @@ __device__ __forceinline__ void add4(int2& A, int2 a, int2 b, int2 c, int2 d) {
 __device__ __forceinline__ void add4(int2& A, int2 a) { A.x += a.x; A.y += a.y; }
 
 
+// Lanczos reductions fused into the up-phase epilogue (Algorithm 1): each
+// thread accumulates <w, f>, <w, w> and <f, f> over its outputs in a fixed
+// order, the CTA sums its threads in a fixed tree, and the per-CTA partials
+// (part[b], part[kPartStride + b], part[2 kPartStride + b]) are summed in
+// index order afterwards, so the result is deterministic.  binary32 outputs
+// use a float-float accumulator (exact product split + TwoSum), as the
+// stand-alone dot kernel does.
+struct FFAcc {
+    float hi = 0.0f, lo = 0.0f;
+    __device__ __forceinline__ void add_product(float x, float y) {
+        const float p = x * y;
+        const float e = fmaf(x, y, -p);
+        const float t = hi + p;
+        const float bb = t - hi;
+        lo += ((hi - (t - bb)) + (p - bb)) + e;
+        hi = t;
+    }
+    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
+};
+
 // Lanczos reductions fused into the up-phase epilogue (Algorithm 1): the CTA
 // sums its threads' <w, f>, <w, w>, <f, f> in a fixed tree and stores the
 // per-CTA partials at part[b], part[kPartStride + b], part[2 kPartStride + b].
@@ -167,6 +187,72 @@ __device__ __forceinline__ void block_sum3_store(double a, double b, double c, d
             part[kPartStride + blockIdx.x] = b;
             part[2 * kPartStride + blockIdx.x] = c;
         }
+    }
+}
+
+// Device-resident Lanczos step control (Algorithm 1): the step in progress is
+// closed with beta_{j+1}; the next step's H*v then reads beta = beta_{j+1} and
+// completes f_{j+1} = (g + ua f_j) * uinv while staging its rows: ua = -a_j
+// when g still holds H f_j - beta_j f_{j-1} (fused sums), 0 when the explicit
+// branch already subtracted a_j f_j.  The roundings are those of the host-driven
+// step (sqrt and the division are correctly rounded on both sides).
+__device__ __forceinline__ void lz_close_step(LzDev* dv, double* hist, double bn, bool fused) {
+    const int j = dv->j;
+    hist[2 * j + 1] = bn;
+    dv->stall = 0;
+    dv->ua = fused ? -dv->a : 0.0;
+    dv->uinv = 1.0 / bn;
+    dv->beta = bn;
+    dv->j = j + 1;
+}
+
+// Closes a fused reduction inside the kernel that made its partials: the CTA
+// that stores its partials last (done counts the nb CTAs and returns to 0) sums
+// them all in index order into part[kRedSlots-1 .. kRedSlots-3] and, for a
+// device-resident step, forms a_j and, unless the difference
+// <w,w> - 2a^2 + a^2 <f,f> cancels more than six digits, beta_{j+1}.  (When it
+// does, the step stalls: kernels enqueued behind it return at once and the host,
+// which finds the mark in the history, runs the explicit branch.)  A kernel
+// of its own for this took 8-9 us of a 40-70 us step on the small sectors.
+__device__ __forceinline__ void close_sums3(double* part, int nb, unsigned* done, LzDev* dv, double* hist) {
+    __shared__ int last;
+    __shared__ double fin[3][32];
+    if (threadIdx.x == 0) {
+        __threadfence();                                  // this CTA's partials before its count
+        last = atomicInc(done, (unsigned)nb - 1u) == (unsigned)nb - 1u;
+    }
+    __syncthreads();
+    if (!last) return;
+    __threadfence();
+    double s[3] = {0.0, 0.0, 0.0};
+    for (int i = threadIdx.x; i < nb; i += blockDim.x)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) s[q] += __ldcg(part + q * kPartStride + i);
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+        if (lane == 0) fin[q][wid] = s[q];
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) {
+        s[q] = fin[q][0];
+        for (int i = 1; i < nw; ++i) s[q] += fin[q][i];
+        part[kRedSlots - 1 - q] = s[q];
+    }
+    if (dv == nullptr) return;
+    const double a = s[0], b2 = s[1] - 2.0 * a * a + a * a * s[2];
+    const int fused = b2 > 1e-6 * s[1];
+    dv->a = a;
+    dv->fused = fused;
+    hist[2 * dv->j] = a;
+    if (fused) {
+        lz_close_step(dv, hist, sqrt(fmax(b2, 0.0)), true);
+    } else {
+        hist[2 * dv->j + 1] = -1.0;                       // no beta is negative: the host runs the explicit branch
+        dv->stall = 1;
     }
 }
 

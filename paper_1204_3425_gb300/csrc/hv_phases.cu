@@ -64,6 +64,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
     using S = typename FxVec<VEC>::T;
     if constexpr (UPD) {
         if (dv != nullptr) {                              // device-resident step: the update's scalars
+            if (dv->stall) return;
             ua = dv->ua;
             uinv = dv->uinv;
         }
@@ -221,26 +222,6 @@ __device__ __forceinline__ void uniform_hops(const uint32_t* __restrict__ list, 
     }
 }
 
-// Lanczos reductions fused into the up-phase epilogue (Algorithm 1): each
-// thread accumulates <w, f>, <w, w> and <f, f> over its outputs in a fixed
-// order, the CTA sums its threads in a fixed tree, and the per-CTA partials
-// (part[b], part[kPartStride + b], part[2 kPartStride + b]) are summed in
-// index order afterwards, so the result is deterministic.  binary32 outputs
-// use a float-float accumulator (exact product split + TwoSum), as the
-// stand-alone dot kernel does.
-struct FFAcc {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add_product(float x, float y) {
-        const float p = x * y;
-        const float e = fmaf(x, y, -p);
-        const float t = hi + p;
-        const float bb = t - hi;
-        lo += ((hi - (t - bb)) + (p - bb)) + e;
-        hi = t;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 // Up phase, binary64 fixed point (Algorithms 2 and 4):
 //   W[u, c] = -t (sum_{(u', s) in hops_up(u)} s X[u', c] + Y[u, c]) + U n(u, c) X[u, c]  [- beta w_old]
 // Row u of W is a signed combination of whole rows u' of X (Eq. H-Kroneckersum),
@@ -371,7 +352,8 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                                                      const uint32_t* __restrict__ sd, EpiParams ep,
                                                      const int* __restrict__ emax_p, int fixed_emax,
                                                      const double* __restrict__ fv, double* part,
-                                                     const LzDev* __restrict__ dv) {
+                                                     unsigned* done, LzDev* dv, double* hist) {
+    if (dv != nullptr && dv->stall) return;
     double s1 = 0.0, s2 = 0.0, s3 = 0.0;
     using IV = typename FxVec<VPL>::T;
     __shared__ long long Bs[33];
@@ -489,6 +471,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
         }
     }
     block_sum3_store(s1, s2, s3, part);
+    close_sums3(part, gridDim.x, done, dv, hist);
 }
 
 __device__ __forceinline__ void addf(float& A, float a, float b, float c, float d) { A += (a + b) + (c + d); }
@@ -520,7 +503,8 @@ __global__ void __launch_bounds__(256, up32_ctas<VPL, RED>()) k_up_f32(const flo
                                                     const uint32_t* __restrict__ list,
                                                     const uint32_t* __restrict__ su,
                                                     const uint32_t* __restrict__ sd, float mt, float U, float mbeta,
-                                                    double* part, const LzDev* __restrict__ dv) {
+                                                    double* part, unsigned* done, LzDev* dv, double* hist) {
+    if (dv != nullptr && dv->stall) return;
     FFAcc s1, s2, s3;
     if (dv != nullptr) mbeta = (float)-dv->beta;          // device-resident step: beta_j on the device
     using V = typename F32Vec<VPL>::T;
@@ -582,7 +566,10 @@ __global__ void __launch_bounds__(256, up32_ctas<VPL, RED>()) k_up_f32(const flo
             }
         }
     }
-    if constexpr (RED) block_sum3_store(s1.value(), s2.value(), s3.value(), part);
+    if constexpr (RED) {
+        block_sum3_store(s1.value(), s2.value(), s3.value(), part);
+        close_sums3(part, gridDim.x, done, dv, hist);
+    }
 }
 
 // ---------------------------------------------------------------------------
@@ -599,6 +586,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f32(std::conditional_t<UPD, fl
     using S = typename F32Vec<VEC>::T;
     if constexpr (UPD) {
         if (dv != nullptr) {
+            if (dv->stall) return;
             ua = (float)dv->ua;
             uinv = (float)dv->uinv;
         }
@@ -756,21 +744,16 @@ bool hv_phases_fuse(const hubbard_sector* H, int dtype) {
     return dtype == HUB_F64 || choose_vec(H->vec_rows, H->Ddn, 4, 4, 0) != 0;
 }
 
-bool hv_phases_capturable(const hubbard_sector* H, int dtype) {
-    // the binary64 path for rows longer than shared memory uploads its fixed
-    // exponent word from host memory on each call
-    return hv_phases_fuse(H, dtype) && (dtype == HUB_F32 || choose_vec(H->vec_rows, H->Ddn, 8, 2, 0) != 0);
-}
-
 int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, double beta, const void* w_old,
                      void* ybuf, int fixed_emax, cudaStream_t s, double* part, int* nparts,
-                     const RowUpdate* upd, const LzDev* dv) {
+                     const RowUpdate* upd, LzDev* dv, double* hist) {
     if (nparts != nullptr) *nparts = 0;
     if (sms() * 5 > kPartStride) part = nullptr;        // partial arrays too short: no fused reduction
     const DevSpin& up = H->dev[0];
     const DevSpin& dn = H->dev[1];
     const int64_t Dup = H->Dup, Ddn = H->Ddn;
     const bool dn16 = dn.ent16 != nullptr;
+    unsigned* done = reinterpret_cast<unsigned*>(H->status + 3);
     // up-phase CTAs: as many as the launch bounds keep resident (the phase is
     // bound by L2 latency, so occupancy is what counts: 4 per SM at <= 64
     // registers for binary64 (3 for the Lanczos variant, whose prefetched
@@ -848,7 +831,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         (const double*)w_old, Dup, Ddn,                                                                    \
         up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax)
 #define UP64_R(V, F)                                                                                        \
-    if (part != nullptr) { UP64(k_up_step_f64x, V, F), (const double*)v, part, dv); }                      \
+    if (part != nullptr) { UP64(k_up_step_f64x, V, F), (const double*)v, part, done, dv, hist); }                      \
     else if (V == 2 && pre) { UP64P(V, F, 3); }                                                            \
     else { UP64(k_up_f64x, V, F)); }
         if (vpl == 2) {
@@ -894,11 +877,11 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         if (part != nullptr)                                                                               \
             k_up_f32<V, true><<<up_grid, 256, 0, s>>>((const float*)v, Y, (float*)w, (const float*)w_old,  \
                 Dup, Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t,           \
-                (float)H->U, (float)-beta, part, dv);                                                      \
+                (float)H->U, (float)-beta, part, done, dv, hist);                                                   \
         else                                                                                               \
             k_up_f32<V, false><<<up_grid, 256, 0, s>>>((const float*)v, Y, (float*)w, (const float*)w_old, \
                 Dup, Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t,           \
-                (float)H->U, (float)-beta, part, nullptr);                                                 \
+                (float)H->U, (float)-beta, part, done, nullptr, nullptr);                                                \
     }
     if (vpl == 4) { UP32(4) } else if (vpl == 2) { UP32(2) } else { UP32(1) }
 #undef UP32

@@ -100,6 +100,8 @@ namespace hub {
 struct SpinEntry;
 // Device staging and streams of hubbard_apply_host (allocated on first use).
 struct HostPipe;
+// Page-locked history buffers and events of a device-resident Lanczos run.
+struct LzHost;
 }
 
 struct hubbard_sector {
@@ -125,6 +127,7 @@ struct hubbard_sector {
     // device-resident Lanczos control (LzDev) and a/b history for lz_cap steps
     void* lz = nullptr;
     int lz_cap = 0;
+    struct hub::LzHost* lz_host = nullptr;     // page-locked copies of a chunk's history, from a process-wide pool
     // stream of the handle's own allocations (nullptr: cudaMalloc / cudaFree;
     // set by sector_create_streamed for handles that live on one stream)
     cudaStream_t mem_stream = nullptr;
@@ -149,15 +152,16 @@ int sector_create_streamed(int Ns, const int32_t* bonds, int n_bonds, int Nup, i
 int batch_create_streamed(const hubbard_sector_desc* sectors, int n_sectors, cudaStream_t ms, hubbard_batch_t* out);
 
 // Device-resident control of a Lanczos run (Algorithm 1 steps enqueued without
-// a host round trip): the scalars the next step's kernels read, written by the
-// one-CTA kernels that close each step (k_lz_finish, k_lz_finish2).
+// a host round trip): the scalars the next step's kernels read, written
+// where a step is closed (close_sums3, k_lz_finish2).
 struct LzDev {
     double beta;      // b_j: coefficient of w_old (= f_{j-1}) in the next H*v
     double ua, uinv;  // the next row phase's deferred update f <- (f + ua fo) * uinv
     double a;         // a_j of the step in progress
     int j;            // steps closed so far (index of the step in progress)
     int fused;        // the step in progress took beta^2 from the fused sums
-    int pad[2];
+    int stall;        // the step in progress waits for the explicit branch: kernels enqueued behind it return at once
+    int pad;
 };
 
 // A Lanczos vector update deferred into the next H*v (Algorithm 1, the
@@ -180,28 +184,25 @@ int launch_hv_reference(const hubbard_sector* H, const void* v, void* w, int dty
 // not support it).
 // upd != nullptr: v is first updated in place as RowUpdate describes.
 // dv != nullptr (device-resident step): beta is read on the device from
-// dv->beta, and the fused sums are closed by k_lz_finish into dv and the
-// history arrays ha, hb (requires part).
+// dv->beta, and the fused sums are closed into dv and the history hist
+// (a_j at 2 j, b_{j+1} at 2 j + 1; requires part).
 int launch_hv_fast(hubbard_sector* H, const void* v, void* w, int dtype, double beta,
                    const void* w_old, int fixed_emax, cudaStream_t s, double* part = nullptr,
                    bool* fused = nullptr, const RowUpdate* upd = nullptr, LzDev* dv = nullptr,
-                   double* ha = nullptr, double* hb = nullptr);
+                   double* hist = nullptr);
 // hv_phases.cu: two-phase shared-memory H*v; -1 when the staging buffers do not fit.
 // fixed_emax > 0 fixes the fixed-point exponent bound (vectors of norm <= 1:
 // 1023); otherwise it is computed from v and w_old.
 // part != nullptr: the up phase writes per-CTA partials of <w, v>, <w, w> and
-// <v, v> at part[b], part[kPartStride + b], part[2 kPartStride + b];
-// *nparts = their count (<= kPartStride).
+// <v, v> at part[b], part[kPartStride + b], part[2 kPartStride + b]
+// (*nparts = their count, <= kPartStride) and closes them (close_sums3).
 // upd != nullptr: v is first updated in place (fused into the row phase where
 // it stages rows in shared memory); -1 is returned before anything is launched.
 int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, double beta, const void* w_old,
                      void* ybuf, int fixed_emax, cudaStream_t s, double* part = nullptr, int* nparts = nullptr,
-                     const RowUpdate* upd = nullptr, const LzDev* dv = nullptr);
+                     const RowUpdate* upd = nullptr, LzDev* dv = nullptr, double* hist = nullptr);
 // whether launch_hv_phases fuses the Lanczos reductions for this sector and dtype
 bool hv_phases_fuse(const hubbard_sector* H, int dtype);
-// whether a fused launch_hv_phases call with a fixed exponent bound enqueues
-// only kernels (no host-memory copies), so a CUDA graph can capture it
-bool hv_phases_capturable(const hubbard_sector* H, int dtype);
 // max biased binary64 exponent of |v| folded into *emax (atomicMax; caller zeroes it)
 void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s);
 // binary64 -> (lo, hi) fixed point with the exponent bound *emax (read on the device)
@@ -215,13 +216,10 @@ int reduce_partials3_host(double* partials, cudaStream_t s, double out[3]);
 // (dv != nullptr: a and inv read on the device from dv->ua, dv->uinv)
 int launch_axpy_scale(double a, double inv, const void* x, void* y, int64_t n, int dtype, cudaStream_t s,
                       const LzDev* dv = nullptr);
-// the explicit branch of a device-resident step: when dv->fused is 0,
-// y <- y - dv->a x with partial sums of y^2 in partials, then k_lz_finish2
-// sums them and closes the step (no-ops when the step was closed fused)
-int launch_lz_explicit(LzDev* dv, const void* x, void* y, int64_t n, int dtype, double* partials, double* hb,
+// the explicit branch of a device-resident step whose fused sums cancelled
+// (dv->stall): y <- y - dv->a x with partial sums of y^2, which close the step
+int launch_lz_explicit(LzDev* dv, const void* x, void* y, int64_t n, int dtype, double* partials, double* hist,
                        cudaStream_t s);
-// k_lz_finish: the fused sums of an up phase (np per-CTA partials) closed into dv, ha, hb
-int launch_lz_finish(double* part, int np, LzDev* dv, double* ha, double* hb, cudaStream_t s);
 int launch_axpy(double a, const void* x, void* y, int64_t n, int dtype, cudaStream_t s);
 int launch_axpy_nrm2(double a, const void* x, void* y, int64_t n, int dtype, double* partials,
                      cudaStream_t s);

@@ -12,6 +12,7 @@
 
 #include "internal.h"
 #include "splitmix.cuh"
+#include "hv_epilogue.cuh"
 
 namespace hub {
 
@@ -258,6 +259,7 @@ __global__ void k_scale(T a, T* __restrict__ y, int64_t n) {
 __global__ void k_axpy_scale_f64(double a, double inv, const double* __restrict__ x, double* __restrict__ y,
                                  int64_t n, const LzDev* __restrict__ dv) {
     if (dv != nullptr) {
+        if (dv->stall) return;
         a = dv->ua;
         inv = dv->uinv;
     }
@@ -267,51 +269,12 @@ __global__ void k_axpy_scale_f64(double a, double inv, const double* __restrict_
 __global__ void k_axpy_scale_f32(float a, float inv, const float* __restrict__ x, float* __restrict__ y, int64_t n,
                                  const LzDev* __restrict__ dv) {
     if (dv != nullptr) {
+        if (dv->stall) return;
         a = (float)dv->ua;
         inv = (float)dv->uinv;
     }
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         y[i] = fmaf(a, x[i], y[i]) * inv;
-}
-
-// Device-resident Lanczos step control (Algorithm 1): the step in progress is
-// closed with beta_{j+1}; the next step's H*v then reads beta = beta_{j+1} and
-// completes f_{j+1} = (g + ua f_j) * uinv while staging its rows: ua = -a_j
-// when g still holds H f_j - beta_j f_{j-1} (fused sums), 0 when the explicit
-// branch already subtracted a_j f_j.  The roundings are those of the host-driven
-// step (sqrt and the division are correctly rounded on both sides).
-__device__ __forceinline__ void lz_close_step(LzDev* dv, double* hb, double bn, bool fused) {
-    const int j = dv->j;
-    hb[j] = bn;
-    dv->ua = fused ? -dv->a : 0.0;
-    dv->uinv = 1.0 / bn;
-    dv->beta = bn;
-    dv->j = j + 1;
-}
-
-// the three fused sums in the order of k_finish_sum3, then a_j and, unless the
-// difference <w,w> - 2a^2 + a^2 <f,f> cancels more than six digits, beta_{j+1}
-__global__ void k_lz_finish(double* partials, int nb, LzDev* dv, double* ha, double* hb) {
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        a += partials[i];
-        b += partials[kPartStride + i];
-        c += partials[2 * kPartStride + i];
-    }
-    a = block_sum(a);
-    b = block_sum(b);
-    c = block_sum(c);
-    if (threadIdx.x == 0) {
-        partials[kRedSlots - 1] = a;
-        partials[kRedSlots - 2] = b;
-        partials[kRedSlots - 3] = c;
-        const double b2 = b - 2.0 * a * a + a * a * c;
-        const int fused = b2 > 1e-6 * b;
-        dv->a = a;
-        dv->fused = fused;
-        ha[dv->j] = a;
-        if (fused) lz_close_step(dv, hb, sqrt(fmax(b2, 0.0)), true);
-    }
 }
 
 // explicit branch: y <- y - a x and partial sums of y^2, as k_axpy_nrm2_*
@@ -342,14 +305,14 @@ __global__ void k_lz_axpy_nrm2_f32(const LzDev* __restrict__ dv, const float* __
     if (threadIdx.x == 0) partials[blockIdx.x] = s;
 }
 // sums the explicit branch's partials in the order of k_finish_sum, closes the step
-__global__ void k_lz_finish2(double* partials, int nb, LzDev* dv, double* hb) {
+__global__ void k_lz_finish2(double* partials, int nb, LzDev* dv, double* hist) {
     if (dv->fused) return;
     double s = 0.0;
     for (int i = threadIdx.x; i < nb; i += blockDim.x) s += partials[i];
     s = block_sum(s);
     if (threadIdx.x == 0) {
         partials[kRedSlots - 1] = s;
-        lz_close_step(dv, hb, sqrt(fmax(s, 0.0)), false);
+        lz_close_step(dv, hist, sqrt(fmax(s, 0.0)), false);
     }
 }
 
@@ -494,25 +457,6 @@ __global__ void k_finish_sum(double* partials, int nb) {
     if (threadIdx.x == 0) partials[kRedSlots - 1] = s;
 }
 
-// the three arrays of a fused reduction (part[q kPartStride .. + nb)), each
-// summed in a fixed order, into part[kRedSlots-1-q]
-__global__ void k_finish_sum3(double* partials, int nb) {
-    double a = 0.0, b = 0.0, c = 0.0;
-    for (int i = threadIdx.x; i < nb; i += blockDim.x) {
-        a += partials[i];
-        b += partials[kPartStride + i];
-        c += partials[2 * kPartStride + i];
-    }
-    a = block_sum(a);
-    b = block_sum(b);
-    c = block_sum(c);
-    if (threadIdx.x == 0) {
-        partials[kRedSlots - 1] = a;
-        partials[kRedSlots - 2] = b;
-        partials[kRedSlots - 3] = c;
-    }
-}
-
 int red_grid(int64_t n) { return grid_for(n, kThreads * 4, kRedBlocks); }
 
 }  // namespace
@@ -546,23 +490,17 @@ void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s) 
 
 int launch_hv_fast(hubbard_sector* H, const void* v, void* w, int dtype, double beta, const void* w_old,
                    int fixed_emax, cudaStream_t s, double* part, bool* fused, const RowUpdate* upd, LzDev* dv,
-                   double* ha, double* hb) {
+                   double* hist) {
     const DevSpin& up = H->dev[0];
     const DevSpin& dn = H->dev[1];
     const int grid = grid_for(H->Dup, 1, sm_count() * 16);
     if (fused != nullptr) *fused = false;
     if (H->fx_bytes >= (size_t)H->D * 16) {
         int np = 0;
-        int rc = launch_hv_phases(H, v, w, dtype, beta, w_old, H->fx_scratch, fixed_emax, s, part, &np, upd, dv);
+        const int rc = launch_hv_phases(H, v, w, dtype, beta, w_old, H->fx_scratch, fixed_emax, s, part, &np, upd, dv,
+                                        hist);
         if (rc != -1) {
             if (rc == HUB_OK && part != nullptr && np > 0) {
-                if (dv != nullptr) {
-                    if ((rc = launch_lz_finish(part, np, dv, ha, hb, s))) return rc;
-                } else {
-                    k_finish_sum3<<<1, 1024, 0, s>>>(part, np);
-                    HUB_CUDA(cudaGetLastError());
-                    count_launches(1);
-                }
                 if (fused != nullptr) *fused = true;
             } else if (rc == HUB_OK && dv != nullptr) {
                 return fail(HUB_EINVAL, "device-resident Lanczos step without fused reductions");
@@ -654,21 +592,14 @@ int launch_axpy_scale(double a, double inv, const void* x, void* y, int64_t n, i
     return HUB_OK;
 }
 
-int launch_lz_explicit(LzDev* dv, const void* x, void* y, int64_t n, int dtype, double* partials, double* hb,
+int launch_lz_explicit(LzDev* dv, const void* x, void* y, int64_t n, int dtype, double* partials, double* hist,
                        cudaStream_t s) {
     const int g = red_grid(n);
     if (dtype == HUB_F64) k_lz_axpy_nrm2_f64<<<g, kThreads, 0, s>>>(dv, (const double*)x, (double*)y, n, partials);
     else k_lz_axpy_nrm2_f32<<<g, kThreads, 0, s>>>(dv, (const float*)x, (float*)y, n, partials);
-    k_lz_finish2<<<1, 1024, 0, s>>>(partials, g, dv, hb);
+    k_lz_finish2<<<1, 1024, 0, s>>>(partials, g, dv, hist);
     HUB_CUDA(cudaGetLastError());
     count_launches(2);
-    return HUB_OK;
-}
-
-int launch_lz_finish(double* part, int np, LzDev* dv, double* ha, double* hb, cudaStream_t s) {
-    k_lz_finish<<<1, 1024, 0, s>>>(part, np, dv, ha, hb);
-    HUB_CUDA(cudaGetLastError());
-    count_launches(1);
     return HUB_OK;
 }
 
