@@ -133,6 +133,20 @@ __device__ __forceinline__ void add4(int2& A, int2 a, int2 b, int2 c, int2 d) {
     A.y += a.y + b.y + c.y + d.y;
 }
 __device__ __forceinline__ void add4(int2& A, int2 a) { A.x += a.x; A.y += a.y; }
+__device__ __forceinline__ void sub4(int4& A, int4 a, int4 b, int4 c, int4 d) {
+    A.x -= a.x + b.x + c.x + d.x;
+    A.y -= a.y + b.y + c.y + d.y;
+    A.z -= a.z + b.z + c.z + d.z;
+    A.w -= a.w + b.w + c.w + d.w;
+}
+__device__ __forceinline__ void sub4(int4& A, int4 a) {
+    A.x -= a.x; A.y -= a.y; A.z -= a.z; A.w -= a.w;
+}
+__device__ __forceinline__ void sub4(int2& A, int2 a, int2 b, int2 c, int2 d) {
+    A.x -= a.x + b.x + c.x + d.x;
+    A.y -= a.y + b.y + c.y + d.y;
+}
+__device__ __forceinline__ void sub4(int2& A, int2 a) { A.x -= a.x; A.y -= a.y; }
 
 
 // Lanczos reductions fused into the up-phase epilogue (Algorithm 1): each

@@ -62,6 +62,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
                                                      const double* __restrict__ fo, double ua, double uinv,
                                                      const LzDev* __restrict__ dv) {
     using S = typename FxVec<VEC>::T;
+    grid_dep_wait();
     if constexpr (UPD) {
         if (dv != nullptr) {                              // device-resident step: the update's scalars
             if (dv->stall) return;
@@ -189,54 +190,75 @@ __global__ void __launch_bounds__(512) k_rows_global_f64x(const int2* __restrict
 // items are (column chunk, block of RB rows); consecutive items share a chunk,
 // which keeps that chunk of X resident in L2 while all rows are combined, and
 // consecutive rows share part of their neighbours (reuse in L1).
-constexpr int kUpRows = 16;
+// An item of 16 rows is two per warp; where that leaves fewer items than CTAs
+// that fit on the device, 8 rows (one per warp) spread the sector wider.
+inline int up_rows(int64_t nchunk, int64_t Dup, int ctas) { return nchunk * ((Dup + 15) / 16) < ctas ? 8 : 16; }
 
 // Signed sum over the warp-uniform hop list of row u: targets t in
 // list[kb .. kb+n), the first np with sign +1.  load(t) returns this lane's
-// operand from row t; four independent loads are issued before they are
-// added.  Loop bounds are warp-uniform, so the sign split costs no divergence.
-template <typename Val, typename Load, typename Add>
+// operand from row t; the operands of a group of four of one sign are requested
+// together, then add(sign, a, b, c, d) or add(sign, a) takes them.  Loop bounds
+// are warp-uniform, so the sign split costs no divergence.
+// TAIL: what is left of a sign after the groups of four is one more group with
+// zeros in place of the missing operands, instead of a memory round each.
+template <typename Val, bool TAIL, typename Load, typename Add>
 __device__ __forceinline__ void uniform_hops(const uint32_t* __restrict__ list, int32_t kb, int n, int np, int lane,
-                                             Val& P, Val& N, Load&& load, Add&& add) {
+                                             Load&& load, Add&& add) {
     for (int k0 = 0; k0 < n; k0 += 32) {
         const int nk = min(32, n - k0);
         const uint32_t mine = lane < nk ? __ldg(list + kb + k0 + lane) : 0u;
         const int pend = max(0, min(nk, np - k0));
-        int q = 0;
-        for (; q + 4 <= pend; q += 4) {
-            const Val a = load(__shfl_sync(0xffffffffu, mine, q));
-            const Val b = load(__shfl_sync(0xffffffffu, mine, q + 1));
-            const Val c = load(__shfl_sync(0xffffffffu, mine, q + 2));
-            const Val d = load(__shfl_sync(0xffffffffu, mine, q + 3));
-            add(P, a, b, c, d);
-        }
-        for (; q < pend; ++q) add(P, load(__shfl_sync(0xffffffffu, mine, q)));
-        for (; q + 4 <= nk; q += 4) {
-            const Val a = load(__shfl_sync(0xffffffffu, mine, q));
-            const Val b = load(__shfl_sync(0xffffffffu, mine, q + 1));
-            const Val c = load(__shfl_sync(0xffffffffu, mine, q + 2));
-            const Val d = load(__shfl_sync(0xffffffffu, mine, q + 3));
-            add(N, a, b, c, d);
-        }
-        for (; q < nk; ++q) add(N, load(__shfl_sync(0xffffffffu, mine, q)));
+        auto span = [&](auto sign, int q, int end) {
+            for (; q + 4 <= end; q += 4) {
+                const Val a = load(__shfl_sync(0xffffffffu, mine, q));
+                const Val b = load(__shfl_sync(0xffffffffu, mine, q + 1));
+                const Val c = load(__shfl_sync(0xffffffffu, mine, q + 2));
+                const Val d = load(__shfl_sync(0xffffffffu, mine, q + 3));
+                add(sign, a, b, c, d);
+            }
+            if constexpr (TAIL) {
+                if (q < end) {
+                    const Val a = load(__shfl_sync(0xffffffffu, mine, q));
+                    Val b{}, c{};
+                    const uint32_t t1 = __shfl_sync(0xffffffffu, mine, q + 1), t2 = __shfl_sync(0xffffffffu, mine, q + 2);
+                    if (q + 1 < end) b = load(t1);
+                    if (q + 2 < end) c = load(t2);
+                    add(sign, a, b, c, Val{});
+                }
+            } else {
+                for (; q < end; ++q) add(sign, load(__shfl_sync(0xffffffffu, mine, q)));
+            }
+        };
+        span(std::integral_constant<int, 1>{}, 0, pend);
+        span(std::integral_constant<int, -1>{}, pend, nk);
     }
 }
+
+// the binary64 accumulation: exact integers, so one accumulator takes both signs
+template <typename IV> struct AddFixed {
+    IV& A;
+    template <typename Sign, typename... Vs>
+    __device__ __forceinline__ void operator()(Sign, Vs... xs) const {
+        if constexpr (Sign::value > 0) add4(A, xs...);
+        else sub4(A, xs...);
+    }
+};
 
 // Up phase, binary64 fixed point (Algorithms 2 and 4):
 //   W[u, c] = -t (sum_{(u', s) in hops_up(u)} s X[u', c] + Y[u, c]) + U n(u, c) X[u, c]  [- beta w_old]
 // Row u of W is a signed combination of whole rows u' of X (Eq. H-Kroneckersum),
 // so a warp builds one row segment of CC = 32 * VPL columns with lanes over
 // columns: the hop list is warp-uniform and every access is coalesced.  Work
-// items are (column chunk, block of kUpRows rows); consecutive items share a
+// items are (column chunk, block of rbr rows); consecutive items share a
 // chunk, which keeps that chunk of X resident in L2 while all rows are
 // combined, and consecutive rows share part of their neighbours (L1 reuse).
 // RED: also accumulate <W, fv>, <W, W> and <fv, fv> into part (block_sum3_store).
 // PRE: the epilogue's own element and Y are requested before the gathers (their
 // HBM latency then overlaps the hop sum); CT: CTAs per SM the launch bounds keep
-template <int VPL, bool FAST, bool PRE = false, int CT = 4>
+template <int VPL, bool FAST, bool TAIL, bool PRE = false, int CT = 4>
 __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
-                                                     const int32_t* __restrict__ ptr,
+                                                     int rbr, const int32_t* __restrict__ ptr,
                                                      const int32_t* __restrict__ npos,
                                                      const uint32_t* __restrict__ list,
                                                      const uint32_t* __restrict__ su,
@@ -246,12 +268,13 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
     __shared__ long long Bs[33];
     for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
     __syncthreads();
+    grid_dep_wait();
     const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
     const int k = 1070 - emax;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     constexpr int CC = 32 * VPL;
     const int64_t nchunk = (Ddn + CC - 1) / CC;
-    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
+    const int64_t nrb = (Dup + rbr - 1) / rbr;
     // item = chunk * nrb + rb, advanced by gridDim.x without division
     int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
     const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
@@ -268,8 +291,8 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
 #pragma unroll
         for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
         const IV* base = reinterpret_cast<const IV*>(X + c);
-        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
-        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
+        const int64_t uend = min(rb * rbr + rbr, Dup);
+        for (int64_t u = rb * rbr + warp; u < uend; u += nw) {
             const int32_t kb = ptr[u];
             [[maybe_unused]] int4 t4p;
             [[maybe_unused]] longlong2 y2p;
@@ -278,10 +301,10 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                 t4p = __ldg(reinterpret_cast<const int4*>(X + J));
                 y2p = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
             }
-            IV P{}, N{};
-            uniform_hops<IV>(list, kb, ptr[u + 1] - kb, npos[u], lane, P, N,
+            IV A{};
+            uniform_hops<IV, TAIL>(list, kb, ptr[u + 1] - kb, npos[u], lane,
                 [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(reinterpret_cast<const int2*>(base) + (int64_t)t * Ddn)); },
-                [](IV& A, auto... xs) { add4(A, xs...); });
+                AddFixed<IV>{A});
             if (act) {
                 const uint32_t su_u = su[u];
                 const int64_t J = u * Ddn + c;
@@ -289,7 +312,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                 int2 xo[VPL];
                 long long yv[VPL];
                 if constexpr (VPL == 2) {
-                    lo[0] = P.x - N.x; hi[0] = P.y - N.y; lo[1] = P.z - N.z; hi[1] = P.w - N.w;
+                    lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
                     int4 t4;
                     longlong2 y2;
                     if constexpr (PRE) {
@@ -304,7 +327,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                     yv[0] = y2.x;
                     yv[1] = y2.y;
                 } else {
-                    lo[0] = P.x - N.x; hi[0] = P.y - N.y;
+                    lo[0] = A.x; hi[0] = A.y;
                     xo[0] = __ldg(X + J);
                     yv[0] = __ldcs(Y + J);
                 }
@@ -345,7 +368,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
 template <int VPL, bool FAST>
 __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
-                                                     const int32_t* __restrict__ ptr,
+                                                     int rbr, const int32_t* __restrict__ ptr,
                                                      const int32_t* __restrict__ npos,
                                                      const uint32_t* __restrict__ list,
                                                      const uint32_t* __restrict__ su,
@@ -353,6 +376,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                                                      const int* __restrict__ emax_p, int fixed_emax,
                                                      const double* __restrict__ fv, double* part,
                                                      unsigned* done, LzDev* dv, double* hist) {
+    grid_dep_wait();
     if (dv != nullptr && dv->stall) return;
     double s1 = 0.0, s2 = 0.0, s3 = 0.0;
     using IV = typename FxVec<VPL>::T;
@@ -369,7 +393,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     constexpr int CC = 32 * VPL;
     const int64_t nchunk = (Ddn + CC - 1) / CC;
-    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
+    const int64_t nrb = (Dup + rbr - 1) / rbr;
     // item = chunk * nrb + rb, advanced by gridDim.x without division
     int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
     const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
@@ -386,8 +410,8 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
 #pragma unroll
         for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
         const IV* base = reinterpret_cast<const IV*>(X + c);
-        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
-        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
+        const int64_t uend = min(rb * rbr + rbr, Dup);
+        for (int64_t u = rb * rbr + warp; u < uend; u += nw) {
             const int32_t kb = ptr[u];
             const int64_t J = u * Ddn + c;
             // streamed operands of the epilogue, requested before the gathers
@@ -406,17 +430,17 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                     fpre[0] = q.x; fpre[1] = q.y;
                 }
             }
-            IV P{}, N{};
-            uniform_hops<IV>(list, kb, ptr[u + 1] - kb, npos[u], lane, P, N,
+            IV A{};
+            uniform_hops<IV, true>(list, kb, ptr[u + 1] - kb, npos[u], lane,
                 [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(reinterpret_cast<const int2*>(base) + (int64_t)t * Ddn)); },
-                [](IV& A, auto... xs) { add4(A, xs...); });
+                AddFixed<IV>{A});
             if (act) {
                 const uint32_t su_u = su[u];
                 int lo[VPL], hi[VPL];
                 int2 xo[VPL];
                 long long yv[VPL];
                 if constexpr (VPL == 2) {
-                    lo[0] = P.x - N.x; hi[0] = P.y - N.y; lo[1] = P.z - N.z; hi[1] = P.w - N.w;
+                    lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
                     const int4 t4 = t4p;
                     xo[0] = make_int2(t4.x, t4.y);
                     xo[1] = make_int2(t4.z, t4.w);
@@ -424,7 +448,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                     yv[0] = y2.x;
                     yv[1] = y2.y;
                 } else {
-                    lo[0] = P.x - N.x; hi[0] = P.y - N.y;
+                    lo[0] = A.x; hi[0] = A.y;
                     xo[0] = __ldg(X + J);
                     yv[0] = __ldcs(Y + J);
                 }
@@ -489,83 +513,346 @@ __device__ __forceinline__ void addf(float4& A, float4 a, float4 b, float4 c, fl
 }
 __device__ __forceinline__ void addf(float4& A, float4 a) { A.x += a.x; A.y += a.y; A.z += a.z; A.w += a.w; }
 
-// Up phase, binary32: same decomposition, float arithmetic
-// CTAs per SM of the binary32 up phase: 5 at <= 51 registers, 4 where 4
-// columns per lane or the Lanczos variant's prefetched operands need more
-template <int VPL, bool RED = false>
-constexpr int up32_ctas() { return (RED || VPL == 4) ? 4 : 5; }
+// Up phase with resident rows: a warp builds one row segment of 32 * VPL * NV
+// columns with lanes over columns, as above, but the rows belong to the CTA.
+//
+// CTA (i, j) of the grid owns row range i and the column chunks j, j + gy, ...;
+// its rows' hop lists are staged in shared memory once and serve every chunk
+// (a range whose lists do not fit goes in blocks, staged again for each chunk).
+// All CTAs sweep the chunks in the same order, so the chunk of X that the rows
+// of every CTA gather from stays in L2.  A segment is then one dependent step:
+// its gathers and its epilogue operands (own element, Y, w_old, f) are all
+// requested at once.  Read per segment, the row pointer, the list and the
+// epilogue operands each added an L2 or HBM latency to the chain, and with
+// registers for 24-32 warps per SM the phase ran at that chain's pace.
+struct UpGrid {
+    int gx, gy;                      // row ranges, interleaved column chunks
+    int cap;                         // rows whose lists fit in shared memory at a time
+    int W;                           // longest hop list
+    size_t smem;
+};
 
-template <int VPL, bool RED>
-__global__ void __launch_bounds__(256, up32_ctas<VPL, RED>()) k_up_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
-                                                    const float* w_old, int64_t Dup, int64_t Ddn,
-                                                    const int32_t* __restrict__ ptr,
-                                                    const int32_t* __restrict__ npos,
-                                                    const uint32_t* __restrict__ list,
-                                                    const uint32_t* __restrict__ su,
-                                                    const uint32_t* __restrict__ sd, float mt, float U, float mbeta,
-                                                    double* part, unsigned* done, LzDev* dv, double* hist) {
+struct UpLists {
+    const uint32_t* list;            // [cap][W] target rows, sign +1 first
+    const int2* cnt;                 // [cap] (+1 targets, targets)
+    const uint32_t* st;              // [cap] basis words
+};
+
+__device__ __forceinline__ void stage_up_lists(unsigned char* smem, int cap, int W, int64_t r0, int nr,
+                                               const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
+                                               const uint32_t* __restrict__ list, const uint32_t* __restrict__ su) {
+    int2* cnt = reinterpret_cast<int2*>(smem);
+    uint32_t* st = reinterpret_cast<uint32_t*>(cnt + cap);
+    uint32_t* L = st + cap;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    for (int r = warp; r < nr; r += nw) {
+        const int32_t kb = ptr[r0 + r];
+        const int n = ptr[r0 + r + 1] - kb;
+        for (int k = lane; k < n; k += 32) L[r * W + k] = list[kb + k];
+        if (lane == 0) {
+            cnt[r] = make_int2(npos[r0 + r], n);
+            st[r] = su[r0 + r];
+        }
+    }
+}
+
+// Sums over a staged hop list, +1 targets then -1 targets: add(neg, entries, k)
+// sees groups of four, the last of each sign with k < 4 valid ones, so that the
+// loads of a group are always requested together (a rest taken one by one is a
+// memory latency for each of its entries).
+template <typename Add>
+__device__ __forceinline__ void list_hops(const uint32_t* L, int np, int n, Add&& add) {
+    int q = 0;
+    for (; q + 4 <= np; q += 4) add(false, L + q, std::integral_constant<int, 4>{}, 4);
+    if (q < np) add(false, L + q, std::integral_constant<int, 0>{}, np - q);
+    for (q = np; q + 4 <= n; q += 4) add(true, L + q, std::integral_constant<int, 4>{}, 4);
+    if (q < n) add(true, L + q, std::integral_constant<int, 0>{}, n - q);
+}
+
+// Cost of a row's segment in units of one hop, besides its hops.
+constexpr int kUpRowCost = 8;
+
+// First row of range i of gx: ranges of equal cost, sum of (hops + kUpRowCost).
+// The hop counts of neighbouring rows are alike (they share their upper sites),
+// so ranges of equally many rows differed enough to leave the SMs idle for a
+// third of the phase.  One warp, 32 probes a round.
+__device__ __forceinline__ int64_t up_range_start(const int32_t* __restrict__ ptr, int64_t Dup, int i, int gx) {
+    const int lane = threadIdx.x & 31;
+    const int64_t total = (int64_t)__ldg(ptr + Dup) + kUpRowCost * Dup;
+    const int64_t want = (total * i + gx - 1) / gx;
+    int64_t lo = 0, hi = Dup;                             // the answer is in [lo, hi]
+    while (hi > lo) {
+        const int64_t step = (hi - lo + 31) / 32;
+        const int64_t r = min(lo + step * lane, hi);
+        const bool below = (int64_t)__ldg(ptr + r) + kUpRowCost * r < want;
+        const int nb = __popc(__ballot_sync(0xffffffffu, below));   // probes below: a prefix of the lanes
+        if (nb == 0) return lo;
+        const int64_t last = min(lo + step * (nb - 1), hi);         // below
+        const int64_t next = nb == 32 ? hi : min(lo + step * nb, hi);
+        lo = min(last + 1, hi);
+        hi = max(next, lo);
+    }
+    return lo;
+}
+
+// the segments of one CTA, seg(row in the staged block, chunk) for every one
+template <typename Seg>
+__device__ __forceinline__ void up_segments(unsigned char* smem, int64_t Dup, int64_t nchunk, const UpGrid& g,
+                                            const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
+                                            const uint32_t* __restrict__ list, const uint32_t* __restrict__ su,
+                                            Seg&& seg) {
+    const int i = blockIdx.x % g.gx, j = blockIdx.x / g.gx;
+    const int warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    __shared__ int64_t range[2];
+    if (warp < 2) {
+        const int64_t r = up_range_start(ptr, Dup, i + warp, g.gx);
+        if ((threadIdx.x & 31) == 0) range[warp] = r;
+    }
+    __syncthreads();
+    const int64_t r0 = range[0];
+    const int nr = (int)(range[1] - r0);
+    if (nr == 0) return;
+    if (nr <= g.cap) {
+        stage_up_lists(smem, g.cap, g.W, r0, nr, ptr, npos, list, su);
+        __syncthreads();
+        // segments in (chunk, row) order, dealt to the warps in turn
+        int64_t chunk = j;
+        int r = warp;
+        while (r >= nr && chunk < nchunk) { r -= nr; chunk += g.gy; }
+        while (chunk < nchunk) {
+            seg(r0, r, chunk);
+            r += nw;
+            while (r >= nr && chunk < nchunk) { r -= nr; chunk += g.gy; }
+        }
+        return;
+    }
+    for (int64_t chunk = j; chunk < nchunk; chunk += g.gy)
+        for (int b = 0; b < nr; b += g.cap) {
+            const int nb = min(g.cap, nr - b);
+            __syncthreads();
+            stage_up_lists(smem, g.cap, g.W, r0 + b, nb, ptr, npos, list, su);
+            __syncthreads();
+            for (int r = warp; r < nb; r += nw) seg(r0 + b, r, chunk);
+        }
+}
+
+// Binary64 fixed point, resident rows.  STEP: the Lanczos step, W = H f - beta w_old with, per
+// CTA, the partials of <W, f>, <W, W> and <f, f> (block_sum3_store).  CT: CTAs
+// per SM the launch bounds keep.
+template <int VPL, bool FAST, bool STEP, int CT>
+__global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
+                                                     double* w, const double* w_old, int64_t Dup, int64_t Ddn,
+                                                     UpGrid g, const int32_t* __restrict__ ptr,
+                                                     const int32_t* __restrict__ npos,
+                                                     const uint32_t* __restrict__ list,
+                                                     const uint32_t* __restrict__ su,
+                                                     const uint32_t* __restrict__ sd,
+                                                     const __grid_constant__ EpiParams ep,
+                                                     const int* __restrict__ emax_p, int fixed_emax,
+                                                     const double* __restrict__ fv, double* part,
+                                                     unsigned* done, LzDev* dv, double* hist) {
+    grid_dep_wait();
+    if (STEP && dv != nullptr && dv->stall) return;
+    using IV = typename FxVec<VPL>::T;
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    __shared__ long long Bs[33];
+    if constexpr (!FAST)
+        for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
+    double mbeta = ep.mbeta;
+    long long Bbeta = ep.Bbeta;
+    if (STEP && dv != nullptr) {                          // device-resident step: beta_j on the device
+        mbeta = -dv->beta;
+        Bbeta = llround(ldexp(mbeta, ep.m));
+    }
+    const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
+    const int k = 1070 - emax;
+    const int lane = threadIdx.x & 31;
+    constexpr int CC = 32 * VPL;
+    const int2* cnt = reinterpret_cast<const int2*>(smem_raw);
+    const uint32_t* st = reinterpret_cast<const uint32_t*>(cnt + g.cap);
+    const uint32_t* L = st + g.cap;
+    const uint32_t rowb = (uint32_t)Ddn * 8u;             // bytes of a row (Ddn <= 2^28, checked by the launcher)
+    double s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    up_segments(smem_raw, Dup, (Ddn + CC - 1) / CC, g, ptr, npos, list, su, [&](int64_t r0, int r, int64_t chunk) {
+        const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
+        const bool act = c_raw < Ddn;
+        const int64_t c = act ? c_raw : Ddn - VPL;     // tail lanes read a valid column, store nothing
+        const int64_t J = (r0 + r) * Ddn + c;
+        const char* base = reinterpret_cast<const char*>(X + c);
+        auto load = [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); };
+        // epilogue operands, requested with the gathers
+        const IV xo4 = __ldg(reinterpret_cast<const IV*>(X + J));
+        long long yv[VPL];
+        double wv[VPL], fj[VPL];
+        uint32_t sdc[VPL];
+        if constexpr (VPL == 2) {
+            const longlong2 y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+            yv[0] = y2.x;
+            yv[1] = y2.y;
+            if (STEP) {
+                if (w_old != nullptr) {
+                    const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
+                    wv[0] = q.x;
+                    wv[1] = q.y;
+                }
+                if (part != nullptr) {
+                    const double2 q = __ldcs(reinterpret_cast<const double2*>(fv + J));
+                    fj[0] = q.x;
+                    fj[1] = q.y;
+                }
+            }
+        } else {
+            yv[0] = __ldcs(Y + J);
+            if (STEP && w_old != nullptr) wv[0] = __ldcs(w_old + J);
+            if (STEP && part != nullptr) fj[0] = __ldcs(fv + J);
+        }
+        IV A{};
+        const int2 np = cnt[r];
+        list_hops(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
+            IV x[4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q) {
+                x[q] = IV{};
+                if (full.value == 4 || q < m) x[q] = load(t[q]);
+            }
+            if (neg) sub4(A, x[0], x[1], x[2], x[3]);
+            else add4(A, x[0], x[1], x[2], x[3]);
+        });
+        if (!act) return;
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) sdc[j] = __ldg(sd + c + j);
+        const uint32_t su_u = st[r];
+        double res[VPL];
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            long long T, xo;
+            if constexpr (VPL == 2) {
+                T = j == 0 ? fx_join(A.x, A.y) : fx_join(A.z, A.w);
+                xo = j == 0 ? fx_join(xo4.x, xo4.y) : fx_join(xo4.z, xo4.w);
+            } else {
+                T = fx_join(A.x, A.y);
+                xo = fx_join(xo4.x, xo4.y);
+            }
+            T += yv[j];
+            const int nd = __popc(su_u & sdc[j]);
+            if constexpr (FAST) {
+                // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
+                long long Pv = T << ep.tshift;
+                if (ep.tneg == 0) Pv = -Pv;
+                Pv += ep.Uint * (long long)nd * xo;
+                res[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
+                if (STEP && w_old != nullptr) res[j] = fma(mbeta, wv[j], res[j]);
+            } else {
+                I128 acc{0ull, 0ll};
+                mac128(acc, T, ep.A);
+                mac128(acc, xo, Bs[nd]);
+                if (STEP && w_old != nullptr) {
+                    int glo, ghi;
+                    fx_split(wv[j], emax, glo, ghi);
+                    mac128(acc, fx_join(glo, ghi), Bbeta);
+                }
+                res[j] = i128_to_double(acc, -(k + ep.m));
+            }
+        }
+        if constexpr (VPL == 2) __stcs(reinterpret_cast<double2*>(w + J), make_double2(res[0], res[1]));
+        else __stcs(w + J, res[0]);
+        if (STEP && part != nullptr) {
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                s1 = fma(res[j], fj[j], s1);
+                s2 = fma(res[j], res[j], s2);
+                s3 = fma(fj[j], fj[j], s3);
+            }
+        }
+    });
+    if (STEP && part != nullptr) {
+        block_sum3_store(s1, s2, s3, part);
+        close_sums3(part, gridDim.x, done, dv, hist);
+    }
+}
+
+// Binary32: same decomposition, float arithmetic.  NV vectors of VPL columns
+// per lane, 32 * VPL columns apart, so rows whose length only allows narrow
+// vectors still keep as many bytes in flight.
+template <int VPL, int NV, bool RED>
+__global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
+                                                   const float* w_old, int64_t Dup, int64_t Ddn, UpGrid g,
+                                                   const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
+                                                   const uint32_t* __restrict__ list, const uint32_t* __restrict__ su,
+                                                   const uint32_t* __restrict__ sd, float mt, float U, float mbeta,
+                                                   double* part, unsigned* done, LzDev* dv, double* hist) {
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    grid_dep_wait();
     if (dv != nullptr && dv->stall) return;
     FFAcc s1, s2, s3;
     if (dv != nullptr) mbeta = (float)-dv->beta;          // device-resident step: beta_j on the device
     using V = typename F32Vec<VPL>::T;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    constexpr int CC = 32 * VPL;
-    const int64_t nchunk = (Ddn + CC - 1) / CC;
-    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
-    int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
-    const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
-    for (; chunk < nchunk; chunk += dch, rb += drb) {
-        if (rb >= nrb) {
-            rb -= nrb;
-            ++chunk;
-            if (chunk >= nchunk) break;
-        }
-        const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
-        const bool act = c_raw < Ddn;
-        const int64_t c = act ? c_raw : Ddn - VPL;
-        uint32_t sdc[VPL];
+    const int lane = threadIdx.x & 31;
+    constexpr int CC = 32 * VPL * NV;
+    const int2* cnt = reinterpret_cast<const int2*>(smem_raw);
+    const uint32_t* st = reinterpret_cast<const uint32_t*>(cnt + g.cap);
+    const uint32_t* L = st + g.cap;
+    const uint32_t rowb = (uint32_t)Ddn * 4u;
+    up_segments(smem_raw, Dup, (Ddn + CC - 1) / CC, g, ptr, npos, list, su, [&](int64_t r0, int r, int64_t chunk) {
+        int64_t c[NV];
+        bool act[NV];
+        V xo[NV], yv[NV], wv[NV], P[NV], N[NV];
 #pragma unroll
-        for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
-        const float* base = v + c;
-        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
-        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
-            const int32_t kb = ptr[u];
-            const int64_t J = u * Ddn + c;
-            V xpre{}, ypre{}, wpre{};
-            if constexpr (RED) {                      // Lanczos step: epilogue operands before the gathers
-                xpre = __ldg(reinterpret_cast<const V*>(v + J));
-                ypre = __ldcs(reinterpret_cast<const V*>(Y + J));
-                if (w_old != nullptr) wpre = __ldcs(reinterpret_cast<const V*>(w_old + J));
+        for (int i = 0; i < NV; ++i) {
+            const int64_t c_raw = chunk * CC + (int64_t)(i * 32 + lane) * VPL;
+            act[i] = c_raw < Ddn;
+            c[i] = act[i] ? c_raw : Ddn - VPL;
+            const int64_t J = (r0 + r) * Ddn + c[i];
+            xo[i] = __ldg(reinterpret_cast<const V*>(v + J));
+            yv[i] = __ldcs(reinterpret_cast<const V*>(Y + J));
+            if (w_old != nullptr) wv[i] = __ldcs(reinterpret_cast<const V*>(w_old + J));
+            P[i] = V{};
+            N[i] = V{};
+        }
+        auto load = [&](uint32_t t, int i) {
+            return __ldg(reinterpret_cast<const V*>(reinterpret_cast<const char*>(v + c[i]) + (uint64_t)t * rowb));
+        };
+        const int2 np = cnt[r];
+        list_hops(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
+            V x[NV][4];
+#pragma unroll
+            for (int q = 0; q < 4; ++q)
+#pragma unroll
+                for (int i = 0; i < NV; ++i) {
+                    x[i][q] = V{};
+                    if (full.value == 4 || q < m) x[i][q] = load(t[q], i);
+                }
+#pragma unroll
+            for (int i = 0; i < NV; ++i) {
+                if (neg) addf(N[i], x[i][0], x[i][1], x[i][2], x[i][3]);
+                else addf(P[i], x[i][0], x[i][1], x[i][2], x[i][3]);
             }
-            V P{}, N{};
-            uniform_hops<V>(list, kb, ptr[u + 1] - kb, npos[u], lane, P, N,
-                [&](uint32_t t) { return __ldg(reinterpret_cast<const V*>(base + (int64_t)t * Ddn)); },
-                [](V& A, auto... xs) { addf(A, xs...); });
-            if (act) {
-                const uint32_t su_u = su[u];
-                const V xo = RED ? xpre : __ldg(reinterpret_cast<const V*>(v + J));
-                const V yv = RED ? ypre : __ldcs(reinterpret_cast<const V*>(Y + J));
-                float r[VPL];
+        });
+        const uint32_t su_u = st[r];
+#pragma unroll
+        for (int i = 0; i < NV; ++i) {
+            if (!act[i]) continue;
+            const int64_t J = (r0 + r) * Ddn + c[i];
+            float res[VPL];
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                const float nd = (float)__popc(su_u & __ldg(sd + c[i] + j));
+                res[j] = fmaf(mt, (comp(P[i], j) - comp(N[i], j)) + comp(yv[i], j), U * nd * comp(xo[i], j));
+                if (w_old != nullptr) res[j] = fmaf(mbeta, comp(wv[i], j), res[j]);
+            }
+            if constexpr (VPL == 4) __stcs(reinterpret_cast<float4*>(w + J), make_float4(res[0], res[1], res[2], res[3]));
+            else if constexpr (VPL == 2) __stcs(reinterpret_cast<float2*>(w + J), make_float2(res[0], res[1]));
+            else __stcs(w + J, res[0]);
+            if constexpr (RED) {
 #pragma unroll
                 for (int j = 0; j < VPL; ++j) {
-                    const float nd = (float)__popc(su_u & sdc[j]);
-                    r[j] = fmaf(mt, (comp(P, j) - comp(N, j)) + comp(yv, j), U * nd * comp(xo, j));
-                    if (w_old != nullptr) r[j] = fmaf(mbeta, RED ? comp(wpre, j) : w_old[J + j], r[j]);
-                }
-                if constexpr (VPL == 4) __stcs(reinterpret_cast<float4*>(w + J), make_float4(r[0], r[1], r[2], r[3]));
-                else if constexpr (VPL == 2) __stcs(reinterpret_cast<float2*>(w + J), make_float2(r[0], r[1]));
-                else __stcs(w + J, r[0]);
-                if constexpr (RED) {
-#pragma unroll
-                    for (int j = 0; j < VPL; ++j) {
-                        s1.add_product(r[j], comp(xo, j));
-                        s2.add_product(r[j], r[j]);
-                        s3.add_product(comp(xo, j), comp(xo, j));
-                    }
+                    s1.add_product(res[j], comp(xo[i], j));
+                    s2.add_product(res[j], res[j]);
+                    s3.add_product(comp(xo[i], j), comp(xo[i], j));
                 }
             }
         }
-    }
+    });
     if constexpr (RED) {
         block_sum3_store(s1.value(), s2.value(), s3.value(), part);
         close_sums3(part, gridDim.x, done, dv, hist);
@@ -584,6 +871,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f32(std::conditional_t<UPD, fl
                                                     const float* __restrict__ fo, float ua, float uinv,
                                                     const LzDev* __restrict__ dv) {
     using S = typename F32Vec<VEC>::T;
+    grid_dep_wait();
     if constexpr (UPD) {
         if (dv != nullptr) {
             if (dv->stall) return;
@@ -725,6 +1013,24 @@ void allow_smem() {
     (void)once;
 }
 
+// Which binary64 up phase takes a sector with rows of even length (odd ones
+// always take the resident-row kernel):
+//   up to kUpSmall elements: work items dealt over all CTAs -- a CTA has one or
+//     two, and staging lists would only lengthen its chain (ring 12 (6,6) step
+//     52.8 us, 57.2 with resident rows; ring 14 (7,7) 322 against 320);
+//   above: resident rows (4x4 (5,5) product 414 -> 376 us, step 600 -> 524 us;
+//     4x4 (8,8) step 5.35 -> 5.24 ms), except
+//   standalone products of more than kUpHbm bytes a vector (4x4 (8,8) 3.80 ms
+//     with items, 4.11 with resident rows; 4x4 (7,7) 2.87, 2.95; ring 16 (6,6),
+//     513 MB: 1.10, 1.05).
+constexpr int64_t kUpSmall = 2500000, kUpHbm = 600ll << 20;
+// Kernels of a sector start while the one before drains (launch_on) when its
+// vectors stay in L2 (ring 12 product 29.9 -> 26.1 us, step 55.9 -> 44.3 us); on
+// HBM-sized ones CTAs that take their places early disturb the sweep (4x4 (8,8)
+// product 3.80 -> 4.10 ms).
+constexpr int64_t kPdlBytes = 100ll << 20;
+constexpr int64_t kMaxRow = (1ll << 29) - 1;       // row pitch in bytes held in 32 bits
+
 // a grid of at most `full` CTAs and no more than the work items
 int grid_cap(int full, int64_t items) { return (int)std::max<int64_t>(1, std::min<int64_t>(full, items)); }
 
@@ -735,11 +1041,32 @@ int choose_vec(int req, int64_t len, int elem_bytes, int vmax, int reserve) {
     return req;
 }
 
+// Row ranges and column groups of the up phase: ranges of about 32 rows, the
+// chunks dealt to as many CTAs of each range as the device holds.  Longer ranges
+// let a list serve more segments, but the CTAs then differ more in how their
+// memory rounds add up (4x4 (5,5) binary64: 403, 385, 376, 392, 414 us with 7,
+// 14, 29, 57, 115 rows; 4x4 (8,8) binary32: 1.95, 1.91, 1.97, 2.01 ms with 21,
+// 42, 85, 169).
+UpGrid up_grid_for(const hubbard_sector* H, int64_t nchunk, int ctas) {
+    UpGrid g;
+    g.W = std::max(H->host[0].W, 1);
+    g.gy = (int)std::max<int64_t>(1, std::min<int64_t>(nchunk, (32 * (int64_t)ctas + H->Dup - 1) / H->Dup));
+    g.gx = (int)std::max<int64_t>(1, std::min<int64_t>(ctas / g.gy, (H->Dup + 7) / 8));
+    // most rows of a range: all of them without hops
+    const int64_t total = (int64_t)H->host[0].tgt.size() + kUpRowCost * H->Dup;
+    const int64_t rows = std::min<int64_t>(H->Dup, total / g.gx / kUpRowCost + 2);
+    const int64_t per_row = 12 + 4 * (int64_t)g.W;
+    g.cap = (int)std::max<int64_t>(1, std::min<int64_t>(rows, 24 * 1024 / per_row));
+    g.smem = (size_t)(g.cap * per_row);
+    return g;
+}
+
 }  // namespace
 
 // Returns HUB_OK and launches, or returns -1 when the staging buffers do not fit
 // (the caller then uses the single-pass gather kernel).
 bool hv_phases_fuse(const hubbard_sector* H, int dtype) {
+    if (H->Ddn > kMaxRow) return false;
     if (sms() * 5 > kPartStride) return false;
     return dtype == HUB_F64 || choose_vec(H->vec_rows, H->Ddn, 4, 4, 0) != 0;
 }
@@ -748,12 +1075,14 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
                      void* ybuf, int fixed_emax, cudaStream_t s, double* part, int* nparts,
                      const RowUpdate* upd, LzDev* dv, double* hist) {
     if (nparts != nullptr) *nparts = 0;
+    if (H->Ddn > kMaxRow) return -1;
     if (sms() * 5 > kPartStride) part = nullptr;        // partial arrays too short: no fused reduction
     const DevSpin& up = H->dev[0];
     const DevSpin& dn = H->dev[1];
     const int64_t Dup = H->Dup, Ddn = H->Ddn;
     const bool dn16 = dn.ent16 != nullptr;
     unsigned* done = reinterpret_cast<unsigned*>(H->status + 3);
+    const bool pdl = H->D * (dtype == HUB_F64 ? 8 : 4) <= kPdlBytes;
     // up-phase CTAs: as many as the launch bounds keep resident (the phase is
     // bound by L2 latency, so occupancy is what counts: 4 per SM at <= 64
     // registers for binary64 (3 for the Lanczos variant, whose prefetched
@@ -800,7 +1129,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         } else {
 #define ROWS64_U(V, E, P, U)                                                                                \
     allow_smem<k_rows_f64x<V, E, U>>();                                                                      \
-    k_rows_f64x<V, E, U><<<LA.blocks, LA.threads, LA.smem, s>>>((double*)const_cast<void*>(v), Y, Xg, Dup,   \
+    launch_on(pdl, k_rows_f64x<V, E, U>, LA.blocks, LA.threads, LA.smem, s, (double*)const_cast<void*>(v), Y, Xg, Dup,   \
         Ddn, dn.blk_off, dn.blk_cnt, P, emax, fixed_emax, upd ? (const double*)upd->fo : nullptr,            \
         upd ? upd->a : 0.0, upd ? upd->inv : 1.0, upd ? upd->dv : nullptr)
 #define ROWS64(V, E, P) if (upd) { ROWS64_U(V, E, P, true); } else { ROWS64_U(V, E, P, false); }
@@ -816,32 +1145,57 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         const EpiParams ep = make_epilogue(H->t, H->U, H->ns, w_old ? beta : 0.0, H->host[0].W + H->host[1].W);
         // columns per lane in the up phase: 2 when Ddn is even (16-byte loads)
         const int vpl = ((Ddn & 1) == 0 && H->vec_cols != 1) ? 2 : 1;
-        const int64_t up_items = ((Ddn + 32 * vpl - 1) / (32 * vpl)) * ((Dup + kUpRows - 1) / kUpRows);
-        const int up_grid = grid_cap(sms() * (part != nullptr ? 3 : 4), up_items);
-        // standalone up phase: request the epilogue's own element and Y before
-        // the gathers (at 3 CTAs/SM for the registers) where that measured
-        // faster -- the 128-bit epilogue and rows staged from global memory --
-        // unless the schedule fixes it (ctas_cols 1: no, 2: yes)
-        const bool pre = H->ctas_cols == 2 || (H->ctas_cols == 0 && (!ep.fast || va == 0));
-#define UP64(K, V, F)                                                                                       \
-    K<V, F><<<up_grid, 256, 0, s>>>(Xg, Y, (double*)w, (const double*)w_old, Dup, Ddn, up.pn_ptr,             \
-        up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax
-#define UP64P(V, F, CT)                                                                                     \
-    k_up_f64x<V, F, true, CT><<<grid_cap(sms() * CT, up_items), 256, 0, s>>>(Xg, Y, (double*)w,               \
-        (const double*)w_old, Dup, Ddn,                                                                    \
-        up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax)
-#define UP64_R(V, F)                                                                                        \
-    if (part != nullptr) { UP64(k_up_step_f64x, V, F), (const double*)v, part, done, dv, hist); }                      \
-    else if (V == 2 && pre) { UP64P(V, F, 3); }                                                            \
-    else { UP64(k_up_f64x, V, F)); }
-        if (vpl == 2) {
-            if (ep.fast) { UP64_R(2, true) } else { UP64_R(2, false) }
+        const bool step = part != nullptr || w_old != nullptr;
+        int up_grid = 0;
+        if (vpl == 1 || (H->D > kUpSmall && (step || H->D * 8 <= kUpHbm))) {
+            const bool three = step || H->ctas_cols == 2;
+            const UpGrid g = up_grid_for(H, (Ddn + 32 * vpl - 1) / (32 * vpl), sms() * (three ? 3 : 4));
+            up_grid = g.gx * g.gy;
+#define UPR64(V, F, ST, CT)                                                                                 \
+    launch_on(pdl, k_upr_f64x<V, F, ST, CT>, up_grid, 256, g.smem, s, Xg, Y, (double*)w, (const double*)w_old, Dup, \
+        Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax, (const double*)v, \
+        part, done, dv, hist)
+#define UPR64_S(V, F) if (step) { UPR64(V, F, true, 3); } else if (three) { UPR64(V, F, false, 3); } else { UPR64(V, F, false, 4); }
+            if (vpl == 2) {
+                if (ep.fast) { UPR64_S(2, true) } else { UPR64_S(2, false) }
+            } else {
+                if (ep.fast) { UPR64_S(1, true) } else { UPR64_S(1, false) }
+            }
+#undef UPR64_S
+#undef UPR64
         } else {
-            if (ep.fast) { UP64_R(1, true) } else { UP64_R(1, false) }
-        }
-#undef UP64_R
+            const int64_t up_chunks = (Ddn + 63) / 64;
+            const int up_full = sms() * (part != nullptr ? 3 : 4);
+            const int rbr = up_rows(up_chunks, Dup, up_full);
+            const int64_t up_items = up_chunks * ((Dup + rbr - 1) / rbr);
+            up_grid = grid_cap(up_full, up_items);
+            // standalone: request the epilogue's own element and Y before the
+            // gathers (at 3 CTAs/SM for the registers) where that measured faster --
+            // the 128-bit epilogue and rows staged from global memory -- unless the
+            // schedule fixes it (ctas_cols 1: no, 2: yes)
+            const bool pre = H->ctas_cols == 2 || (H->ctas_cols == 0 && (!ep.fast || va == 0));
+            const bool tail = H->D <= kUpSmall;
+#define UP64(K)                                                                                             \
+    launch_on(pdl, K, up_grid, 256, 0, s, Xg, Y, (double*)w, (const double*)w_old, Dup, Ddn, rbr,  \
+        up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax
+#define UP64P(F, T)                                                                                         \
+    launch_on(pdl, k_up_f64x<2, F, T, true, 3>, grid_cap(sms() * 3, up_items), 256, 0, s, Xg, Y, (double*)w, \
+        (const double*)w_old, Dup, Ddn, rbr, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep,  \
+        emax, fixed_emax)
+#define UP64_T(F, T)                                                                                        \
+    if (pre) { UP64P(F, T); } else { UP64((k_up_f64x<2, F, T>))); }
+            if (part != nullptr) {                        // a Lanczos step; a replayed one (w_old alone) goes below
+                if (ep.fast) { UP64((k_up_step_f64x<2, true>)), (const double*)v, part, done, dv, hist); }
+                else { UP64((k_up_step_f64x<2, false>)), (const double*)v, part, done, dv, hist); }
+            } else if (tail) {
+                if (ep.fast) { UP64_T(true, true) } else { UP64_T(false, true) }
+            } else {
+                if (ep.fast) { UP64_T(true, false) } else { UP64_T(false, false) }
+            }
+#undef UP64_T
 #undef UP64P
 #undef UP64
+        }
         if (part != nullptr && nparts != nullptr) *nparts = up_grid;
         HUB_CUDA(cudaGetLastError());
         count_launches(1 + extra + (fixed_emax <= 0 ? (w_old ? 2 : 1) : 0));
@@ -858,7 +1212,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     if (H->vec_cols > 0 && H->vec_cols < vpl) vpl = H->vec_cols;
 #define ROWS32_U(V, E, P, U)                                                                               \
     allow_smem<k_rows_f32<V, E, U>>();                                                                      \
-    k_rows_f32<V, E, U><<<LA.blocks, LA.threads, LA.smem, s>>>((float*)const_cast<void*>(v), Y, Dup, Ddn,   \
+    launch_on(pdl, k_rows_f32<V, E, U>, LA.blocks, LA.threads, LA.smem, s, (float*)const_cast<void*>(v), Y, Dup, Ddn,   \
         dn.blk_off, dn.blk_cnt, P, upd ? (const float*)upd->fo : nullptr, upd ? (float)upd->a : 0.0f,       \
         upd ? (float)upd->inv : 1.0f, upd ? upd->dv : nullptr)
 #define ROWS32(V, E, P) if (upd) { ROWS32_U(V, E, P, true); } else { ROWS32_U(V, E, P, false); }
@@ -870,20 +1224,15 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #undef ROWS32
 #undef ROWS32_U
     int up_grid = 0;
-#define UP32(V)                                                                                            \
+#define UP32(V, NV)                                                                                        \
     {                                                                                                      \
-        up_grid = grid_cap(sms() * (part != nullptr ? up32_ctas<V, true>() : up32_ctas<V, false>()),      \
-                           ((Ddn + 32 * V - 1) / (32 * V)) * ((Dup + kUpRows - 1) / kUpRows));             \
-        if (part != nullptr)                                                                               \
-            k_up_f32<V, true><<<up_grid, 256, 0, s>>>((const float*)v, Y, (float*)w, (const float*)w_old,  \
-                Dup, Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t,           \
-                (float)H->U, (float)-beta, part, done, dv, hist);                                                   \
-        else                                                                                               \
-            k_up_f32<V, false><<<up_grid, 256, 0, s>>>((const float*)v, Y, (float*)w, (const float*)w_old, \
-                Dup, Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t,           \
-                (float)H->U, (float)-beta, part, done, nullptr, nullptr);                                                \
+        const UpGrid g = up_grid_for(H, (Ddn + 32 * V * NV - 1) / (32 * V * NV), sms() * 4);               \
+        up_grid = g.gx * g.gy;                                                                             \
+        launch_on(pdl, part != nullptr ? k_up_f32<V, NV, true> : k_up_f32<V, NV, false>, up_grid, 256, g.smem, s, \
+            (const float*)v, Y, (float*)w, (const float*)w_old, Dup, Ddn, g, up.pn_ptr, up.pn_npos,         \
+            up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U, (float)-beta, part, done, dv, hist); \
     }
-    if (vpl == 4) { UP32(4) } else if (vpl == 2) { UP32(2) } else { UP32(1) }
+    if (vpl == 4) { UP32(4, 1) } else if (vpl == 2) { UP32(2, 2) } else { UP32(1, 2) }
 #undef UP32
     if (part != nullptr && nparts != nullptr) *nparts = up_grid;
     HUB_CUDA(cudaGetLastError());
