@@ -41,6 +41,15 @@ __device__ __forceinline__ void mac128(I128& acc, long long a, long long b) {
     acc.lo = nlo;
 }
 
+// acc + a * 2^s, 0 <= s < 62 (a product with a power of two)
+__device__ __forceinline__ void addshift128(I128& acc, long long a, int s) {
+    const unsigned long long plo = (unsigned long long)a << s;
+    const long long phi = s == 0 ? a >> 63 : a >> (64 - s);
+    const unsigned long long nlo = acc.lo + plo;
+    acc.hi += phi + (nlo < plo ? 1 : 0);
+    acc.lo = nlo;
+}
+
 // (hi * 2^64 + lo) * 2^e2, rounded to nearest (ties to even)
 __device__ __forceinline__ double i128_to_double(I128 v, int e2) {
     unsigned long long lo = v.lo;
@@ -117,7 +126,14 @@ struct EpiParams {
     int ju;
     long long Uint;       // U * 2^ju
     double mbeta;         // -beta, applied after the exact part in the int64 path
+    int apow;             // A = +-2^apow exactly (t a power of two), or -1
 };
+
+// acc += A T: a shift where t is a power of two (the same 128-bit value)
+__device__ __forceinline__ void mac_t(I128& acc, long long T, const EpiParams& ep) {
+    if (ep.apow >= 0) addshift128(acc, ep.A < 0 ? -T : T, ep.apow);
+    else mac128(acc, T, ep.A);
+}
 
 __device__ __forceinline__ void add4(int4& A, int4 a, int4 b, int4 c, int4 d) {
     A.x += a.x + b.x + c.x + d.x;
@@ -295,12 +311,14 @@ inline EpiParams make_epilogue(double t, double U, int ns, double beta, int W) {
     // H v is formed exactly in int64 and rounded once; a -beta w_old term is then added with
     // one fused multiply-add (a second rounding)
     p.fast = 0;
+    p.apow = -1;
     p.mbeta = -beta;
     if (t != 0.0) {
         int et = 0;
         const double mt = std::frexp(std::fabs(t), &et);   // |t| = mt * 2^et, mt in [0.5, 1)
         if (mt == 0.5) {
             et -= 1;                                        // |t| = 2^et
+            if (et + m >= 0 && et + m < 62) p.apow = et + m;
             for (int ju = 0; ju <= 8; ++ju) {
                 const double us = std::ldexp(U, ju);
                 if (us == std::floor(us) && std::fabs(us) * ns < 16384.0 && et + ju >= 0 && et + ju <= 6) {

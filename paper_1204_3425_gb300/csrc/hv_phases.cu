@@ -58,7 +58,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
                                                      const int64_t* __restrict__ boff,
                                                      const int32_t* __restrict__ bcnt,
                                                      const EntT* __restrict__ ent,
-                                                     const int* __restrict__ emax_p, int fixed_emax,
+                                                     int* emax_p, int fixed_emax, int scan,
                                                      const double* __restrict__ fo, double ua, double uinv,
                                                      const LzDev* __restrict__ dv) {
     using S = typename FxVec<VEC>::T;
@@ -72,7 +72,26 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
     }
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S* X = reinterpret_cast<S*>(smem_raw);
-    const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
+    int emax = fixed_emax;
+    if (!UPD && scan) {
+        // a sector this small: every CTA finds max|v| itself (the same word from
+        // all of them), which saves the pass before this one
+        __shared__ int emax_s;
+        if (threadIdx.x == 0) emax_s = 1;
+        __syncthreads();
+        int m = 1;
+        const int n = (int)(Dup * Ddn);
+#pragma unroll 8
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            m = max(m, (int)(((unsigned long long)__double_as_longlong(v[i]) >> 52) & 0x7FF));
+        m = __reduce_max_sync(0xffffffffu, m);
+        if ((threadIdx.x & 31) == 0) atomicMax(&emax_s, m);
+        __syncthreads();
+        emax = emax_s;
+        if (threadIdx.x == 0) *emax_p = emax;
+    } else if (fixed_emax <= 0) {
+        emax = max(*emax_p, 1);
+    }
     const int lane = threadIdx.x & 31;
     const int64_t nblk = (Dup + VEC - 1) / VEC;
     const int64_t step = blockDim.x;
@@ -151,6 +170,71 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
     }
 }
 
+// Row phase for binary64 rows of which only one 4-byte word per element fits in
+// shared memory (28672 < D_dn <= 58000): the (lo, hi) words are staged and summed
+// apart.  A plane is one word of one row; the 2 Dup planes, split into groups of
+// 32 columns, are dealt to the CTAs in equal contiguous ranges, so a few long
+// rows still fill the device evenly (153 rows of 48620 elements are two waves of
+// one row per SM).  A gather from L2 fetched a 32-byte sector at L2 latency for
+// eight bytes; here it is two conflict-free shared loads (153 x 48620 elements:
+// product 304 -> 236 us).  The CTA that begins a row's lo plane also writes its
+// fixed-point copy X.  Ys holds the two word sums of an element side by side and
+// the up phase joins them: joined here, each CTA would stage both words of two
+// rows instead of three planes (259 us).
+template <typename EntT>
+__global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* __restrict__ v, int* __restrict__ Ys,
+                                                            int2* __restrict__ Xg, int64_t Dup, int64_t Ddn,
+                                                            const int64_t* __restrict__ boff,
+                                                            const int32_t* __restrict__ bcnt,
+                                                            const EntT* __restrict__ ent,
+                                                            const int* __restrict__ emax_p, int fixed_emax) {
+    grid_dep_wait();
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int* Xs = reinterpret_cast<int*>(smem_raw);
+    const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int n = (int)Ddn, z0 = (int)staged_slots(Ddn) - 32;
+    if (threadIdx.x < 32) Xs[z0 + threadIdx.x] = 0;
+    const int64_t G = (Ddn + 31) >> 5, T = 2 * Dup * G;
+    const int64_t t1 = T * (blockIdx.x + 1) / gridDim.x;
+    for (int64_t t = T * blockIdx.x / gridDim.x; t < t1;) {
+        const int64_t q = t / G, u = q >> 1;
+        const int plane = (int)(q & 1);
+        const int g0 = (int)(t - q * G), g1 = (int)min(G, t1 - q * G);
+        const double* row = v + u * Ddn;
+        int2* xrow = plane == 0 && g0 == 0 ? Xg + u * Ddn : nullptr;
+        constexpr int NL = 8;
+        for (int d0 = threadIdx.x; d0 < n; d0 += NL * blockDim.x) {
+            double x[NL];
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                const int d = d0 + i * blockDim.x;
+                x[i] = d < n ? __ldg(row + d) : 0.0;
+            }
+#pragma unroll
+            for (int i = 0; i < NL; ++i) {
+                const int d = d0 + i * blockDim.x;
+                if (d >= n) break;
+                int lo, hi;
+                fx_split(x[i], emax, lo, hi);
+                Xs[d] = plane ? hi : lo;
+                if (xrow != nullptr) xrow[d] = make_int2(lo, hi);
+            }
+        }
+        __syncthreads();
+        for (int g = g0 + warp; g < g1; g += nw) {
+            int a = 0;
+            for_each_hop<EntT>(ent + boff[g], bcnt[g], lane, [&](uint32_t e) {
+                a += RowEnt<EntT>::sgn(e) * Xs[RowEnt<EntT>::idx(e)];
+            });
+            const int d = g * 32 + lane;
+            if (d < n) Ys[2 * (u * Ddn + d) + plane] = a;
+        }
+        __syncthreads();
+        t = q * G + g1;
+    }
+}
+
 // Row phase for binary64 rows too long for shared memory: the fixed-point
 // copy X is already in global memory (k_to_fixed) and the down-hop gathers
 // read row u of it through L1/L2.
@@ -181,6 +265,14 @@ __global__ void __launch_bounds__(512) k_rows_global_f64x(const int2* __restrict
     }
 }
 
+
+// The last CTA of a kernel sets the exponent word it has read back to 0 for the
+// next product (counter: nullptr, nothing to do; it returns to 0 by itself).
+__device__ __forceinline__ void reset_exponent(int* emax_p, unsigned* counter) {
+    if (counter == nullptr || threadIdx.x != 0) return;
+    __threadfence();
+    if (atomicInc(counter, gridDim.x - 1) == gridDim.x - 1) *emax_p = 0;
+}
 
 // Up phase, binary64 fixed point (Algorithms 2 and 4):
 //   W[u, c] = -t (sum_{(u', s) in hops_up(u)} s X[u', c] + Y[u, c]) + U n(u, c) X[u, c]  [- beta w_old]
@@ -263,7 +355,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                                                      const uint32_t* __restrict__ list,
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd, EpiParams ep,
-                                                     const int* __restrict__ emax_p, int fixed_emax) {
+                                                     int* emax_p, int fixed_emax, unsigned* reset) {
     using IV = typename FxVec<VPL>::T;
     __shared__ long long Bs[33];
     for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
@@ -343,7 +435,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                         if (w_old != nullptr) r[j] = fma(ep.mbeta, w_old[J + j], r[j]);
                     } else {
                         I128 acc{0ull, 0ll};
-                        mac128(acc, fx_join(lo[j], hi[j]) + yv[j], ep.A);
+                        mac_t(acc, fx_join(lo[j], hi[j]) + yv[j], ep);
                         mac128(acc, fx_join(xo[j].x, xo[j].y), Bs[__popc(su_u & sdc[j])]);
                         if (w_old != nullptr) {
                             int glo, ghi;
@@ -358,6 +450,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
             }
         }
     }
+    reset_exponent(emax_p, reset);
 }
 
 // Lanczos-step variant of k_up_f64x (Algorithm 1 fused with Algorithms 2, 4):
@@ -464,7 +557,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                         if (w_old != nullptr) r[j] = fma(ep.mbeta, VPL == 2 ? wpre[j] : w_old[J + j], r[j]);
                     } else {
                         I128 acc{0ull, 0ll};
-                        mac128(acc, fx_join(lo[j], hi[j]) + yv[j], ep.A);
+                        mac_t(acc, fx_join(lo[j], hi[j]) + yv[j], ep);
                         mac128(acc, fx_join(xo[j].x, xo[j].y), Bs[__popc(su_u & sdc[j])]);
                         if (w_old != nullptr) {
                             int glo, ghi;
@@ -638,8 +731,8 @@ __device__ __forceinline__ void up_segments(unsigned char* smem, int64_t Dup, in
 
 // Binary64 fixed point, resident rows.  STEP: the Lanczos step, W = H f - beta w_old with, per
 // CTA, the partials of <W, f>, <W, W> and <f, f> (block_sum3_store).  CT: CTAs
-// per SM the launch bounds keep.
-template <int VPL, bool FAST, bool STEP, int CT>
+// per SM the launch bounds keep.  YS: Y holds word pairs (k_rows_planes_f64x).
+template <int VPL, bool FAST, bool STEP, bool YS, int CT>
 __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
                                                      UpGrid g, const int32_t* __restrict__ ptr,
@@ -648,7 +741,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
-                                                     const int* __restrict__ emax_p, int fixed_emax,
+                                                     int* emax_p, int fixed_emax, unsigned* reset,
                                                      const double* __restrict__ fv, double* part,
                                                      unsigned* done, LzDev* dv, double* hist) {
     grid_dep_wait();
@@ -733,7 +826,8 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                 T = fx_join(A.x, A.y);
                 xo = fx_join(xo4.x, xo4.y);
             }
-            T += yv[j];
+            if constexpr (YS) T += fx_join((int)yv[j], (int)(yv[j] >> 32));
+            else T += yv[j];
             const int nd = __popc(su_u & sdc[j]);
             if constexpr (FAST) {
                 // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
@@ -744,7 +838,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                 if (STEP && w_old != nullptr) res[j] = fma(mbeta, wv[j], res[j]);
             } else {
                 I128 acc{0ull, 0ll};
-                mac128(acc, T, ep.A);
+                mac_t(acc, T, ep);
                 mac128(acc, xo, Bs[nd]);
                 if (STEP && w_old != nullptr) {
                     int glo, ghi;
@@ -769,6 +863,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
         block_sum3_store(s1, s2, s3, part);
         close_sums3(part, gridDim.x, done, dv, hist);
     }
+    if (!STEP) reset_exponent(emax_p, reset);
 }
 
 // Binary32: same decomposition, float arithmetic.  NV vectors of VPL columns
@@ -1029,6 +1124,9 @@ constexpr int64_t kUpSmall = 2500000, kUpHbm = 600ll << 20;
 // HBM-sized ones CTAs that take their places early disturb the sweep (4x4 (8,8)
 // product 3.80 -> 4.10 ms).
 constexpr int64_t kPdlBytes = 100ll << 20;
+// up to this many elements every row-phase CTA scans v for its largest exponent
+// (ring 8 (4,4) product: two kernels instead of a memset and three)
+constexpr int64_t kScanElems = 16384;
 constexpr int64_t kMaxRow = (1ll << 29) - 1;       // row pitch in bytes held in 32 bits
 
 // a grid of at most `full` CTAs and no more than the work items
@@ -1090,7 +1188,13 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     // to 2 columns per lane; measured best)
     if (dtype == HUB_F64) {
         const int va = choose_vec(H->vec_rows, Ddn, 8, 2, 0);
-        int* emax = H->status;
+        // exponent word: found by the row phase itself on the smallest sectors,
+        // by a pass of its own otherwise; on sectors that launch overlapped the
+        // word is one that the last CTA of the product's up phase sets back to
+        // 0, so no memset breaks the chain of kernels
+        const int scan = fixed_emax <= 0 && w_old == nullptr && va > 0 && H->D <= kScanElems;
+        const bool self_reset = fixed_emax <= 0 && w_old == nullptr && pdl && !scan;
+        int* emax = self_reset ? H->status + 2 : H->status;
         // the deferred update goes into the row phase when it stages rows in
         // shared memory with a fixed exponent bound; otherwise it is one pass first
         if (upd != nullptr && (va == 0 || fixed_emax <= 0)) {
@@ -1098,9 +1202,9 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
                 return rc;
             upd = nullptr;
         }
-        if (fixed_emax <= 0) {
-            HUB_CUDA(cudaMemsetAsync(emax, 0, sizeof(int), s));
-            launch_max_exponent((const double*)v, H->D, emax, s);
+        if (fixed_emax <= 0 && !scan) {
+            if (!self_reset) HUB_CUDA(cudaMemsetAsync(emax, 0, sizeof(int), s));
+            launch_max_exponent((const double*)v, H->D, emax, s, self_reset);
             if (w_old != nullptr) launch_max_exponent((const double*)w_old, H->D, emax, s);
         }
         Launch LA = shape((size_t)staged_slots(Ddn) * 8 * std::max(va, 1), H->ctas_rows);
@@ -1108,8 +1212,21 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         long long* Y = (long long*)ybuf;
         int2* Xg = (int2*)((char*)ybuf + (size_t)H->D * 8);
         int extra = 0;
-        if (va == 0) {
-            // rows longer than shared memory: fixed-point copy first, then gathers through L1/L2
+        const bool ysplit = va == 0 && staged_slots(Ddn) * 4 <= smem_optin();
+        if (ysplit) {
+            // rows of which one word per element fits in shared memory
+            const size_t sm = (size_t)staged_slots(Ddn) * 4;
+            const int64_t groups = 2 * Dup * ((Ddn + 31) / 32);
+            const int blocks = grid_cap(sms(), (groups + 31) / 32);
+            extra = 1;
+#define PLANES64(E, P)                                                                                      \
+    allow_smem<k_rows_planes_f64x<E>>();                                                                    \
+    launch_on(pdl, k_rows_planes_f64x<E>, blocks, 1024, sm, s, (const double*)v, (int*)Y, Xg, Dup, Ddn, \
+        dn.blk_off, dn.blk_cnt, P, emax, fixed_emax)
+            if (dn16) { PLANES64(uint16_t, dn.ent16); } else { PLANES64(uint32_t, dn.ent32); }
+#undef PLANES64
+        } else if (va == 0) {
+            // longer rows still: fixed-point copy first, then gathers through L1/L2
             int* em = emax;
             int* fixed_word = H->status + 1;
             if (fixed_emax > 0) {
@@ -1130,7 +1247,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #define ROWS64_U(V, E, P, U)                                                                                \
     allow_smem<k_rows_f64x<V, E, U>>();                                                                      \
     launch_on(pdl, k_rows_f64x<V, E, U>, LA.blocks, LA.threads, LA.smem, s, (double*)const_cast<void*>(v), Y, Xg, Dup,   \
-        Ddn, dn.blk_off, dn.blk_cnt, P, emax, fixed_emax, upd ? (const double*)upd->fo : nullptr,            \
+        Ddn, dn.blk_off, dn.blk_cnt, P, emax, fixed_emax, scan, upd ? (const double*)upd->fo : nullptr,            \
         upd ? upd->a : 0.0, upd ? upd->inv : 1.0, upd ? upd->dv : nullptr)
 #define ROWS64(V, E, P) if (upd) { ROWS64_U(V, E, P, true); } else { ROWS64_U(V, E, P, false); }
         if (va == 2) {
@@ -1146,16 +1263,21 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         // columns per lane in the up phase: 2 when Ddn is even (16-byte loads)
         const int vpl = ((Ddn & 1) == 0 && H->vec_cols != 1) ? 2 : 1;
         const bool step = part != nullptr || w_old != nullptr;
+        unsigned* reset = self_reset ? done : nullptr;
         int up_grid = 0;
-        if (vpl == 1 || (H->D > kUpSmall && (step || H->D * 8 <= kUpHbm))) {
-            const bool three = step || H->ctas_cols == 2;
+        if (vpl == 1 || ysplit || (H->D > kUpSmall && (step || H->D * 8 <= kUpHbm))) {
+            const bool three = step || (H->ctas_cols == 2 && !ysplit);
             const UpGrid g = up_grid_for(H, (Ddn + 32 * vpl - 1) / (32 * vpl), sms() * (three ? 3 : 4));
             up_grid = g.gx * g.gy;
-#define UPR64(V, F, ST, CT)                                                                                 \
-    launch_on(pdl, k_upr_f64x<V, F, ST, CT>, up_grid, 256, g.smem, s, Xg, Y, (double*)w, (const double*)w_old, Dup, \
-        Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax, (const double*)v, \
+#define UPR64(V, F, ST, YS, CT)                                                                             \
+    launch_on(pdl, k_upr_f64x<V, F, ST, YS, CT>, up_grid, 256, g.smem, s, Xg, Y, (double*)w, (const double*)w_old, Dup, \
+        Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax, reset, (const double*)v, \
         part, done, dv, hist)
-#define UPR64_S(V, F) if (step) { UPR64(V, F, true, 3); } else if (three) { UPR64(V, F, false, 3); } else { UPR64(V, F, false, 4); }
+#define UPR64_S(V, F)                                                                                      \
+    if (ysplit) { if (step) { UPR64(V, F, true, true, 3); } else { UPR64(V, F, false, true, 4); } }        \
+    else if (step) { UPR64(V, F, true, false, 3); }                                                        \
+    else if (three) { UPR64(V, F, false, false, 3); }                                                      \
+    else { UPR64(V, F, false, false, 4); }
             if (vpl == 2) {
                 if (ep.fast) { UPR64_S(2, true) } else { UPR64_S(2, false) }
             } else {
@@ -1181,9 +1303,9 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #define UP64P(F, T)                                                                                         \
     launch_on(pdl, k_up_f64x<2, F, T, true, 3>, grid_cap(sms() * 3, up_items), 256, 0, s, Xg, Y, (double*)w, \
         (const double*)w_old, Dup, Ddn, rbr, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep,  \
-        emax, fixed_emax)
+        emax, fixed_emax, reset)
 #define UP64_T(F, T)                                                                                        \
-    if (pre) { UP64P(F, T); } else { UP64((k_up_f64x<2, F, T>))); }
+    if (pre) { UP64P(F, T); } else { UP64((k_up_f64x<2, F, T>)), reset); }
             if (part != nullptr) {                        // a Lanczos step; a replayed one (w_old alone) goes below
                 if (ep.fast) { UP64((k_up_step_f64x<2, true>)), (const double*)v, part, done, dv, hist); }
                 else { UP64((k_up_step_f64x<2, false>)), (const double*)v, part, done, dv, hist); }
@@ -1198,7 +1320,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         }
         if (part != nullptr && nparts != nullptr) *nparts = up_grid;
         HUB_CUDA(cudaGetLastError());
-        count_launches(1 + extra + (fixed_emax <= 0 ? (w_old ? 2 : 1) : 0));
+        count_launches(1 + extra + (fixed_emax <= 0 && !scan ? (w_old ? 2 : 1) : 0));
         return HUB_OK;
     }
     // binary32

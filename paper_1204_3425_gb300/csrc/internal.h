@@ -233,7 +233,8 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 // whether launch_hv_phases fuses the Lanczos reductions for this sector and dtype
 bool hv_phases_fuse(const hubbard_sector* H, int dtype);
 // max biased binary64 exponent of |v| folded into *emax (atomicMax; caller zeroes it)
-void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s);
+// (pdl: launched as launch_on)
+void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s, bool pdl = false);
 // binary64 -> (lo, hi) fixed point with the exponent bound *emax (read on the device)
 void launch_to_fixed(const double* v, int64_t n, void* X, const int* emax, cudaStream_t s);
 int launch_dot(const hubbard_sector* H, const void* x, const void* y, int64_t n, int dtype,

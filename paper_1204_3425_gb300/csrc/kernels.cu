@@ -80,6 +80,7 @@ __global__ void k_hv_reference(const T* __restrict__ v, T* __restrict__ w, int64
 
 // max biased exponent of |v| -> *emax (atomicMax; *emax must start at 0)
 __global__ void k_max_exponent(const double* __restrict__ v, int64_t n, int* emax) {
+    grid_dep_wait();
     int m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v[i]);
@@ -483,9 +484,9 @@ void launch_to_fixed(const double* v, int64_t n, void* X, const int* emax, cudaS
     k_to_fixed<<<g2, kThreads, 0, s>>>(v, (int2*)X, n, emax);
 }
 
-void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s) {
+void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s, bool pdl) {
     const int g2 = grid_for(n, kThreads * 8, sm_count() * 8);
-    k_max_exponent<<<g2, kThreads, 0, s>>>(v, n, emax);
+    launch_on(pdl, k_max_exponent, g2, kThreads, 0, s, v, n, emax);
 }
 
 int launch_hv_fast(hubbard_sector* H, const void* v, void* w, int dtype, double beta, const void* w_old,

@@ -35,3 +35,26 @@ def test_exact_products_round_once(lattice, nup, ndn, U, bits):
         want[r] = float(sum(int(c) * int(x) for c, x in zip(coef[sl], Xo[Hx.indices[sl]]))) * 2.0 ** -48
     assert np.array_equal(got, want)
     H.close()
+
+
+@pytest.mark.parametrize("nup,ndn,U", [(0, 8, 4.0), (1, 9, 7.3), (1, 10, 4.0), (2, 8, 0.0)])
+def test_long_rows_match_the_reference_kernel(nup, ndn, U):
+    """Rows of 43758 and 48620 elements: one word per element staged at a time.
+    Bound: 1e-12 |t| max|v| for the fixed-point path plus the native kernel's own
+    rounding, (W + U n) 2^-52 max|v| < 1e-13."""
+    import paper_1204_3425_gb300 as hub
+    from workload import ring
+    H = hub.hubbard_sector_create(18, ring(18), nup, ndn, 1.0, U)
+    v = torch.from_numpy(np.random.default_rng(7).uniform(-1, 1, H.D)).cuda()
+    w, r = torch.empty_like(v), torch.empty_like(v)
+    hub.hubbard_apply(H, v, w)
+    hub.hubbard_apply_reference(H, v, r)
+    assert float((w - r).abs().max()) <= 1.1e-12
+    # the Lanczos step reads the same row sums: a_1, b_2 of a unit vector
+    f = v / v.norm()
+    res = hub.lanczos_ground_state(H, f, 3, 0.0)
+    hub.hubbard_apply_reference(H, f, r)
+    a = float(f @ r)
+    b = float((r - a * f).norm())
+    assert abs(res["alpha"][0] - a) <= 1e-11 * max(1.0, abs(a)) and abs(res["beta"][0] - b) <= 1e-11 * b
+    H.close()
