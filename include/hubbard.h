@@ -525,7 +525,7 @@ int hubbard_batch_schedule_table(hubbard_batch_t B, int64_t* rows, int cap, int*
  * HUB_EINVAL on a null batch or an out-of-range shape or mode. */
 int hubbard_batch_set_shape_mode(hubbard_batch_t B, int shape, int mode);
 
-/* CTAs (0 by default) that start on the one-CTA tasks at once while the rest
+/* CTAs (32 by default) that start on the one-CTA tasks at once while the rest
  * of the grid runs the sweep (the sweep CTAs join the tasks when it ends);
  * capped at the number of tasks, and at half the grid.  A sector's arithmetic
  * does not depend on it.  HUB_EINVAL on a null batch or a negative count. */

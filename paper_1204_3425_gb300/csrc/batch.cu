@@ -31,6 +31,7 @@
 #include "internal.h"
 #include "row_blocks.cuh"
 #include "splitmix.cuh"
+#include "hv_epilogue.cuh"
 
 namespace hub {
 namespace {
@@ -177,7 +178,9 @@ __device__ bool grid_barrier(unsigned int* ctr, int nctas, unsigned gen, long lo
     return *flag != 0;
 }
 
-// ---- device tridiagonal helpers (thread-serial; m <= max_iters) -------------
+// ---- device tridiagonal helpers of the one-CTA tasks (m <= max_iters) --------
+// (The serving tests hold the queued solver's tasks to the time they took with
+// these; the sweep, where every other CTA waits for a test, uses the warp's.)
 // Number of eigenvalues of T_m below x: sign changes of the characteristic
 // polynomials p_0 = 1, p_1 = a_0 - x, p_k = (a_{k-1} - x) p_{k-1} - b_{k-2}^2 p_{k-2}
 // (Sturm sequence).  No division (the binary64 divide is slow on this part);
@@ -278,6 +281,141 @@ __device__ __noinline__ double d_last_component(const double* a, const double* b
     return exp2(-0.5 * scale_log) / sqrt(n2);
 }
 
+// ---- device tridiagonal helpers of the sweep, run by one warp ----------------
+// The FP64 pipe takes two lanes a clock, so a test on all 15 warps of a CTA
+// cost 15 times the pipe time of one on a single warp for half the rounds:
+// some 0.5 ms at 100 steps, more than the 8 steps between two tests.
+
+// (double) n for 0 <= n <= 32, by integer operations
+__device__ __forceinline__ double small_double(int n) {
+    const int e = 31 - __clz(n);
+    return __hiloint2double(n ? ((1023 + e) << 20) | ((n << (20 - e)) & 0xFFFFF) : 0, 0);
+}
+__device__ __forceinline__ int exp_bits(double x) { return (__double2hiint(x) >> 20) & 0x7FF; }
+
+// Number of eigenvalues of T_m below each lane's x: sign changes of the
+// characteristic polynomials p_0 = 1, p_1 = a_0 - x,
+// p_k = (a_{k-1} - x) p_{k-1} - b_{k-2}^2 p_{k-2} (Sturm sequence).  No division;
+// both terms are rescaled by 2^-600 / 2^600 when they leave a safe range, tested
+// every fourth step while every entry is below 2^50 in magnitude (a step then
+// grows them at most 2^102 times), every step otherwise.  Signs and magnitudes
+// are read from the bits.  A zero p_k takes the sign of p_{k-1}.
+__device__ __noinline__ int warp_sturm(const double* a, const double* b, int m, double x, bool large) {
+    double p0 = 1.0, p1 = a[0] - x;
+    int s1 = p1 < 0.0;                                    // sign used for counting
+    int c = s1;
+    for (int i0 = 1; i0 < m; i0 += 4) {
+        double av[4], bv[4];
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            const int i = min(i0 + q, m - 1);
+            av[q] = a[i] - x;
+            bv[q] = b[i - 1] * b[i - 1];
+        }
+#pragma unroll
+        for (int q = 0; q < 4; ++q) {
+            if (i0 + q < m) {
+                const double p2 = fma(av[q], p1, -(bv[q] * p0));
+                const int hi = __double2hiint(p2), lo = __double2loint(p2);
+                const int s2 = ((hi << 1) | lo) != 0 ? (int)((unsigned)hi >> 31) : s1;
+                c += s2 != s1;
+                s1 = s2;
+                p0 = p1;
+                p1 = p2;
+                if (q == 3 || large) {
+                    const int e = max(exp_bits(p0), exp_bits(p1));
+                    if (e > 1023 + 600) {
+                        p0 *= 0x1p-600;
+                        p1 *= 0x1p-600;
+                    } else if (e < 1023 - 600 && (p0 != 0.0 || p1 != 0.0)) {
+                        p0 *= 0x1p600;
+                        p1 *= 0x1p600;
+                    }
+                }
+            }
+        }
+    }
+    return c;
+}
+
+// Lowest eigenvalue of T_m by multisection: every lane of the warp evaluates the
+// Sturm count at its own point of the bracket, which shrinks 33 times a round.
+// prev (or NaN) is an upper bound from an earlier step (interlacing).
+__device__ double warp_lowest_eig(const double* a, const double* b, int m, double prev) {
+    const int lane = threadIdx.x & 31;
+    double glo = a[0], ghi = a[0];
+    for (int i = lane; i < m; i += 32) {
+        const double r = (i > 0 ? fabs(b[i - 1]) : 0.0) + (i + 1 < m ? fabs(b[i]) : 0.0);
+        glo = fmin(glo, a[i] - r);
+        ghi = fmax(ghi, a[i] + r);
+    }
+    for (int o = 16; o > 0; o >>= 1) {
+        glo = fmin(glo, __shfl_xor_sync(0xffffffffu, glo, o));
+        ghi = fmax(ghi, __shfl_xor_sync(0xffffffffu, ghi, o));
+    }
+    const bool large = !(fmax(fabs(glo), fabs(ghi)) < 0x1p50);
+    double lo = glo, hi = ghi;
+    if (prev == prev) {
+        // warm bracket [prev - 1e-6, prev + 1e-12] (relative), checked by two lanes
+        const double wl = prev - 1e-6 * fmax(1.0, fabs(prev)), wh = prev + 1e-12 * fmax(1.0, fabs(prev));
+        const int c = warp_sturm(a, b, m, lane == 0 ? wl : wh, large);
+        const bool okl = wl > glo && __shfl_sync(0xffffffffu, c, 0) == 0;
+        const bool okh = wh < ghi && __shfl_sync(0xffffffffu, c, 1) >= 1;
+        if (okh) hi = wh;
+        if (okl && okh) lo = wl;
+    }
+    for (int round = 0; round < 20; ++round) {
+        if (!(hi - lo > 4e-16 * fmax(fabs(lo), fabs(hi)))) break;
+        const double x = lo + (hi - lo) * (double)(lane + 1) / 33.0;
+        // the first point with a positive count bounds the eigenvalue (computed
+        // counts need not be monotone in x near an eigenvalue)
+        const unsigned pos = __ballot_sync(0xffffffffu, warp_sturm(a, b, m, x, large) >= 1);
+        const int k = pos ? __ffs((int)pos) - 1 : 32;
+        const double nlo = k == 0 ? lo : __shfl_sync(0xffffffffu, x, k - 1 & 31);
+        const double nhi = k == 32 ? hi : __shfl_sync(0xffffffffu, x, k & 31);
+        if (!(nhi - nlo < hi - lo)) break;                // the points no longer divide the bracket
+        lo = nlo;
+        hi = nhi;
+    }
+    return 0.5 * (lo + hi);
+}
+
+// |last component| of the unit eigenvector of T_m for eigenvalue th: solve the
+// eigen-equations backwards from y_m = 1 (the lowest eigenvector grows in that
+// direction), rescaling by powers of two; returns 1 / |y|.  The warp takes the
+// reciprocals of 32 off-diagonals at a time, the recurrence runs in every lane.
+__device__ __noinline__ double warp_last_component(const double* a, const double* b, int m, double th) {
+    if (m == 1) return 1.0;
+    const int lane = threadIdx.x & 31;
+    double y1 = 0.0, y0 = 1.0;                         // y_{i+2}, y_{i+1} before row i
+    double n2 = 1.0;
+    double scale_log = 0.0;                            // n2 and the y's carry 2^scale_log
+    // row i (i = m-1 .. 1): b_{i-1} y_{i-1} + (a_i - th) y_i + b_i y_{i+1} = 0
+    for (int t0 = m - 1; t0 >= 1; t0 -= 32) {
+        const int i = t0 - lane;
+        const double ai = i >= 1 ? a[i] - th : 0.0;
+        const double bi = i >= 1 && i < m - 1 ? b[i] : 0.0;
+        const double ri = i >= 1 ? 1.0 / b[i - 1] : 0.0;
+        const int n = min(32, t0);
+        for (int q = 0; q < n; ++q) {
+            const double d = __shfl_sync(0xffffffffu, ai, q), e = __shfl_sync(0xffffffffu, bi, q),
+                         r = __shfl_sync(0xffffffffu, ri, q);
+            const double ym = -(d * y0 + e * y1) * r;
+            y1 = y0;
+            y0 = ym;
+            n2 += ym * ym;
+            if (max(exp_bits(y0), exp_bits(y1)) > 1023 + 300) {
+                y0 *= 0x1p-300;
+                y1 *= 0x1p-300;
+                n2 *= 0x1p-600;
+                scale_log += 600.0;
+            }
+        }
+    }
+    // |y|^2 = n2 * 2^scale_log; y_m was 1 in the unscaled frame
+    return exp2(-0.5 * scale_log) / sqrt(n2);
+}
+
 // One sector as seen by the element pass.
 struct SecView {
     const int2* X;         // fixed-point copy of f (global)
@@ -286,7 +424,7 @@ struct SecView {
     const int32_t *urp, *drp;
     const uint32_t *uent, *dent, *ust, *dst;
     int64_t Ddn;
-    double U, scale;       // scale = -t * 2^-47
+    double U, mt;          // mt = -t (of the hop sum in units of 2^-47)
     // down-spin row table (nullptr: per-lane CSR lists instead); used when the
     // row is staged with its zero slots
     const int64_t* dbo = nullptr;
@@ -308,6 +446,9 @@ __host__ __device__ __forceinline__ int64_t row_slots(int64_t Ddn) { return (Ddn
 // elements) the down-hops walk the coloured row table: the same slot count
 // for all lanes of a group and no shared-memory bank conflicts; otherwise each
 // lane walks its own CSR list.  Adds this lane's <q,f>, <q,q>, <f,f> over the row.
+// SWEEP: the conversions of the epilogue by integer operations (five slots of
+// the FP64 pipe for the hop sum, two for the occupation; the same bits).
+template <bool SWEEP>
 __device__ __forceinline__ void row_pass(const SecView& V, int64_t u, int2* buf, double beta, double& ap,
                                          double& qq, double& ff) {
     const int lane = threadIdx.x & 31;
@@ -362,7 +503,10 @@ __device__ __forceinline__ void row_pass(const SecView& V, int64_t u, int2* buf,
             const int64_t j = u * Ddn + d;
             const long long Sx = ((long long)hi << 24) + (long long)lo;
             const double fj = __ldcg(V.f + j);
-            const double q = fma(-beta, __ldcg(V.g + j), fma(V.U * (double)__popc(su_u & V.dst[d]), fj, V.scale * (double)Sx));
+            const int nd = __popc(su_u & V.dst[d]);
+            const double Un = V.U * (SWEEP ? small_double(nd) : (double)nd);
+            const double hop = SWEEP ? V.mt * i64_scaled_to_double(Sx, -47) : (V.mt * 0x1p-47) * (double)Sx;
+            const double q = fma(-beta, __ldcg(V.g + j), fma(Un, fj, hop));
             V.g[j] = q;
             ap = fma(q, fj, ap);
             qq = fma(q, q, qq);
@@ -390,8 +534,8 @@ __device__ __forceinline__ double warp_sum(double v) {
 // Vector data written in one phase and read in another goes through L2
 // (__ldcg): the near-breakdown pass of phase R rewrites rows that other SMs
 // read next.
-__device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double* red, int* flag, int* sh_flags,
-                                         double* sh_k, int* sh_stop, double* sh_out) {
+__device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double* red, int* flag, int* sh_stop,
+                                         double* sh_out) {
     unsigned ggen = 0;
     const int G = P.sweep_ctas;                        // CTAs of the sweep: blockIdx.x < G
     auto gsync = [&]() -> bool {
@@ -405,11 +549,10 @@ __device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double*
     if (blockIdx.x == 0 && threadIdx.x == 0) *P.nactive = P.nswp;
     // rows of the element and update phases are claimed one at a time (heaviest
     // sectors first), so warps that drew cheap rows take more of them
-    auto claim = [&](int c) -> int64_t {
-        unsigned long long r = 0ull;
-        if (lane == 0) r = atomicAdd(P.claim + c, 1ull);
-        return (int64_t)__shfl_sync(0xffffffffu, r, 0);
-    };
+    // (the next row's claim goes out before the current row's work, which hides
+    // the atomic's round trip)
+    auto ask = [&](int c) -> unsigned long long { return lane == 0 ? atomicAdd(P.claim + c, 1ull) : 0ull; };
+    auto told = [&](unsigned long long r) -> int64_t { return (int64_t)__shfl_sync(0xffffffffu, r, 0); };
     // a claimed row of a sector that has stopped: move the counter past the
     // sector's last row (the counter only grows, so every row it skips is of
     // that sector), and the other warps stop claiming its rows one by one
@@ -461,7 +604,9 @@ __device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double*
         double* fp = (it & 1) ? P.g : P.f;          // f_j and f_{j-1} swap pools each step
         double* gp = (it & 1) ? P.f : P.g;
         // E
-        for (int64_t r = claim(0); r < nrows; r = claim(0)) {
+        unsigned long long nx = 0ull;
+        for (int64_t r = told(ask(0)); r < nrows; r = told(nx)) {
+            nx = ask(0);
             const int k = locate(r);
             if (!__ldcg(&P.sst[k].active)) {
                 skip_sector(0, k);
@@ -476,10 +621,10 @@ __device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double*
             const bool blk = S.dn_blk >= 0 && row_slots(S.Ddn) <= slice;
             const SecView V{P.xg + S.voff, fp + S.voff, gp + S.voff, P.rp + S.up_rp, P.rp + S.dn_rp,
                             P.ent + S.up_ent, P.ent + S.dn_ent, P.st + S.up_st, P.st + S.dn_st, S.Ddn, S.U,
-                            -S.t * 0x1p-47, blk ? P.bo + S.dn_blk : nullptr, blk ? P.bc + S.dn_blk : nullptr,
+                            -S.t, blk ? P.bo + S.dn_blk : nullptr, blk ? P.bc + S.dn_blk : nullptr,
                             P.be};
             double ap = 0.0, qq = 0.0, ff = 0.0;
-            row_pass(V, r - P.rowoff[k], buf, __ldcg(&P.sst[k].beta), ap, qq, ff);
+            row_pass<true>(V, r - P.rowoff[k], buf, __ldcg(&P.sst[k].beta), ap, qq, ff);
             ap = warp_sum(ap);
             qq = warp_sum(qq);
             ff = warp_sum(ff);
@@ -526,9 +671,13 @@ __device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double*
             st.broke = bn <= 1e-13 * st.amax;
             if (st.broke || (m >= 8 && (m % (m >= 32 ? 2 * kCheckEvery : kCheckEvery)) == 0) || m == mcap) {
                 __syncthreads();                         // A, B written by thread 0
-                const double th = cta_lowest_eig(A, B, m, st.prev, sh_flags, sh_k);
+                double th = 0.0, sl = 0.0;
+                if (threadIdx.x < 32) {
+                    th = warp_lowest_eig(A, B, m, st.prev);
+                    sl = warp_last_component(A, B, m, th);
+                }
                 if (threadIdx.x == 0) {
-                    const double rho = bn * d_last_component(A, B, m, th);
+                    const double rho = bn * sl;
                     const int conv = st.broke || (rho < P.tol * fmax(1.0, fabs(th)));
                     *sh_stop = conv || m == mcap;
                     sh_out[0] = th;
@@ -563,7 +712,8 @@ __device__ __noinline__ bool sweep_solve(const BatchParams& P, int2* xs, double*
         if (!gsync()) return false;
         // U
         if (blockIdx.x == 0 && threadIdx.x == 0) P.claim[0] = 0ull;   // E of the next step starts after a barrier
-        for (int64_t r = claim(1); r < nrows; r = claim(1)) {
+        for (int64_t r = told(ask(1)); r < nrows; r = told(nx)) {
+            nx = ask(1);
             const int k = locate(r);
             if (!__ldcg(&P.sst[k].active)) {
                 skip_sector(1, k);
@@ -610,7 +760,7 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_lanczos(BatchParams 
     __shared__ double sh_out[2];
     // the larger sectors first, in lock step over the whole grid; then the
     // smaller ones, one CTA each
-    if (P.nswp > 0 && (int)blockIdx.x < P.sweep_ctas && !sweep_solve(P, xs, red, &flag, sh_flags, sh_k, &stop, sh_out))
+    if (P.nswp > 0 && (int)blockIdx.x < P.sweep_ctas && !sweep_solve(P, xs, red, &flag, &stop, sh_out))
         return;
     __shared__ int sh_task;
     const bool queued = P.q_posted != nullptr;
@@ -727,10 +877,10 @@ __global__ void __launch_bounds__(kBatchThreads, 2) k_batch_lanczos(BatchParams 
                 }
             } else {
                 // global copy (L2): a warp per row (row_pass)
-                const SecView V{X, f, g, urp, drp, uent, dent, ust, dst, Ddn, S.U, scale,
+                const SecView V{X, f, g, urp, drp, uent, dent, ust, dst, Ddn, S.U, -S.t,
                                 blk ? P.bo + S.dn_blk : nullptr, blk ? P.bc + S.dn_blk : nullptr, P.be};
                 int2* buf = rowbuf ? xs + (int64_t)warp * rstride : nullptr;
-                for (int64_t u = warp; u < Dup; u += nwarps) row_pass(V, u, buf, beta, ap, qq, ff);
+                for (int64_t u = warp; u < Dup; u += nwarps) row_pass<false>(V, u, buf, beta, ap, qq, ff);
             }
             double sv[3] = {ap, qq, ff};
             cta_sum(3, sv);
@@ -845,7 +995,11 @@ struct hubbard_batch {
     uint16_t* d_be = nullptr;
     // schedule
     int64_t elems_per_cta = 1 << 14;
-    int task_ctas = 0;                         // CTAs that start on the one-CTA tasks while the rest sweep
+    // CTAs that start on the one-CTA tasks while the rest sweep: the sweep of a
+    // mix does not fill the device in its later steps (256 sectors: 92.9 ms with
+    // 0, 79.9 / 61.7 / 61.2 / 60.8 with 16 / 32 / 64 / 96; 64 sectors: 72.6 ms
+    // with 0, 38.2 with 32)
+    int task_ctas = 32;
     int* d_tasks = nullptr;
     int ntasks = 0;
     size_t tasks_cap = 0;
