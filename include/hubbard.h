@@ -272,11 +272,15 @@ int hubbard_lanczos_step(hubbard_t H, const void* f, void* g, double beta_j, int
  *   psi_out    optional binary64 device vector of D elements (16-byte
  *              aligned, not overlapping the workspace) receiving the
  *              normalised Ritz vector psi = sum_j s_j f_j of the lowest Ritz
- *              value.  The Lanczos vectors are not stored: a second pass
- *              replays the same recurrence with the recorded a_j, b_j (the
- *              kernels are deterministic, so the replayed f_j are the ones of
- *              the first pass) and accumulates psi in binary64, which doubles
- *              the H*v count.  NULL skips it.
+ *              value.  The Lanczos vectors the first pass could keep are
+ *              combined in one pass: up to 1 GiB of them, taken for the call
+ *              from a pool of the library's own that holds at most as much
+ *              between calls (none where there is no room, or above 2.5e7
+ *              elements).  The rest is replayed: the same recurrence with the
+ *              recorded a_j, b_j (the kernels are deterministic, so the
+ *              replayed f_j are the ones of the first pass), accumulated in
+ *              j order (binary64; binary32 vectors in float-float), so psi is
+ *              the same however many were kept.  NULL skips it.
  *   alpha_out, beta_out  optional host arrays of max_iters doubles receiving
  *              a_1..a_m and b_2..b_{m+1}
  *   out        host result: energy (lowest Ritz value), residual rho,

@@ -7,6 +7,7 @@
 #include <functional>
 #include <list>
 #include <map>
+#include <memory>
 #include <mutex>
 #include <new>
 #include <set>
@@ -1248,42 +1249,119 @@ static int psi_accumulate(const void* f, int dtype, double* psi, int64_t n, doub
 }
 
 // Ritz vector psi = sum_j s_j f_j (binary64, accumulated in j order) of a
-// finished lanczos_core run, by replaying its recurrence: f_0 = v0 / |v0| as
-// in the run, then g <- H f_j - b_j g with the recorded b_j, and f_{j+1} =
-// (g - a_j f_j) / b_{j+1} completed inside the next H*v (the run's own
-// kernels with the same operands, hence the same f_j bit for bit).  f, g:
-// two vectors of dtype; psi is normalised on return.
-static int replay_ritz_vector(hubbard_t H, const void* v0, int v0_dtype, int dtype, const LanczosRun& R,
-                              const std::vector<double>& sv, void* f, void* g, double* psi, cudaStream_t s) {
+// finished lanczos_core run: one pass over the k f_j it stored (store + j *
+// stride bytes), the rest by replaying its recurrence from the last two of them,
+// or, with none, from f_0 = v0 / |v0|: g <- H f_j - b_j g with the recorded b_j,
+// and f_{j+1} = (g - a_j f_j) / b_{j+1} completed inside the next H*v (the run's
+// own kernels with the same operands, hence the same f_j, and the same psi
+// whatever k is, bit for bit).  f, g: two vectors of dtype; psi is normalised
+// on return.
+static int ritz_vector(hubbard_t H, const void* v0, int v0_dtype, int dtype, const LanczosRun& R,
+                       const std::vector<double>& sv, void* f, void* g, double* psi, const char* store, size_t stride,
+                       int k, cudaStream_t s) {
     int rc;
     const int m = (int)R.a.size();
-    double n0 = 0.0;
-    if ((rc = launch_dot(H, v0, v0, H->D, v0_dtype, H->red, s)) || (rc = reduce_partials_host(H->red, s, &n0)))
-        return rc;
-    if (v0_dtype == dtype) rc = launch_copy_normalise(v0, f, H->D, dtype, 1.0 / std::sqrt(n0), s);
-    else rc = launch_f64_to_f32_scaled((const double*)v0, (float*)f, H->D, 1.0 / std::sqrt(n0), s);
-    if (rc) return rc;
-    if (cudaMemsetAsync(g, 0, (size_t)H->D * elem_size(dtype), s) != cudaSuccess) return fail(HUB_ECUDA, "memset");
-    if ((rc = psi_accumulate(f, dtype, psi, H->D, sv[0], true, s))) return rc;
-    RowUpdate ru{};
-    bool have = false;
-    for (int j = 0; j + 1 < m; ++j) {
-        const double bj = j == 0 ? 0.0 : R.b[(size_t)j - 1];
-        if ((rc = launch_hv_fast(H, f, g, dtype, bj, g, 1023, s, nullptr, nullptr, have ? &ru : nullptr))) return rc;
-        if (have && (rc = psi_accumulate(f, dtype, psi, H->D, sv[(size_t)j], false, s))) return rc;
-        ru = RowUpdate{f, -R.a[(size_t)j], 1.0 / R.b[(size_t)j]};
-        have = true;
-        std::swap(f, g);
+    const size_t vbytes = (size_t)H->D * elem_size(dtype);
+    k = std::min(k, m);
+    if (k >= 1) {
+        if (dtype == HUB_F64)
+            rc = launch_psi_multi_f64((const double*)store, (int64_t)(stride / 8), k, sv.data(), H->red, psi, H->D, s);
+        else
+            rc = launch_psi_multi((const float*)store, (int64_t)(stride / 4), k, sv.data(), H->red, psi, H->D, k == m, s);
+        if (rc) return rc;
     }
-    if (have) {
-        if ((rc = launch_axpy_scale(ru.a, ru.inv, ru.fo, f, H->D, dtype, s))) return rc;
-        if ((rc = psi_accumulate(f, dtype, psi, H->D, sv[(size_t)m - 1], false, s))) return rc;
+    if (k < m) {
+        int j0 = 0;
+        if (k >= 2) {
+            if (cudaMemcpyAsync(f, store + (size_t)(k - 1) * stride, vbytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess ||
+                cudaMemcpyAsync(g, store + (size_t)(k - 2) * stride, vbytes, cudaMemcpyDeviceToDevice, s) != cudaSuccess)
+                return fail(HUB_ECUDA, "resume from stored vectors");
+            j0 = k - 1;
+        } else {
+            double n0 = 0.0;
+            if ((rc = launch_dot(H, v0, v0, H->D, v0_dtype, H->red, s)) || (rc = reduce_partials_host(H->red, s, &n0)))
+                return rc;
+            if (v0_dtype == dtype) rc = launch_copy_normalise(v0, f, H->D, dtype, 1.0 / std::sqrt(n0), s);
+            else rc = launch_f64_to_f32_scaled((const double*)v0, (float*)f, H->D, 1.0 / std::sqrt(n0), s);
+            if (rc) return rc;
+            if (cudaMemsetAsync(g, 0, vbytes, s) != cudaSuccess) return fail(HUB_ECUDA, "memset");
+            if (k == 0 && (rc = psi_accumulate(f, dtype, psi, H->D, sv[0], true, s))) return rc;
+        }
+        RowUpdate ru{};
+        bool have = false;
+        for (int j = j0; j + 1 < m; ++j) {
+            const double bj = j == 0 ? 0.0 : R.b[(size_t)j - 1];
+            if ((rc = launch_hv_fast(H, f, g, dtype, bj, g, 1023, s, nullptr, nullptr, have ? &ru : nullptr))) return rc;
+            if (have && (rc = psi_accumulate(f, dtype, psi, H->D, sv[(size_t)j], false, s))) return rc;
+            ru = RowUpdate{f, -R.a[(size_t)j], 1.0 / R.b[(size_t)j]};
+            have = true;
+            std::swap(f, g);
+        }
+        if (have) {
+            if ((rc = launch_axpy_scale(ru.a, ru.inv, ru.fo, f, H->D, dtype, s))) return rc;
+            if ((rc = psi_accumulate(f, dtype, psi, H->D, sv[(size_t)m - 1], false, s))) return rc;
+        }
+        if (dtype == HUB_F32 && (rc = launch_psi_finish(psi, H->D, s))) return rc;
     }
-    if (dtype == HUB_F32 && (rc = launch_psi_finish(psi, H->D, s))) return rc;
     double pn = 0.0;
     if ((rc = launch_dot(H, psi, psi, H->D, HUB_F64, H->red, s)) || (rc = reduce_partials_host(H->red, s, &pn))) return rc;
     return launch_scale(1.0 / std::sqrt(pn), psi, H->D, HUB_F64, s);
 }
+
+// Room for the Lanczos vectors of one lanczos_ground_state call that wants a
+// Ritz vector: replaying the recurrence doubles the H*v count, the stored
+// vectors are one pass.  Taken for the call from a pool of the library's own on
+// the call's stream (one pool per device, safe across threads and streams), at
+// most kStoreBytes; the pool keeps at most that much between calls.  nullptr
+// when there is no room: the recurrence is then replayed.
+constexpr size_t kStoreBytes = 1ull << 30;
+constexpr int kStoreMin = 8;                         // fewer vectors save less than they take
+
+static cudaMemPool_t store_pool(int device) {
+    static std::mutex mu;
+    static std::map<int, cudaMemPool_t> pools;
+    std::lock_guard<std::mutex> lk(mu);
+    auto it = pools.find(device);
+    if (it != pools.end()) return it->second;
+    cudaMemPoolProps props{};
+    props.allocType = cudaMemAllocationTypePinned;
+    props.location.type = cudaMemLocationTypeDevice;
+    props.location.id = device;
+    cudaMemPool_t pool = nullptr;
+    uint64_t keep = kStoreBytes;
+    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
+        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+        cudaGetLastError();
+        if (pool) cudaMemPoolDestroy(pool);
+        pool = nullptr;
+    }
+    pools[device] = pool;
+    return pool;
+}
+
+struct VectorStore {
+    char* p = nullptr;
+    size_t stride = 0;
+    int cap = 0;
+    cudaStream_t s;
+    VectorStore(hubbard_t H, int dtype, int steps, cudaStream_t st) : s(st) {
+        stride = align_up((size_t)H->D * elem_size(dtype), 256);
+        const int n = (int)std::min<size_t>((size_t)std::min(steps, kRedSlots), kStoreBytes / stride);
+        if (n < std::min(steps, kStoreMin)) return;
+        cudaMemPool_t pool = store_pool(H->device);
+        if (pool == nullptr || cudaMallocFromPoolAsync((void**)&p, (size_t)n * stride, pool, s) != cudaSuccess) {
+            cudaGetLastError();
+            p = nullptr;
+            return;
+        }
+        cap = n;
+    }
+    VectorStore(const VectorStore&) = delete;
+    VectorStore& operator=(const VectorStore&) = delete;
+    ~VectorStore() {
+        if (p) cudaFreeAsync(p, s);
+    }
+};
 
 int lanczos_ground_state(hubbard_t H, const void* v0, int max_iters, double tol, int dtype, void* workspace,
                          size_t ws_bytes, void* psi_out, void* stream, double* alpha_out, double* beta_out,
@@ -1312,7 +1390,14 @@ int lanczos_ground_state(hubbard_t H, const void* v0, int max_iters, double tol,
     char* ws = (char*)workspace;
     ScratchGuard guard(H, ws + 2 * vec, (size_t)H->D * 16);
     LanczosRun R;
-    if ((rc = lanczos_core(H, v0, dtype, max_iters, tol, dtype, ws, ws + vec, s, R))) return rc;
+    // sectors with device-resident steps keep their vectors for psi where there is room
+    const int steps = (int)std::min<int64_t>(max_iters, H->D);
+    std::unique_ptr<VectorStore> kept;
+    if (psi_out != nullptr && !lanczos_host_driven(H, dtype)) kept = std::make_unique<VectorStore>(H, dtype, steps, s);
+    char* store = kept ? kept->p : nullptr;
+    const size_t stride = kept ? kept->stride : 0;
+    const int cap = kept ? kept->cap : 0;
+    if ((rc = lanczos_core(H, v0, dtype, max_iters, tol, dtype, ws, ws + vec, s, R, 0.0, store, stride, cap))) return rc;
     const int m = (int)R.a.size();
     if (alpha_out) std::memcpy(alpha_out, R.a.data(), m * sizeof(double));
     if (beta_out) std::memcpy(beta_out, R.b.data(), m * sizeof(double));
@@ -1321,7 +1406,7 @@ int lanczos_ground_state(hubbard_t H, const void* v0, int max_iters, double tol,
         std::vector<double> sv((size_t)m);
         double th = 0.0;
         tridiag_lowest_vector(R.a.data(), R.b.data(), m, &th, sv.data());
-        if ((rc = replay_ritz_vector(H, v0, dtype, dtype, R, sv, ws, ws + vec, (double*)psi_out, s))) return rc;
+        if ((rc = ritz_vector(H, v0, dtype, dtype, R, sv, ws, ws + vec, (double*)psi_out, store, stride, cap, s))) return rc;
         if (cudaStreamSynchronize(s) != cudaSuccess) return fail(HUB_ECUDA, "lanczos synchronise");
     }
     out->energy = R.theta;

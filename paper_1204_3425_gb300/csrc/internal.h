@@ -268,6 +268,10 @@ int launch_psi_accumulate_f64(const double* f, double* psi, int64_t n, double sj
 int launch_psi_multi(const float* base, int64_t stride, int m, const double* sv, void* dev, double* psi, int64_t n,
                      bool fin, cudaStream_t s);
 
+// the same for binary64 vectors, bit-identical to m launch_psi_accumulate_f64 calls
+int launch_psi_multi_f64(const double* base, int64_t stride, int m, const double* sv, double* dev, double* psi, int64_t n,
+                         cudaStream_t s);
+
 // A <- A + ca f, B <- B + cb f (binary64)
 int launch_acc2_f64(const double* f, double* A, double* B, int64_t n, double ca, double cb, cudaStream_t s);
 // A <- A + sum_{j<m} c_j f_j, B <- B + sum_{j<m} c_{m+j} f_j, f_j = base + j * stride

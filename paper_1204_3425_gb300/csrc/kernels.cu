@@ -427,6 +427,44 @@ __global__ void __launch_bounds__(256) k_psi_multi(const float* __restrict__ bas
     }
 }
 
+// psi = sum_j s_j f_j over m stored binary64 vectors, per element in j order with
+// the operations of successive k_psi_acc_f64 launches (the first a product), so
+// bit-identical to them.  Two elements per thread, eight vectors' loads in
+// flight; base, stride and psi must keep 16-byte alignment.
+__global__ void __launch_bounds__(256) k_psi_multi_f64(const double* __restrict__ base, int64_t stride, int m,
+                                                       const double* __restrict__ s, double* __restrict__ psi,
+                                                       int64_t n) {
+    constexpr int U = 8;
+    const int64_t n2 = n / 2;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
+        const double* p = base + 2 * i;
+        const double2 x0 = __ldcs(reinterpret_cast<const double2*>(p));
+        double ax = s[0] * x0.x, ay = s[0] * x0.y;
+        int j = 1;
+        for (; j + U <= m; j += U) {
+            double2 x[U];
+#pragma unroll
+            for (int q = 0; q < U; ++q) x[q] = __ldcs(reinterpret_cast<const double2*>(p + (int64_t)(j + q) * stride));
+#pragma unroll
+            for (int q = 0; q < U; ++q) {
+                ax = fma(s[j + q], x[q].x, ax);
+                ay = fma(s[j + q], x[q].y, ay);
+            }
+        }
+        for (; j < m; ++j) {
+            const double2 x = __ldcs(reinterpret_cast<const double2*>(p + (int64_t)j * stride));
+            ax = fma(s[j], x.x, ax);
+            ay = fma(s[j], x.y, ay);
+        }
+        reinterpret_cast<double2*>(psi)[i] = make_double2(ax, ay);
+    }
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        double acc = s[0] * base[n - 1];
+        for (int j = 1; j < m; ++j) acc = fma(s[j], base[(int64_t)j * stride + n - 1], acc);
+        psi[n - 1] = acc;
+    }
+}
+
 // A <- A + ca f, B <- B + cb f (binary64): one Lanczos vector's share of the
 // real and imaginary parts of a Krylov propagation
 __global__ void k_acc2_f64(const double* __restrict__ f, double* __restrict__ A, double* __restrict__ B, int64_t n,
@@ -712,6 +750,16 @@ int launch_psi_multi(const float* base, int64_t stride, int m, const double* sv,
     HUB_CUDA(cudaMemcpyAsync(dev, c.data(), c.size() * sizeof(SplitCoef), cudaMemcpyHostToDevice, s));   // pageable: staged
     const int g = grid_for(n, kThreads * 4, sm_count() * 8);
     k_psi_multi<<<g, kThreads, 0, s>>>(base, stride, m, (const SplitCoef*)dev, psi, n, fin ? 1 : 0);
+    HUB_CUDA(cudaGetLastError());
+    count_launches(1);
+    return HUB_OK;
+}
+
+int launch_psi_multi_f64(const double* base, int64_t stride, int m, const double* sv, double* dev, double* psi, int64_t n,
+                         cudaStream_t s) {
+    HUB_CUDA(cudaMemcpyAsync(dev, sv, (size_t)m * sizeof(double), cudaMemcpyHostToDevice, s));   // pageable: staged
+    const int g = grid_for(n, kThreads * 2, sm_count() * 8);
+    k_psi_multi_f64<<<g, kThreads, 0, s>>>(base, stride, m, dev, psi, n);
     HUB_CUDA(cudaGetLastError());
     count_launches(1);
     return HUB_OK;

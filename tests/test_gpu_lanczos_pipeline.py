@@ -57,3 +57,28 @@ def test_stored_vectors_end_inside_a_run(stored):
     p = psi.cpu().numpy()
     assert abs(p @ (Hx @ p) - E0) <= 1e-6 * abs(E0)
     H.close()
+
+
+@pytest.mark.parametrize("lattice,nup,ndn,U,dtype", [("ring6", 1, 1, 4.0, "f64"), ("ring8", 4, 4, 7.3, "f32"),
+                                                     ("ring13", 6, 6, 8.0, "f64"), ("ring13", 6, 7, 8.0, "f32")])
+def test_ritz_vector_of_kept_and_replayed_vectors(lattice, nup, ndn, U, dtype):
+    """All Lanczos vectors kept, or (2.9e6 elements: 46 of some 60 binary64 ones) the
+    last part replayed: psi solves the eigenproblem to the residual reported, plus
+    rounding (binary32: 2^-24 per element and operation, 1e-5 here)."""
+    import paper_1204_3425_gb300 as hub
+    from workload import lattice_by_name
+    ns, bonds = lattice_by_name(lattice)
+    H = hub.hubbard_sector_create(ns, bonds, nup, ndn, 1.0, U)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(11)
+    v = torch.rand(H.D, dtype=torch.float64, device="cuda", generator=g) * 2 - 1
+    tol = 1e-9 if dtype == "f64" else 1e-4
+    psi = torch.empty_like(v)
+    r = hub.lanczos_ground_state(H, v if dtype == "f64" else v.float(), 400, tol, psi_out=psi)
+    w = torch.empty_like(psi)
+    hub.hubbard_apply(H, psi, w)
+    theta = float(psi @ w)
+    assert abs(float(psi.norm()) - 1.0) <= 1e-12
+    assert abs(theta - r["energy"]) <= (1e-10 if dtype == "f64" else 1e-5) * abs(theta)
+    assert float((w - theta * psi).norm()) <= 2 * tol + (1e-10 if dtype == "f64" else 1e-3)
+    H.close()
