@@ -1076,10 +1076,15 @@ static bool lanczos_record_step(LanczosRun& R, double aj, double bn, double tol,
 // a_j, b_{j+1} are the same bit for bit.  A step whose fused sums cancel
 // (near breakdown) stalls the ones behind it; the host then runs the explicit
 // branch and enqueues them again.
-// Steps per chunk: two chunks cover the host's test of one (a few us a step),
-// and the steps past the end stay few.
-static int lanczos_chunk(hubbard_t H) {
-    return (int)std::max<int64_t>(1, std::min<int64_t>(4, (int64_t)(4e6 / (double)H->D)));
+// Steps per chunk: the chunk in flight covers the host's test of the one before
+// (10 to 25 us a step, growing with the steps so far, and a chunk's wait), and
+// what is run past the end is one chunk.  A run with a caller's stop test is
+// short, its tests cheap and its end a larger share (4x3 propagation, two runs
+// of 16 steps: 3.19 ms with 4 steps a chunk, 3.08 with 2; a ring 12 ground state:
+// 5.59 and 5.83).
+static int lanczos_chunk(hubbard_t H, bool short_run) {
+    if (H->D > 2000000) return 1;
+    return short_run && H->D > 100000 ? 2 : 4;
 }
 
 // whether lanczos_core takes the host-driven loop: above 2.5e7 elements a step
@@ -1091,20 +1096,24 @@ static bool lanczos_host_driven(hubbard_t H, int dtype) {
 
 static int lanczos_core(hubbard_t H, const void* v0, int v0_dtype, int max_iters, double tol, int dtype, void* f,
                         void* g, cudaStream_t s, LanczosRun& R, double rel_tol = 0.0, char* store = nullptr,
-                        size_t store_stride = 0, int store_cap = 0, const LanczosStop* stop = nullptr) {
+                        size_t store_stride = 0, int store_cap = 0, const LanczosStop* stop = nullptr,
+                        double v0_norm = 0.0) {
     if (lanczos_host_driven(H, dtype))
         return lanczos_core_host(H, v0, v0_dtype, max_iters, tol, dtype, f, g, s, R, rel_tol, store, store_stride,
                                  store_cap, stop);
     int rc;
-    const int chunk = lanczos_chunk(H);
+    const int chunk = lanczos_chunk(H, stop != nullptr);
     const int m_cap = (int)std::min<int64_t>(max_iters, H->D);
     if ((rc = ensure_lz(H, m_cap))) return rc;
     LzDev* dv = reinterpret_cast<LzDev*>(H->lz);
     double* hist = reinterpret_cast<double*>((char*)H->lz + 256);
     LzHost* pin = H->lz_host;
-    double n0 = 0.0;
-    if ((rc = launch_dot(H, v0, v0, H->D, v0_dtype, H->red, s)) || (rc = reduce_partials_host(H->red, s, &n0))) return rc;
-    n0 = std::sqrt(n0);
+    double n0 = v0_norm;                             // known to the caller (the same reduction), or 0
+    if (n0 == 0.0) {
+        if ((rc = launch_dot(H, v0, v0, H->D, v0_dtype, H->red, s)) || (rc = reduce_partials_host(H->red, s, &n0)))
+            return rc;
+        n0 = std::sqrt(n0);
+    }
     if (!(n0 > 0.0) || !std::isfinite(n0)) return fail(HUB_EINVAL, "start vector has zero or non-finite norm");
     // f_j lives in its slot of the store, past the last slot in f and g by turns;
     // step j writes H f_j - b_j f_{j-1} where f_{j+1} will be completed
@@ -1749,6 +1758,10 @@ int hubbard_time_evolve(hubbard_t H, const void* v_re, const void* v_im, double 
         if (info->steps >= kMaxSteps) return fail(HUB_ENOTCONV, "time evolution: too many steps");
         // norms of the parts of the current state; each part's share of the budget
         for (int q = 0; q < 2; ++q) {
+            if (info->steps == 0) {                  // as found above
+                nn[q] = std::sqrt(nn[q]);
+                continue;
+            }
             nn[q] = 0.0;
             if (q == 1 && !has_im) continue;
             if ((rc = launch_dot(H, part[q], part[q], H->D, HUB_F64, H->red, s)) ||
@@ -1776,7 +1789,7 @@ int hubbard_time_evolve(hubbard_t H, const void* v_re, const void* v_im, double 
             char* st = stored ? store + (size_t)q * kmax * vec : nullptr;
             if (in_store) rc = lanczos_core_in_store(H, part[q], kmax, st, vec, g, s, run.R, &stop);
             else rc = lanczos_core(H, part[q], HUB_F64, kmax, 0.0, HUB_F64, f, g, s, run.R, 0.0, st, vec,
-                                   stored ? kmax : 0, &stop);
+                                   stored ? kmax : 0, &stop, nn[q]);
             if (rc) return rc;
             const int m = (int)run.R.a.size();
             if (!krylov_exp_ends(run.R.a.data(), run.R.b.data(), m, run.E))

@@ -186,36 +186,26 @@ struct FFAcc {
 };
 
 // Lanczos reductions fused into the up-phase epilogue (Algorithm 1): the CTA
-// sums its threads' <w, f>, <w, w>, <f, f> in a fixed tree and stores the
-// per-CTA partials at part[b], part[kPartStride + b], part[2 kPartStride + b].
+// (at most 256 threads) sums its threads' <w, f>, <w, w>, <f, f> in a fixed order
+// and stores the per-CTA partials at part[b], part[kPartStride + b],
+// part[2 kPartStride + b].  One warp takes each sum, column by column over the
+// warps and then across its lanes: 39 FP64 instructions a CTA instead of the 135
+// of shuffles in every warp, which were a quarter of that pipe's work in a ring
+// 12 step.
 __device__ __forceinline__ void block_sum3_store(double a, double b, double c, double* part) {
-    __shared__ double red[3][32];
-    for (int o = 16; o > 0; o >>= 1) {
-        a += __shfl_xor_sync(0xffffffffu, a, o);
-        b += __shfl_xor_sync(0xffffffffu, b, o);
-        c += __shfl_xor_sync(0xffffffffu, c, o);
-    }
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (lane == 0) {
-        red[0][wid] = a;
-        red[1][wid] = b;
-        red[2][wid] = c;
-    }
+    __shared__ double red[3][256];
+    red[0][threadIdx.x] = a;
+    red[1][threadIdx.x] = b;
+    red[2][threadIdx.x] = c;
     __syncthreads();
-    if (wid == 0) {
-        const int nw = (blockDim.x + 31) >> 5;
-        a = lane < nw ? red[0][lane] : 0.0;
-        b = lane < nw ? red[1][lane] : 0.0;
-        c = lane < nw ? red[2][lane] : 0.0;
-        for (int o = 16; o > 0; o >>= 1) {
-            a += __shfl_xor_sync(0xffffffffu, a, o);
-            b += __shfl_xor_sync(0xffffffffu, b, o);
-            c += __shfl_xor_sync(0xffffffffu, c, o);
-        }
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    if (wid < 3) {
+        double s = 0.0;
+        for (int i = lane; i < (int)blockDim.x; i += 32) s += red[wid][i];
+        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
         if (lane == 0) {
-            part[blockIdx.x] = a;
-            part[kPartStride + blockIdx.x] = b;
-            part[2 * kPartStride + blockIdx.x] = c;
+            part[wid * kPartStride + blockIdx.x] = s;
+            __threadfence();                              // before the CTA is counted (close_sums3)
         }
     }
 }
@@ -247,8 +237,9 @@ __device__ __forceinline__ void lz_close_step(LzDev* dv, double* hist, double bn
 __device__ __forceinline__ void close_sums3(double* part, int nb, unsigned* done, LzDev* dv, double* hist) {
     __shared__ int last;
     __shared__ double fin[3][32];
+    __syncthreads();                                      // this CTA's partials are stored
     if (threadIdx.x == 0) {
-        __threadfence();                                  // this CTA's partials before its count
+        __threadfence();
         last = atomicInc(done, (unsigned)nb - 1u) == (unsigned)nb - 1u;
     }
     __syncthreads();
@@ -259,19 +250,22 @@ __device__ __forceinline__ void close_sums3(double* part, int nb, unsigned* done
 #pragma unroll
         for (int q = 0; q < 3; ++q) s[q] += __ldcg(part + q * kPartStride + i);
     const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
+    for (int o = 16; o > 0; o >>= 1)
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        for (int o = 16; o > 0; o >>= 1) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-        if (lane == 0) fin[q][wid] = s[q];
-    }
+        for (int q = 0; q < 3; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+    if (lane == 0)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) fin[q][wid] = s[q];
     __syncthreads();
-    if (threadIdx.x != 0) return;
+    if (wid != 0) return;
 #pragma unroll
-    for (int q = 0; q < 3; ++q) {
-        s[q] = fin[q][0];
-        for (int i = 1; i < nw; ++i) s[q] += fin[q][i];
-        part[kRedSlots - 1 - q] = s[q];
-    }
+    for (int q = 0; q < 3; ++q) s[q] = lane < nw ? fin[q][lane] : 0.0;
+    for (int o = 16; o > 0; o >>= 1)
+#pragma unroll
+        for (int q = 0; q < 3; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
+    if (lane != 0) return;
+#pragma unroll
+    for (int q = 0; q < 3; ++q) part[kRedSlots - 1 - q] = s[q];
     if (dv == nullptr) return;
     const double a = s[0], b2 = s[1] - 2.0 * a * a + a * a * s[2];
     const int fused = b2 > 1e-6 * s[1];

@@ -354,7 +354,8 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                                                      const int32_t* __restrict__ npos,
                                                      const uint32_t* __restrict__ list,
                                                      const uint32_t* __restrict__ su,
-                                                     const uint32_t* __restrict__ sd, EpiParams ep,
+                                                     const uint32_t* __restrict__ sd,
+                                                     const __grid_constant__ EpiParams ep,
                                                      int* emax_p, int fixed_emax, unsigned* reset) {
     using IV = typename FxVec<VPL>::T;
     __shared__ long long Bs[33];
@@ -465,7 +466,8 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                                                      const int32_t* __restrict__ npos,
                                                      const uint32_t* __restrict__ list,
                                                      const uint32_t* __restrict__ su,
-                                                     const uint32_t* __restrict__ sd, EpiParams ep,
+                                                     const uint32_t* __restrict__ sd,
+                                                     const __grid_constant__ EpiParams ep,
                                                      const int* __restrict__ emax_p, int fixed_emax,
                                                      const double* __restrict__ fv, double* part,
                                                      unsigned* done, LzDev* dv, double* hist) {
@@ -474,13 +476,13 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
     double s1 = 0.0, s2 = 0.0, s3 = 0.0;
     using IV = typename FxVec<VPL>::T;
     __shared__ long long Bs[33];
+    __shared__ long long sh_bb;
     for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
+    double mbeta = ep.mbeta;
+    if (dv != nullptr) mbeta = -dv->beta;                 // device-resident step: beta_j on the device
+    if (!FAST && threadIdx.x == 0) sh_bb = dv != nullptr ? llround(ldexp(mbeta, ep.m)) : ep.Bbeta;
     __syncthreads();
-    if (dv != nullptr) {                                  // device-resident step: beta_j on the device
-        const double b = dv->beta;
-        ep.mbeta = -b;
-        ep.Bbeta = llround(ldexp(-b, ep.m));
-    }
+    const long long Bbeta = FAST ? 0 : sh_bb;
     const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
     const int k = 1070 - emax;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
@@ -554,7 +556,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                         if (ep.tneg == 0) Pv = -Pv;
                         Pv += ep.Uint * (long long)__popc(su_u & sdc[j]) * fx_join(xo[j].x, xo[j].y);
                         r[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
-                        if (w_old != nullptr) r[j] = fma(ep.mbeta, VPL == 2 ? wpre[j] : w_old[J + j], r[j]);
+                        if (w_old != nullptr) r[j] = fma(mbeta, VPL == 2 ? wpre[j] : w_old[J + j], r[j]);
                     } else {
                         I128 acc{0ull, 0ll};
                         mac_t(acc, fx_join(lo[j], hi[j]) + yv[j], ep);
@@ -562,7 +564,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                         if (w_old != nullptr) {
                             int glo, ghi;
                             fx_split(w_old[J + j], emax, glo, ghi);
-                            mac128(acc, fx_join(glo, ghi), ep.Bbeta);
+                            mac128(acc, fx_join(glo, ghi), Bbeta);
                         }
                         r[j] = i128_to_double(acc, -(k + ep.m));
                     }
@@ -752,11 +754,9 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
     if constexpr (!FAST)
         for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
     double mbeta = ep.mbeta;
-    long long Bbeta = ep.Bbeta;
-    if (STEP && dv != nullptr) {                          // device-resident step: beta_j on the device
-        mbeta = -dv->beta;
-        Bbeta = llround(ldexp(mbeta, ep.m));
-    }
+    if (STEP && dv != nullptr) mbeta = -dv->beta;         // device-resident step: beta_j on the device
+    __shared__ long long sh_bb;                           // synchronised with the staged lists
+    if (STEP && !FAST && threadIdx.x == 0) sh_bb = dv != nullptr ? llround(ldexp(mbeta, ep.m)) : ep.Bbeta;
     const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
     const int k = 1070 - emax;
     const int lane = threadIdx.x & 31;
@@ -843,7 +843,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                 if (STEP && w_old != nullptr) {
                     int glo, ghi;
                     fx_split(wv[j], emax, glo, ghi);
-                    mac128(acc, fx_join(glo, ghi), Bbeta);
+                    mac128(acc, fx_join(glo, ghi), sh_bb);
                 }
                 res[j] = i128_to_double(acc, -(k + ep.m));
             }
