@@ -129,6 +129,16 @@ struct EpiParams {
     int apow;             // A = +-2^apow exactly (t a power of two), or -1
 };
 
+// The int64 epilogue of one element (EpiParams::fast), exact: T the hop sum, xo the
+// own element's words, n the doubly occupied sites; |T| < 2^55, |X| <= 2^48,
+// |Uint n| < 2^14 and tshift <= 6.  The own element's words are multiplied apart
+// (32 x 32 -> 64 bits) and joined once.
+__device__ __forceinline__ long long fast_sum(long long T, int2 xo, int n, const EpiParams& ep) {
+    const int c = (int)ep.Uint * n;
+    const long long t = T << ep.tshift;
+    return (ep.tneg ? t : -t) + (((long long)c * xo.y) << 24) + (long long)c * xo.x;
+}
+
 // acc += A T: a shift where t is a power of two (the same 128-bit value)
 __device__ __forceinline__ void mac_t(I128& acc, long long T, const EpiParams& ep) {
     if (ep.apow >= 0) addshift128(acc, ep.A < 0 ? -T : T, ep.apow);

@@ -366,6 +366,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
     const int k = 1070 - emax;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     constexpr int CC = 32 * VPL;
+    const uint32_t rowb = (uint32_t)Ddn * 8u;             // bytes of a row (Ddn <= kMaxRow)
     const int64_t nchunk = (Ddn + CC - 1) / CC;
     const int64_t nrb = (Dup + rbr - 1) / rbr;
     // item = chunk * nrb + rb, advanced by gridDim.x without division
@@ -383,7 +384,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
         uint32_t sdc[VPL];
 #pragma unroll
         for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
-        const IV* base = reinterpret_cast<const IV*>(X + c);
+        const char* base = reinterpret_cast<const char*>(X + c);
         const int64_t uend = min(rb * rbr + rbr, Dup);
         for (int64_t u = rb * rbr + warp; u < uend; u += nw) {
             const int32_t kb = ptr[u];
@@ -396,7 +397,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
             }
             IV A{};
             uniform_hops<IV, TAIL>(list, kb, ptr[u + 1] - kb, npos[u], lane,
-                [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(reinterpret_cast<const int2*>(base) + (int64_t)t * Ddn)); },
+                [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); },
                 AddFixed<IV>{A});
             if (act) {
                 const uint32_t su_u = su[u];
@@ -429,9 +430,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                 for (int j = 0; j < VPL; ++j) {
                     if constexpr (FAST) {
                         // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
-                        long long Pv = (fx_join(lo[j], hi[j]) + yv[j]) << ep.tshift;
-                        if (ep.tneg == 0) Pv = -Pv;
-                        Pv += ep.Uint * (long long)__popc(su_u & sdc[j]) * fx_join(xo[j].x, xo[j].y);
+                        const long long Pv = fast_sum(fx_join(lo[j], hi[j]) + yv[j], xo[j], __popc(su_u & sdc[j]), ep);
                         r[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
                         if (w_old != nullptr) r[j] = fma(ep.mbeta, w_old[J + j], r[j]);
                     } else {
@@ -504,7 +503,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
         uint32_t sdc[VPL];
 #pragma unroll
         for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
-        const IV* base = reinterpret_cast<const IV*>(X + c);
+        const int2* base = X + c;
         const int64_t uend = min(rb * rbr + rbr, Dup);
         for (int64_t u = rb * rbr + warp; u < uend; u += nw) {
             const int32_t kb = ptr[u];
@@ -527,7 +526,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
             }
             IV A{};
             uniform_hops<IV, true>(list, kb, ptr[u + 1] - kb, npos[u], lane,
-                [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(reinterpret_cast<const int2*>(base) + (int64_t)t * Ddn)); },
+                [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (int64_t)t * Ddn)); },
                 AddFixed<IV>{A});
             if (act) {
                 const uint32_t su_u = su[u];
@@ -551,6 +550,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
 #pragma unroll
                 for (int j = 0; j < VPL; ++j) {
                     if constexpr (FAST) {
+                        // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
                         // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
                         long long Pv = (fx_join(lo[j], hi[j]) + yv[j]) << ep.tshift;
                         if (ep.tneg == 0) Pv = -Pv;
@@ -764,7 +764,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
     const int2* cnt = reinterpret_cast<const int2*>(smem_raw);
     const uint32_t* st = reinterpret_cast<const uint32_t*>(cnt + g.cap);
     const uint32_t* L = st + g.cap;
-    const uint32_t rowb = (uint32_t)Ddn * 8u;             // bytes of a row (Ddn <= 2^28, checked by the launcher)
+    const uint32_t rowb = (uint32_t)Ddn * 8u;             // bytes of a row (Ddn <= kMaxRow)
     double s1 = 0.0, s2 = 0.0, s3 = 0.0;
     up_segments(smem_raw, Dup, (Ddn + CC - 1) / CC, g, ptr, npos, list, su, [&](int64_t r0, int r, int64_t chunk) {
         const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
@@ -818,28 +818,27 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
         double res[VPL];
 #pragma unroll
         for (int j = 0; j < VPL; ++j) {
-            long long T, xo;
+            long long T;
+            int2 xo;
             if constexpr (VPL == 2) {
                 T = j == 0 ? fx_join(A.x, A.y) : fx_join(A.z, A.w);
-                xo = j == 0 ? fx_join(xo4.x, xo4.y) : fx_join(xo4.z, xo4.w);
+                xo = j == 0 ? make_int2(xo4.x, xo4.y) : make_int2(xo4.z, xo4.w);
             } else {
                 T = fx_join(A.x, A.y);
-                xo = fx_join(xo4.x, xo4.y);
+                xo = xo4;
             }
             if constexpr (YS) T += fx_join((int)yv[j], (int)(yv[j] >> 32));
             else T += yv[j];
             const int nd = __popc(su_u & sdc[j]);
             if constexpr (FAST) {
                 // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
-                long long Pv = T << ep.tshift;
-                if (ep.tneg == 0) Pv = -Pv;
-                Pv += ep.Uint * (long long)nd * xo;
+                const long long Pv = fast_sum(T, xo, nd, ep);
                 res[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
                 if (STEP && w_old != nullptr) res[j] = fma(mbeta, wv[j], res[j]);
             } else {
                 I128 acc{0ull, 0ll};
                 mac_t(acc, T, ep);
-                mac128(acc, xo, Bs[nd]);
+                mac128(acc, fx_join(xo.x, xo.y), Bs[nd]);
                 if (STEP && w_old != nullptr) {
                     int glo, ghi;
                     fx_split(wv[j], emax, glo, ghi);
