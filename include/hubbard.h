@@ -181,8 +181,8 @@ int hubbard_apply_reference(hubbard_t H, const void* v, void* w, int dtype, void
  * or 4; binary64 uses at most 2, and a width the row length does not divide
  * is narrowed); ctas_rows: row-phase CTAs per SM (0 = automatic, 1 or 2);
  * ctas_cols: binary64 up phase of a standalone H*v (0 = automatic; 1 = 4 CTAs
- * per SM, epilogue operands loaded after the hop sum; 2 = 3 CTAs per SM, the
- * own element and row-phase sum requested before it).  A choice whose buffers
+ * per SM; 2 = 3 CTAs per SM, the own element and row-phase sum requested before
+ * the hop sum in every kernel).  A choice whose buffers
  * do not fit in shared memory falls back to the largest one that does.
  * Results do not depend on the schedule: every output sums its hops in one
  * fixed order (binary32) or exactly (binary64 fixed point). */

@@ -274,14 +274,6 @@ __device__ __forceinline__ void reset_exponent(int* emax_p, unsigned* counter) {
     if (atomicInc(counter, gridDim.x - 1) == gridDim.x - 1) *emax_p = 0;
 }
 
-// Up phase, binary64 fixed point (Algorithms 2 and 4):
-//   W[u, c] = -t (sum_{(u', s) in hops_up(u)} s X[u', c] + Y[u, c]) + U n(u, c) X[u, c]  [- beta w_old]
-// Row u of W is a signed combination of whole rows u' of X (Eq. H-Kroneckersum),
-// so a warp builds one row segment of CC = 32 * VPL columns with lanes over
-// columns: the hop list is warp-uniform and every access is coalesced.  Work
-// items are (column chunk, block of RB rows); consecutive items share a chunk,
-// which keeps that chunk of X resident in L2 while all rows are combined, and
-// consecutive rows share part of their neighbours (reuse in L1).
 // An item of 16 rows is two per warp; where that leaves fewer items than CTAs
 // that fit on the device, 8 rows (one per warp) spread the sector wider.
 inline int up_rows(int64_t nchunk, int64_t Dup, int ctas) { return nchunk * ((Dup + 15) / 16) < ctas ? 8 : 16; }
@@ -339,15 +331,14 @@ template <typename IV> struct AddFixed {
 // Up phase, binary64 fixed point (Algorithms 2 and 4):
 //   W[u, c] = -t (sum_{(u', s) in hops_up(u)} s X[u', c] + Y[u, c]) + U n(u, c) X[u, c]  [- beta w_old]
 // Row u of W is a signed combination of whole rows u' of X (Eq. H-Kroneckersum),
-// so a warp builds one row segment of CC = 32 * VPL columns with lanes over
-// columns: the hop list is warp-uniform and every access is coalesced.  Work
-// items are (column chunk, block of rbr rows); consecutive items share a
+// so a warp builds one row segment of CC = 64 columns, two per lane (rows of even
+// length), with lanes over columns: the hop list is warp-uniform and every access
+// is coalesced.  Work items are (column chunk, block of rbr rows); consecutive items share a
 // chunk, which keeps that chunk of X resident in L2 while all rows are
 // combined, and consecutive rows share part of their neighbours (L1 reuse).
-// RED: also accumulate <W, fv>, <W, W> and <fv, fv> into part (block_sum3_store).
 // PRE: the epilogue's own element and Y are requested before the gathers (their
 // HBM latency then overlaps the hop sum); CT: CTAs per SM the launch bounds keep
-template <int VPL, bool FAST, bool TAIL, bool PRE = false, int CT = 4>
+template <bool FAST, bool TAIL, bool PRE = false, int CT = 4>
 __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
                                                      int rbr, const int32_t* __restrict__ ptr,
@@ -357,7 +348,8 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
                                                      int* emax_p, int fixed_emax, unsigned* reset) {
-    using IV = typename FxVec<VPL>::T;
+    constexpr int VPL = 2;
+    using IV = int4;
     __shared__ long long Bs[33];
     for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
     __syncthreads();
@@ -390,7 +382,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
             const int32_t kb = ptr[u];
             [[maybe_unused]] int4 t4p;
             [[maybe_unused]] longlong2 y2p;
-            if constexpr (PRE && VPL == 2) {
+            if constexpr (PRE) {
                 const int64_t J = u * Ddn + c;
                 t4p = __ldg(reinterpret_cast<const int4*>(X + J));
                 y2p = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
@@ -405,26 +397,20 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                 int lo[VPL], hi[VPL];
                 int2 xo[VPL];
                 long long yv[VPL];
-                if constexpr (VPL == 2) {
-                    lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
-                    int4 t4;
-                    longlong2 y2;
-                    if constexpr (PRE) {
-                        t4 = t4p;
-                        y2 = y2p;
-                    } else {
-                        t4 = __ldg(reinterpret_cast<const int4*>(X + J));
-                        y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
-                    }
-                    xo[0] = make_int2(t4.x, t4.y);
-                    xo[1] = make_int2(t4.z, t4.w);
-                    yv[0] = y2.x;
-                    yv[1] = y2.y;
+                lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
+                int4 t4;
+                longlong2 y2;
+                if constexpr (PRE) {
+                    t4 = t4p;
+                    y2 = y2p;
                 } else {
-                    lo[0] = A.x; hi[0] = A.y;
-                    xo[0] = __ldg(X + J);
-                    yv[0] = __ldcs(Y + J);
+                    t4 = __ldg(reinterpret_cast<const int4*>(X + J));
+                    y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
                 }
+                xo[0] = make_int2(t4.x, t4.y);
+                xo[1] = make_int2(t4.z, t4.w);
+                yv[0] = y2.x;
+                yv[1] = y2.y;
                 double r[VPL];
 #pragma unroll
                 for (int j = 0; j < VPL; ++j) {
@@ -445,8 +431,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                         r[j] = i128_to_double(acc, -(k + ep.m));
                     }
                 }
-                if constexpr (VPL == 2) __stcs(reinterpret_cast<double2*>(w + J), make_double2(r[0], r[1]));
-                else __stcs(w + J, r[0]);
+                __stcs(reinterpret_cast<double2*>(w + J), make_double2(r[0], r[1]));
             }
         }
     }
@@ -458,7 +443,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
 // <f, f> (block_sum3_store).  Its epilogue streams four arrays (own element,
 // Y, w_old, f), so with 16-byte vectors their loads are issued before the
 // gathers; the extra live registers cost one CTA per SM (3 instead of 4).
-template <int VPL, bool FAST>
+template <bool FAST>
 __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
                                                      int rbr, const int32_t* __restrict__ ptr,
@@ -473,7 +458,8 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
     grid_dep_wait();
     if (dv != nullptr && dv->stall) return;
     double s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    using IV = typename FxVec<VPL>::T;
+    constexpr int VPL = 2;
+    using IV = int4;
     __shared__ long long Bs[33];
     __shared__ long long sh_bb;
     for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
@@ -512,18 +498,17 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
             double wpre[VPL], fpre[VPL];
             int4 t4p;
             longlong2 y2p;
-            if constexpr (VPL == 2) {
-                t4p = __ldg(reinterpret_cast<const int4*>(X + J));
-                y2p = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
-                if (w_old != nullptr) {
-                    const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
-                    wpre[0] = q.x; wpre[1] = q.y;
-                }
-                {
-                    const double2 q = __ldcs(reinterpret_cast<const double2*>(fv + J));
-                    fpre[0] = q.x; fpre[1] = q.y;
-                }
+            t4p = __ldg(reinterpret_cast<const int4*>(X + J));
+            y2p = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+            if (w_old != nullptr) {
+                const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
+                wpre[0] = q.x; wpre[1] = q.y;
             }
+            {
+                const double2 q = __ldcs(reinterpret_cast<const double2*>(fv + J));
+                fpre[0] = q.x; fpre[1] = q.y;
+            }
+
             IV A{};
             uniform_hops<IV, true>(list, kb, ptr[u + 1] - kb, npos[u], lane,
                 [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (int64_t)t * Ddn)); },
@@ -533,19 +518,13 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                 int lo[VPL], hi[VPL];
                 int2 xo[VPL];
                 long long yv[VPL];
-                if constexpr (VPL == 2) {
-                    lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
-                    const int4 t4 = t4p;
-                    xo[0] = make_int2(t4.x, t4.y);
-                    xo[1] = make_int2(t4.z, t4.w);
-                    const longlong2 y2 = y2p;
-                    yv[0] = y2.x;
-                    yv[1] = y2.y;
-                } else {
-                    lo[0] = A.x; hi[0] = A.y;
-                    xo[0] = __ldg(X + J);
-                    yv[0] = __ldcs(Y + J);
-                }
+                lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
+                const int4 t4 = t4p;
+                xo[0] = make_int2(t4.x, t4.y);
+                xo[1] = make_int2(t4.z, t4.w);
+                const longlong2 y2 = y2p;
+                yv[0] = y2.x;
+                yv[1] = y2.y;
                 double r[VPL];
 #pragma unroll
                 for (int j = 0; j < VPL; ++j) {
@@ -556,7 +535,7 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                         if (ep.tneg == 0) Pv = -Pv;
                         Pv += ep.Uint * (long long)__popc(su_u & sdc[j]) * fx_join(xo[j].x, xo[j].y);
                         r[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
-                        if (w_old != nullptr) r[j] = fma(mbeta, VPL == 2 ? wpre[j] : w_old[J + j], r[j]);
+                        if (w_old != nullptr) r[j] = fma(mbeta, wpre[j], r[j]);
                     } else {
                         I128 acc{0ull, 0ll};
                         mac_t(acc, fx_join(lo[j], hi[j]) + yv[j], ep);
@@ -569,16 +548,12 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
                         r[j] = i128_to_double(acc, -(k + ep.m));
                     }
                 }
-                if constexpr (VPL == 2) __stcs(reinterpret_cast<double2*>(w + J), make_double2(r[0], r[1]));
-                else __stcs(w + J, r[0]);
+                __stcs(reinterpret_cast<double2*>(w + J), make_double2(r[0], r[1]));
                 {
                     double fj[VPL];
-                    if constexpr (VPL == 2) {
-                        fj[0] = fpre[0];
-                        fj[1] = fpre[1];
-                    } else {
-                        fj[0] = __ldcs(fv + J);
-                    }
+                    fj[0] = fpre[0];
+                    fj[1] = fpre[1];
+
 #pragma unroll
                     for (int j = 0; j < VPL; ++j) {
                         s1 = fma(r[j], fj[j], s1);
@@ -1300,14 +1275,14 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     launch_on(pdl, K, up_grid, 256, 0, s, Xg, Y, (double*)w, (const double*)w_old, Dup, Ddn, rbr,  \
         up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax
 #define UP64P(F, T)                                                                                         \
-    launch_on(pdl, k_up_f64x<2, F, T, true, 3>, grid_cap(sms() * 3, up_items), 256, 0, s, Xg, Y, (double*)w, \
+    launch_on(pdl, k_up_f64x<F, T, true, 3>, grid_cap(sms() * 3, up_items), 256, 0, s, Xg, Y, (double*)w, \
         (const double*)w_old, Dup, Ddn, rbr, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep,  \
         emax, fixed_emax, reset)
 #define UP64_T(F, T)                                                                                        \
-    if (pre) { UP64P(F, T); } else { UP64((k_up_f64x<2, F, T>)), reset); }
+    if (pre) { UP64P(F, T); } else { UP64((k_up_f64x<F, T>)), reset); }
             if (part != nullptr) {                        // a Lanczos step; a replayed one (w_old alone) goes below
-                if (ep.fast) { UP64((k_up_step_f64x<2, true>)), (const double*)v, part, done, dv, hist); }
-                else { UP64((k_up_step_f64x<2, false>)), (const double*)v, part, done, dv, hist); }
+                if (ep.fast) { UP64((k_up_step_f64x<true>)), (const double*)v, part, done, dv, hist); }
+                else { UP64((k_up_step_f64x<false>)), (const double*)v, part, done, dv, hist); }
             } else if (tail) {
                 if (ep.fast) { UP64_T(true, true) } else { UP64_T(false, true) }
             } else {
