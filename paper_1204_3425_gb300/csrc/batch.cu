@@ -470,7 +470,27 @@ __device__ __forceinline__ void row_pass(const SecView& V, int64_t u, int2* buf,
         const bool act = d < Ddn;
         const int64_t dd = act ? d : Ddn - 1;
         int lo = 0, hi = 0;
-        if (nh <= 32) {
+        if (SWEEP && nh <= 32) {
+            // groups of four requested together; past the list's end the row itself
+            // with factor 0 (taken one by one, two or three of a row's six or seven
+            // neighbours were a memory round each)
+            for (int k = 0; k < nh; k += 4) {
+                int2 x[4];
+                int sg[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const uint32_t e = __shfl_sync(0xffffffffu, mine, k + i);
+                    const bool in = k + i < nh;
+                    sg[i] = in ? 1 - 2 * (int)(e & 1u) : 0;
+                    x[i] = __ldcg(V.X + (in ? (int64_t)(e >> 1) : u) * Ddn + dd);
+                }
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    lo += sg[i] * x[i].x;
+                    hi += sg[i] * x[i].y;
+                }
+            }
+        } else if (nh <= 32) {
 #pragma unroll 4
             for (int k = 0; k < nh; ++k) {
                 const uint32_t e = __shfl_sync(0xffffffffu, mine, k);
