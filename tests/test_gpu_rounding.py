@@ -58,3 +58,39 @@ def test_long_rows_match_the_reference_kernel(nup, ndn, U):
     b = float((r - a * f).norm())
     assert abs(res["alpha"][0] - a) <= 1e-11 * max(1.0, abs(a)) and abs(res["beta"][0] - b) <= 1e-11 * b
     H.close()
+
+
+@pytest.mark.parametrize("lattice,nup,ndn,U", [
+    ("sq4x4", 8, 3, 8.0),      # many rows, several column groups per row range
+    ("sq4x4", 3, 8, 7.3),      # few rows, many chunks
+    ("ring16", 8, 2, 4.0),     # short even rows
+    ("ring16", 1, 8, 4.0),     # 16 rows
+    ("ring13", 6, 5, 2.5),     # odd rows
+    ("ring20", 10, 1, 4.0),    # more rows per range than lists fit at a time
+    ("ring11", 5, 10, 4.0),    # a few columns
+])
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_up_phase_forms_match_the_reference_kernel(lattice, nup, ndn, U, dtype):
+    """Every form of the up phase against one thread per element.  binary64: 1e-12
+    max|v| plus the native kernel's rounding; binary32: 2^-24 per operation on
+    either side, 2 (W + 2) 2^-24 max(1, U N) with W <= 48."""
+    import paper_1204_3425_gb300 as hub
+    from workload import lattice_by_name
+    ns, bonds = lattice_by_name(lattice)
+    H = hub.hubbard_sector_create(ns, bonds, nup, ndn, 1.0, U)
+    g = torch.Generator(device="cuda")
+    g.manual_seed(13)
+    v = torch.rand(H.D, dtype=torch.float64, device="cuda", generator=g) * 2 - 1
+    if dtype == "f32":
+        v = v.float()
+    w, r = torch.empty_like(v), torch.empty_like(v)
+    hub.hubbard_apply_reference(H, v, r)
+    bound = 1.2e-12 if dtype == "f64" else 2 * 50 * 2.0 ** -24 * max(1.0, U * min(nup, ndn))
+    for _ in range(2):                                  # the second product reads an exponent word set back by the first
+        w.fill_(float("nan"))
+        hub.hubbard_apply(H, v, w)
+        assert float((w - r).abs().max()) <= bound
+    small = v * 2.0 ** -20                              # a smaller exponent must not meet the last one's
+    hub.hubbard_apply(H, small, w)
+    assert float((w * 2.0 ** 20 - r).abs().max()) <= bound
+    H.close()
