@@ -177,11 +177,10 @@ __device__ __forceinline__ void sub4(int2& A, int2 a) { A.x -= a.x; A.y -= a.y; 
 
 // Lanczos reductions fused into the up-phase epilogue (Algorithm 1): each
 // thread accumulates <w, f>, <w, w> and <f, f> over its outputs in a fixed
-// order, the CTA sums its threads in a fixed tree, and the per-CTA partials
-// (part[b], part[kPartStride + b], part[2 kPartStride + b]) are summed in
-// index order afterwards, so the result is deterministic.  binary32 outputs
-// use a float-float accumulator (exact product split + TwoSum), as the
-// stand-alone dot kernel does.
+// order, the CTA sums its threads, and the last CTA the per-CTA partials
+// (part[b], part[kPartStride + b], part[2 kPartStride + b]), in fixed trees, so
+// the result is deterministic.  binary32 outputs use a float-float accumulator
+// (exact product split + TwoSum), as the stand-alone dot kernel does.
 struct FFAcc {
     float hi = 0.0f, lo = 0.0f;
     __device__ __forceinline__ void add_product(float x, float y) {
@@ -195,26 +194,39 @@ struct FFAcc {
     __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
 };
 
-// Lanczos reductions fused into the up-phase epilogue (Algorithm 1): the CTA
-// (at most 256 threads) sums its threads' <w, f>, <w, w>, <f, f> in a fixed order
-// and stores the per-CTA partials at part[b], part[kPartStride + b],
-// part[2 kPartStride + b].  One warp takes each sum, column by column over the
-// warps and then across its lanes: 39 FP64 instructions a CTA instead of the 135
-// of shuffles in every warp, which were a quarter of that pipe's work in a ring
-// 12 step.
-__device__ __forceinline__ void block_sum3_store(double a, double b, double c, double* part) {
-    __shared__ double red[3][256];
-    red[0][threadIdx.x] = a;
-    red[1][threadIdx.x] = b;
-    red[2][threadIdx.x] = c;
+// The three sums of a step in one order, whatever forms them: 256 threads a CTA
+// (vt = 0 .. 255), a warp's 32 values by the tree of partners 16, 8, 4, 2, 1
+// apart, the warps' sums by the same tree, and the CTAs' partials (close_sums3)
+// as the 256 threads' were.  a_j and b_{j+1} depend on it in their last bits, and
+// with them everything a long run makes of rounding: the step it stops at, the
+// small components of a Ritz vector and its sign.
+constexpr int kSumPad = 33, kSumSlots = 3 * 32 * 9;
+
+// One warp takes the trees of all eight warps, lane (q, w) those of warp w's sum
+// q: 34 FP64 instructions a CTA where shuffles in every warp took 135, a quarter
+// of that pipe's work in a ring 12 step.  Threads with vt < 0 only synchronise.
+__device__ __forceinline__ void block_sum3_store(double a, double b, double c, double* part, double* red, int vt) {
+    if (vt >= 0) {
+        const int o = (vt >> 5) * kSumPad + (vt & 31);
+        red[o] = a;
+        red[8 * kSumPad + o] = b;
+        red[16 * kSumPad + o] = c;
+    }
     __syncthreads();
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-    if (wid < 3) {
-        double s = 0.0;
-        for (int i = lane; i < (int)blockDim.x; i += 32) s += red[wid][i];
-        for (int o = 16; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
-        if (lane == 0) {
-            part[wid * kPartStride + blockIdx.x] = s;
+    if (threadIdx.x < 32) {
+        const int lane = threadIdx.x, q = lane >> 3;
+        const double* x = red + min(lane, 23) * kSumPad;
+        double t[16];
+#pragma unroll
+        for (int i = 0; i < 16; ++i) t[i] = x[i] + x[i + 16];
+#pragma unroll
+        for (int o = 8; o > 0; o >>= 1)
+#pragma unroll
+            for (int i = 0; i < o; ++i) t[i] += t[i + o];
+        double s = t[0];
+        for (int o = 4; o > 0; o >>= 1) s += __shfl_xor_sync(0xffffffffu, s, o);
+        if ((lane & 7) == 0 && q < 3) {
+            part[q * kPartStride + blockIdx.x] = s;
             __threadfence();                              // before the CTA is counted (close_sums3)
         }
     }
@@ -238,15 +250,14 @@ __device__ __forceinline__ void lz_close_step(LzDev* dv, double* hist, double bn
 
 // Closes a fused reduction inside the kernel that made its partials: the CTA
 // that stores its partials last (done counts the nb CTAs and returns to 0) sums
-// them all in index order into part[kRedSlots-1 .. kRedSlots-3] and, for a
+// them all in the order above into part[kRedSlots-1 .. kRedSlots-3] and, for a
 // device-resident step, forms a_j and, unless the difference
 // <w,w> - 2a^2 + a^2 <f,f> cancels more than six digits, beta_{j+1}.  (When it
 // does, the step stalls: kernels enqueued behind it return at once and the host,
 // which finds the mark in the history, runs the explicit branch.)  A kernel
 // of its own for this took 8-9 us of a 40-70 us step on the small sectors.
-__device__ __forceinline__ void close_sums3(double* part, int nb, unsigned* done, LzDev* dv, double* hist) {
+__device__ __forceinline__ void close_sums3(double* part, int nb, unsigned* done, LzDev* dv, double* hist, double* red) {
     __shared__ int last;
-    __shared__ double fin[3][32];
     __syncthreads();                                      // this CTA's partials are stored
     if (threadIdx.x == 0) {
         __threadfence();
@@ -255,25 +266,31 @@ __device__ __forceinline__ void close_sums3(double* part, int nb, unsigned* done
     __syncthreads();
     if (!last) return;
     __threadfence();
-    double s[3] = {0.0, 0.0, 0.0};
-    for (int i = threadIdx.x; i < nb; i += blockDim.x)
+    // 32 groups of 32 partials (nb <= kPartStride): partners 16 and 8 apart by
+    // the threads that load them, the rest of a group by one lane, then the groups
+    for (int t = threadIdx.x; t < 3 * 32 * 8; t += blockDim.x) {
+        const int q = t >> 8, g = (t >> 3) & 31, i = t & 7;
+        double x[4];
 #pragma unroll
-        for (int q = 0; q < 3; ++q) s[q] += __ldcg(part + q * kPartStride + i);
-    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5, nw = (blockDim.x + 31) >> 5;
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-    if (lane == 0)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) fin[q][wid] = s[q];
+        for (int c = 0; c < 4; ++c) {
+            const int k = 32 * g + i + 8 * c;
+            x[c] = k < nb ? __ldcg(part + q * kPartStride + k) : 0.0;
+        }
+        red[(q * 32 + g) * 9 + i] = 32 * g < nb ? (x[0] + x[2]) + (x[1] + x[3]) : 0.0;
+    }
     __syncthreads();
-    if (wid != 0) return;
-#pragma unroll
-    for (int q = 0; q < 3; ++q) s[q] = lane < nw ? fin[q][lane] : 0.0;
-    for (int o = 16; o > 0; o >>= 1)
-#pragma unroll
-        for (int q = 0; q < 3; ++q) s[q] += __shfl_xor_sync(0xffffffffu, s[q], o);
-    if (lane != 0) return;
+    const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+    __shared__ double fin[3];
+    if (wid < 3) {
+        const double* x = red + (wid * 32 + lane) * 9;
+        double t = 0.0;
+        if (32 * lane < nb) t = ((x[0] + x[4]) + (x[2] + x[6])) + ((x[1] + x[5]) + (x[3] + x[7]));
+        for (int o = 16; o > 0; o >>= 1) t += __shfl_xor_sync(0xffffffffu, t, o);
+        if (lane == 0) fin[wid] = t;
+    }
+    __syncthreads();
+    if (threadIdx.x != 0) return;
+    const double s[3] = {fin[0], fin[1], fin[2]};
 #pragma unroll
     for (int q = 0; q < 3; ++q) part[kRedSlots - 1 - q] = s[q];
     if (dv == nullptr) return;

@@ -283,8 +283,8 @@ inline int up_rows(int64_t nchunk, int64_t Dup, int ctas) { return nchunk * ((Du
 // operand from row t; the operands of a group of four of one sign are requested
 // together, then add(sign, a, b, c, d) or add(sign, a) takes them.  Loop bounds
 // are warp-uniform, so the sign split costs no divergence.
-// TAIL: what is left of a sign after the groups of four is one more group with
-// zeros in place of the missing operands, instead of a memory round each.
+// TAIL: what is left of a sign after the groups of four is requested together,
+// zeros in place of the missing operands, and added one by one as without it.
 template <typename Val, bool TAIL, typename Load, typename Add>
 __device__ __forceinline__ void uniform_hops(const uint32_t* __restrict__ list, int32_t kb, int n, int np, int lane,
                                              Load&& load, Add&& add) {
@@ -307,7 +307,9 @@ __device__ __forceinline__ void uniform_hops(const uint32_t* __restrict__ list, 
                     const uint32_t t1 = __shfl_sync(0xffffffffu, mine, q + 1), t2 = __shfl_sync(0xffffffffu, mine, q + 2);
                     if (q + 1 < end) b = load(t1);
                     if (q + 2 < end) c = load(t2);
-                    add(sign, a, b, c, Val{});
+                    add(sign, a);
+                    add(sign, b);
+                    add(sign, c);
                 }
             } else {
                 for (; q < end; ++q) add(sign, load(__shfl_sync(0xffffffffu, mine, q)));
@@ -317,6 +319,32 @@ __device__ __forceinline__ void uniform_hops(const uint32_t* __restrict__ list, 
         span(std::integral_constant<int, -1>{}, pend, nk);
     }
 }
+
+__device__ __forceinline__ void addf(float& A, float a, float b, float c, float d) { A += (a + b) + (c + d); }
+__device__ __forceinline__ void addf(float& A, float a) { A += a; }
+__device__ __forceinline__ void addf(float2& A, float2 a, float2 b, float2 c, float2 d) {
+    A.x += (a.x + b.x) + (c.x + d.x);
+    A.y += (a.y + b.y) + (c.y + d.y);
+}
+__device__ __forceinline__ void addf(float2& A, float2 a) { A.x += a.x; A.y += a.y; }
+__device__ __forceinline__ void addf(float4& A, float4 a, float4 b, float4 c, float4 d) {
+    A.x += (a.x + b.x) + (c.x + d.x);
+    A.y += (a.y + b.y) + (c.y + d.y);
+    A.z += (a.z + b.z) + (c.z + d.z);
+    A.w += (a.w + b.w) + (c.w + d.w);
+}
+__device__ __forceinline__ void addf(float4& A, float4 a) { A.x += a.x; A.y += a.y; A.z += a.z; A.w += a.w; }
+
+// the binary32 accumulation: the two signs apart, in list order
+template <typename V> struct AddFloat {
+    V& P;
+    V& N;
+    template <typename Sign, typename... Vs>
+    __device__ __forceinline__ void operator()(Sign, Vs... xs) const {
+        if constexpr (Sign::value > 0) addf(P, xs...);
+        else addf(N, xs...);
+    }
+};
 
 // the binary64 accumulation: exact integers, so one accumulator takes both signs
 template <typename IV> struct AddFixed {
@@ -438,30 +466,36 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
     reset_exponent(emax_p, reset);
 }
 
+// Work of the Lanczos step kernels: items of 32 * VPL columns by kUpRows rows,
+// dealt to the CTAs in turn, thread (warp, lane) of a CTA taking rows warp and
+// warp + 8 of an item and columns lane * VPL + j.  The step's sums are over a
+// thread's elements in that order (then block_sum3_store), so this division is
+// part of the result: a schedule may not change it.
+constexpr int kUpRows = 16;
+
 // Lanczos-step variant of k_up_f64x (Algorithm 1 fused with Algorithms 2, 4):
 // W = H f - beta w_old and, per CTA, the partials of <W, f>, <W, W> and
-// <f, f> (block_sum3_store).  Its epilogue streams four arrays (own element,
-// Y, w_old, f), so with 16-byte vectors their loads are issued before the
-// gathers; the extra live registers cost one CTA per SM (3 instead of 4).
-template <bool FAST>
-__global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
-                                                     double* w, const double* w_old, int64_t Dup, int64_t Ddn,
-                                                     int rbr, const int32_t* __restrict__ ptr,
-                                                     const int32_t* __restrict__ npos,
-                                                     const uint32_t* __restrict__ list,
-                                                     const uint32_t* __restrict__ su,
-                                                     const uint32_t* __restrict__ sd,
-                                                     const __grid_constant__ EpiParams ep,
-                                                     const int* __restrict__ emax_p, int fixed_emax,
-                                                     const double* __restrict__ fv, double* part,
-                                                     unsigned* done, LzDev* dv, double* hist) {
+// <f, f>, closed by the last CTA.  Its epilogue streams four arrays (own element,
+// Y, w_old, f), whose loads are issued before the gathers; the extra live
+// registers cost one CTA per SM (3 instead of 4).  YS: Y holds word pairs
+// (k_rows_planes_f64x).
+// NT = 512: a sector of no more items than SMs, one item a CTA and one row a
+// warp; warps 8-15 continue the sums of warps 0-7, in the order above, so a CTA
+// has two rows' memory rounds in flight instead of one after the other (3x3 (4,4)
+// ground state with its vector 2.04 -> 1.92 ms).
+template <int VPL, bool FAST, bool TAIL, bool YS, int NT>
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 3) k_up_step_f64x(
+        const int2* __restrict__ X, const long long* __restrict__ Y, double* w, const double* w_old, int64_t Dup,
+        int64_t Ddn, const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
+        const uint32_t* __restrict__ list, const uint32_t* __restrict__ su, const uint32_t* __restrict__ sd,
+        const __grid_constant__ EpiParams ep, const int* __restrict__ emax_p, int fixed_emax,
+        const double* __restrict__ fv, double* part, unsigned* done, LzDev* dv, double* hist) {
     grid_dep_wait();
     if (dv != nullptr && dv->stall) return;
-    double s1 = 0.0, s2 = 0.0, s3 = 0.0;
-    constexpr int VPL = 2;
-    using IV = int4;
+    using IV = typename FxVec<VPL>::T;
     __shared__ long long Bs[33];
     __shared__ long long sh_bb;
+    __shared__ double red[kSumSlots];
     for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
     double mbeta = ep.mbeta;
     if (dv != nullptr) mbeta = -dv->beta;                 // device-resident step: beta_j on the device
@@ -470,10 +504,21 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
     const long long Bbeta = FAST ? 0 : sh_bb;
     const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
     const int k = 1070 - emax;
-    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
-    constexpr int CC = 32 * VPL;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    constexpr int nw = NT / 32, CC = 32 * VPL;
     const int64_t nchunk = (Ddn + CC - 1) / CC;
-    const int64_t nrb = (Dup + rbr - 1) / rbr;
+    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
+    double s1 = 0.0, s2 = 0.0, s3 = 0.0;
+    double r[VPL], fj[VPL];                               // this thread's elements of a row
+    bool have = false;                                    // NT = 512: r, fj hold its only row
+    auto add_row = [&] {
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) {
+            s1 = fma(r[j], fj[j], s1);
+            s2 = fma(r[j], r[j], s2);
+            s3 = fma(fj[j], fj[j], s3);
+        }
+    };
     // item = chunk * nrb + rb, advanced by gridDim.x without division
     int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
     const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
@@ -490,98 +535,163 @@ __global__ void __launch_bounds__(256, 3) k_up_step_f64x(const int2* __restrict_
 #pragma unroll
         for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
         const int2* base = X + c;
-        const int64_t uend = min(rb * rbr + rbr, Dup);
-        for (int64_t u = rb * rbr + warp; u < uend; u += nw) {
+        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
+        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
             const int32_t kb = ptr[u];
             const int64_t J = u * Ddn + c;
             // streamed operands of the epilogue, requested before the gathers
-            double wpre[VPL], fpre[VPL];
-            int4 t4p;
-            longlong2 y2p;
-            t4p = __ldg(reinterpret_cast<const int4*>(X + J));
-            y2p = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
-            if (w_old != nullptr) {
-                const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
-                wpre[0] = q.x; wpre[1] = q.y;
-            }
-            {
+            double wv[VPL];
+            long long yv[VPL];
+            const IV xo4 = __ldg(reinterpret_cast<const IV*>(X + J));
+            if constexpr (VPL == 2) {
+                const longlong2 y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+                yv[0] = y2.x; yv[1] = y2.y;
+                if (w_old != nullptr) {
+                    const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
+                    wv[0] = q.x; wv[1] = q.y;
+                }
                 const double2 q = __ldcs(reinterpret_cast<const double2*>(fv + J));
-                fpre[0] = q.x; fpre[1] = q.y;
+                fj[0] = q.x; fj[1] = q.y;
+            } else {
+                yv[0] = __ldcs(Y + J);
+                if (w_old != nullptr) wv[0] = __ldcs(w_old + J);
+                fj[0] = __ldcs(fv + J);
             }
-
             IV A{};
-            uniform_hops<IV, true>(list, kb, ptr[u + 1] - kb, npos[u], lane,
+            uniform_hops<IV, TAIL>(list, kb, ptr[u + 1] - kb, npos[u], lane,
                 [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (int64_t)t * Ddn)); },
                 AddFixed<IV>{A});
-            if (act) {
-                const uint32_t su_u = su[u];
-                int lo[VPL], hi[VPL];
-                int2 xo[VPL];
-                long long yv[VPL];
-                lo[0] = A.x; hi[0] = A.y; lo[1] = A.z; hi[1] = A.w;
-                const int4 t4 = t4p;
-                xo[0] = make_int2(t4.x, t4.y);
-                xo[1] = make_int2(t4.z, t4.w);
-                const longlong2 y2 = y2p;
-                yv[0] = y2.x;
-                yv[1] = y2.y;
-                double r[VPL];
+            if (!act) continue;
+            const uint32_t su_u = su[u];
 #pragma unroll
-                for (int j = 0; j < VPL; ++j) {
-                    if constexpr (FAST) {
-                        // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
-                        // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
-                        long long Pv = (fx_join(lo[j], hi[j]) + yv[j]) << ep.tshift;
-                        if (ep.tneg == 0) Pv = -Pv;
-                        Pv += ep.Uint * (long long)__popc(su_u & sdc[j]) * fx_join(xo[j].x, xo[j].y);
-                        r[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
-                        if (w_old != nullptr) r[j] = fma(mbeta, wpre[j], r[j]);
-                    } else {
-                        I128 acc{0ull, 0ll};
-                        mac_t(acc, fx_join(lo[j], hi[j]) + yv[j], ep);
-                        mac128(acc, fx_join(xo[j].x, xo[j].y), Bs[__popc(su_u & sdc[j])]);
-                        if (w_old != nullptr) {
-                            int glo, ghi;
-                            fx_split(w_old[J + j], emax, glo, ghi);
-                            mac128(acc, fx_join(glo, ghi), Bbeta);
-                        }
-                        r[j] = i128_to_double(acc, -(k + ep.m));
-                    }
+            for (int j = 0; j < VPL; ++j) {
+                long long T;
+                int2 xo;
+                if constexpr (VPL == 2) {
+                    T = j == 0 ? fx_join(A.x, A.y) : fx_join(A.z, A.w);
+                    xo = j == 0 ? make_int2(xo4.x, xo4.y) : make_int2(xo4.z, xo4.w);
+                } else {
+                    T = fx_join(A.x, A.y);
+                    xo = xo4;
                 }
-                __stcs(reinterpret_cast<double2*>(w + J), make_double2(r[0], r[1]));
-                {
-                    double fj[VPL];
-                    fj[0] = fpre[0];
-                    fj[1] = fpre[1];
+                if constexpr (YS) T += fx_join((int)yv[j], (int)(yv[j] >> 32));
+                else T += yv[j];
+                const int nd = __popc(su_u & sdc[j]);
+                if constexpr (FAST) {
+                    r[j] = i64_scaled_to_double(fast_sum(T, xo, nd, ep), -(k + ep.ju));
+                    if (w_old != nullptr) r[j] = fma(mbeta, wv[j], r[j]);
+                } else {
+                    I128 acc{0ull, 0ll};
+                    mac_t(acc, T, ep);
+                    mac128(acc, fx_join(xo.x, xo.y), Bs[nd]);
+                    if (w_old != nullptr) {
+                        int glo, ghi;
+                        fx_split(wv[j], emax, glo, ghi);
+                        mac128(acc, fx_join(glo, ghi), Bbeta);
+                    }
+                    r[j] = i128_to_double(acc, -(k + ep.m));
+                }
+            }
+            if constexpr (VPL == 2) __stcs(reinterpret_cast<double2*>(w + J), make_double2(r[0], r[1]));
+            else __stcs(w + J, r[0]);
+            if constexpr (NT == 512) have = true;
+            else add_row();
+        }
+    }
+    if constexpr (NT == 512) {
+        __shared__ double car[3][256];
+        const int t = threadIdx.x & 255;
+        if (warp < 8) {
+            if (have) add_row();
+            car[0][t] = s1;
+            car[1][t] = s2;
+            car[2][t] = s3;
+        }
+        __syncthreads();
+        if (warp >= 8) {
+            s1 = car[0][t];
+            s2 = car[1][t];
+            s3 = car[2][t];
+            if (have) add_row();
+        }
+    }
+    block_sum3_store(s1, s2, s3, part, red, (int)threadIdx.x - (NT - 256));
+    close_sums3(part, gridDim.x, done, dv, hist, red);
+}
 
+// Lanczos-step variant of the binary32 up phase, items and sums as above.  What is
+// left of a hop list is requested at once on every size (4x4 (8,8) step 2.75 ->
+// 2.62 ms, ring 14 (7,7) 162 -> 146 us).
+template <int VPL>
+__global__ void __launch_bounds__(256, 4) k_up_step_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
+                                                        const float* w_old, int64_t Dup, int64_t Ddn,
+                                                        const int32_t* __restrict__ ptr,
+                                                        const int32_t* __restrict__ npos,
+                                                        const uint32_t* __restrict__ list,
+                                                        const uint32_t* __restrict__ su,
+                                                        const uint32_t* __restrict__ sd, float mt, float U, float mbeta,
+                                                        double* part, unsigned* done, LzDev* dv, double* hist) {
+    grid_dep_wait();
+    if (dv != nullptr && dv->stall) return;
+    __shared__ double red[kSumSlots];
+    FFAcc s1, s2, s3;
+    if (dv != nullptr) mbeta = (float)-dv->beta;          // device-resident step: beta_j on the device
+    using V = typename F32Vec<VPL>::T;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    constexpr int CC = 32 * VPL;
+    const int64_t nchunk = (Ddn + CC - 1) / CC;
+    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
+    int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
+    const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
+    for (; chunk < nchunk; chunk += dch, rb += drb) {
+        if (rb >= nrb) {
+            rb -= nrb;
+            ++chunk;
+            if (chunk >= nchunk) break;
+        }
+        const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
+        const bool act = c_raw < Ddn;
+        const int64_t c = act ? c_raw : Ddn - VPL;
+        uint32_t sdc[VPL];
 #pragma unroll
-                    for (int j = 0; j < VPL; ++j) {
-                        s1 = fma(r[j], fj[j], s1);
-                        s2 = fma(r[j], r[j], s2);
-                        s3 = fma(fj[j], fj[j], s3);
-                    }
-                }
+        for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
+        const float* base = v + c;
+        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
+        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
+            const int32_t kb = ptr[u];
+            const int64_t J = u * Ddn + c;
+            // epilogue operands, requested before the gathers
+            const V xo = __ldg(reinterpret_cast<const V*>(v + J));
+            const V yv = __ldcs(reinterpret_cast<const V*>(Y + J));
+            V wv{};
+            if (w_old != nullptr) wv = __ldcs(reinterpret_cast<const V*>(w_old + J));
+            V P{}, N{};
+            uniform_hops<V, true>(list, kb, ptr[u + 1] - kb, npos[u], lane,
+                [&](uint32_t t) { return __ldg(reinterpret_cast<const V*>(base + (int64_t)t * Ddn)); },
+                AddFloat<V>{P, N});
+            if (!act) continue;
+            const uint32_t su_u = su[u];
+            float r[VPL];
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                const float nd = (float)__popc(su_u & sdc[j]);
+                r[j] = fmaf(mt, (comp(P, j) - comp(N, j)) + comp(yv, j), U * nd * comp(xo, j));
+                if (w_old != nullptr) r[j] = fmaf(mbeta, comp(wv, j), r[j]);
+            }
+            if constexpr (VPL == 4) __stcs(reinterpret_cast<float4*>(w + J), make_float4(r[0], r[1], r[2], r[3]));
+            else if constexpr (VPL == 2) __stcs(reinterpret_cast<float2*>(w + J), make_float2(r[0], r[1]));
+            else __stcs(w + J, r[0]);
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                s1.add_product(r[j], comp(xo, j));
+                s2.add_product(r[j], r[j]);
+                s3.add_product(comp(xo, j), comp(xo, j));
             }
         }
     }
-    block_sum3_store(s1, s2, s3, part);
-    close_sums3(part, gridDim.x, done, dv, hist);
+    block_sum3_store(s1.value(), s2.value(), s3.value(), part, red, threadIdx.x);
+    close_sums3(part, gridDim.x, done, dv, hist, red);
 }
-
-__device__ __forceinline__ void addf(float& A, float a, float b, float c, float d) { A += (a + b) + (c + d); }
-__device__ __forceinline__ void addf(float& A, float a) { A += a; }
-__device__ __forceinline__ void addf(float2& A, float2 a, float2 b, float2 c, float2 d) {
-    A.x += (a.x + b.x) + (c.x + d.x);
-    A.y += (a.y + b.y) + (c.y + d.y);
-}
-__device__ __forceinline__ void addf(float2& A, float2 a) { A.x += a.x; A.y += a.y; }
-__device__ __forceinline__ void addf(float4& A, float4 a, float4 b, float4 c, float4 d) {
-    A.x += (a.x + b.x) + (c.x + d.x);
-    A.y += (a.y + b.y) + (c.y + d.y);
-    A.z += (a.z + b.z) + (c.z + d.z);
-    A.w += (a.w + b.w) + (c.w + d.w);
-}
-__device__ __forceinline__ void addf(float4& A, float4 a) { A.x += a.x; A.y += a.y; A.z += a.z; A.w += a.w; }
 
 // Up phase with resident rows: a warp builds one row segment of 32 * VPL * NV
 // columns with lanes over columns, as above, but the rows belong to the CTA.
@@ -626,17 +736,21 @@ __device__ __forceinline__ void stage_up_lists(unsigned char* smem, int cap, int
     }
 }
 
-// Sums over a staged hop list, +1 targets then -1 targets: add(neg, entries, k)
-// sees groups of four, the last of each sign with k < 4 valid ones, so that the
+// Sums over a staged hop list in the order of uniform_hops: windows of 32 entries,
+// in each the +1 targets and then the -1 targets.  add(neg, entries, k) sees
+// groups of four, then what is left of the sign as one group of k < 4, so that the
 // loads of a group are always requested together (a rest taken one by one is a
 // memory latency for each of its entries).
 template <typename Add>
 __device__ __forceinline__ void list_hops(const uint32_t* L, int np, int n, Add&& add) {
-    int q = 0;
-    for (; q + 4 <= np; q += 4) add(false, L + q, std::integral_constant<int, 4>{}, 4);
-    if (q < np) add(false, L + q, std::integral_constant<int, 0>{}, np - q);
-    for (q = np; q + 4 <= n; q += 4) add(true, L + q, std::integral_constant<int, 4>{}, 4);
-    if (q < n) add(true, L + q, std::integral_constant<int, 0>{}, n - q);
+    for (int k0 = 0; k0 < n; k0 += 32) {
+        const int end = min(k0 + 32, n), pend = max(k0, min(end, np));
+        int q = k0;
+        for (; q + 4 <= pend; q += 4) add(false, L + q, std::integral_constant<int, 4>{}, 4);
+        if (q < pend) add(false, L + q, std::integral_constant<int, 0>{}, pend - q);
+        for (q = pend; q + 4 <= end; q += 4) add(true, L + q, std::integral_constant<int, 4>{}, 4);
+        if (q < end) add(true, L + q, std::integral_constant<int, 0>{}, end - q);
+    }
 }
 
 // Cost of a row's segment in units of one hop, besides its hops.
@@ -706,10 +820,10 @@ __device__ __forceinline__ void up_segments(unsigned char* smem, int64_t Dup, in
         }
 }
 
-// Binary64 fixed point, resident rows.  STEP: the Lanczos step, W = H f - beta w_old with, per
-// CTA, the partials of <W, f>, <W, W> and <f, f> (block_sum3_store).  CT: CTAs
-// per SM the launch bounds keep.  YS: Y holds word pairs (k_rows_planes_f64x).
-template <int VPL, bool FAST, bool STEP, bool YS, int CT>
+// Binary64 fixed point, resident rows.  OLD: a replayed Lanczos step, W = H f -
+// beta w_old.  CT: CTAs per SM the launch bounds keep.  YS: Y holds word pairs
+// (k_rows_planes_f64x).
+template <int VPL, bool FAST, bool OLD, bool YS, int CT>
 __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
                                                      UpGrid g, const int32_t* __restrict__ ptr,
@@ -718,20 +832,13 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
-                                                     int* emax_p, int fixed_emax, unsigned* reset,
-                                                     const double* __restrict__ fv, double* part,
-                                                     unsigned* done, LzDev* dv, double* hist) {
+                                                     int* emax_p, int fixed_emax, unsigned* reset) {
     grid_dep_wait();
-    if (STEP && dv != nullptr && dv->stall) return;
     using IV = typename FxVec<VPL>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     __shared__ long long Bs[33];
     if constexpr (!FAST)
         for (int i = threadIdx.x; i < 33; i += blockDim.x) Bs[i] = i < ep.nB ? ep.B[i] : 0;
-    double mbeta = ep.mbeta;
-    if (STEP && dv != nullptr) mbeta = -dv->beta;         // device-resident step: beta_j on the device
-    __shared__ long long sh_bb;                           // synchronised with the staged lists
-    if (STEP && !FAST && threadIdx.x == 0) sh_bb = dv != nullptr ? llround(ldexp(mbeta, ep.m)) : ep.Bbeta;
     const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
     const int k = 1070 - emax;
     const int lane = threadIdx.x & 31;
@@ -740,7 +847,6 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
     const uint32_t* st = reinterpret_cast<const uint32_t*>(cnt + g.cap);
     const uint32_t* L = st + g.cap;
     const uint32_t rowb = (uint32_t)Ddn * 8u;             // bytes of a row (Ddn <= kMaxRow)
-    double s1 = 0.0, s2 = 0.0, s3 = 0.0;
     up_segments(smem_raw, Dup, (Ddn + CC - 1) / CC, g, ptr, npos, list, su, [&](int64_t r0, int r, int64_t chunk) {
         const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
         const bool act = c_raw < Ddn;
@@ -751,28 +857,20 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
         // epilogue operands, requested with the gathers
         const IV xo4 = __ldg(reinterpret_cast<const IV*>(X + J));
         long long yv[VPL];
-        double wv[VPL], fj[VPL];
+        double wv[VPL];
         uint32_t sdc[VPL];
         if constexpr (VPL == 2) {
             const longlong2 y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
             yv[0] = y2.x;
             yv[1] = y2.y;
-            if (STEP) {
-                if (w_old != nullptr) {
-                    const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
-                    wv[0] = q.x;
-                    wv[1] = q.y;
-                }
-                if (part != nullptr) {
-                    const double2 q = __ldcs(reinterpret_cast<const double2*>(fv + J));
-                    fj[0] = q.x;
-                    fj[1] = q.y;
-                }
+            if constexpr (OLD) {
+                const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
+                wv[0] = q.x;
+                wv[1] = q.y;
             }
         } else {
             yv[0] = __ldcs(Y + J);
-            if (STEP && w_old != nullptr) wv[0] = __ldcs(w_old + J);
-            if (STEP && part != nullptr) fj[0] = __ldcs(fv + J);
+            if constexpr (OLD) wv[0] = __ldcs(w_old + J);
         }
         IV A{};
         const int2 np = cnt[r];
@@ -809,52 +907,36 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                 // exact: |T| < 2^55, |X| <= 2^48, |Uint * n| < 2^14 and tshift <= 6
                 const long long Pv = fast_sum(T, xo, nd, ep);
                 res[j] = i64_scaled_to_double(Pv, -(k + ep.ju));
-                if (STEP && w_old != nullptr) res[j] = fma(mbeta, wv[j], res[j]);
+                if constexpr (OLD) res[j] = fma(ep.mbeta, wv[j], res[j]);
             } else {
                 I128 acc{0ull, 0ll};
                 mac_t(acc, T, ep);
                 mac128(acc, fx_join(xo.x, xo.y), Bs[nd]);
-                if (STEP && w_old != nullptr) {
+                if constexpr (OLD) {
                     int glo, ghi;
                     fx_split(wv[j], emax, glo, ghi);
-                    mac128(acc, fx_join(glo, ghi), sh_bb);
+                    mac128(acc, fx_join(glo, ghi), ep.Bbeta);
                 }
                 res[j] = i128_to_double(acc, -(k + ep.m));
             }
         }
         if constexpr (VPL == 2) __stcs(reinterpret_cast<double2*>(w + J), make_double2(res[0], res[1]));
         else __stcs(w + J, res[0]);
-        if (STEP && part != nullptr) {
-#pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                s1 = fma(res[j], fj[j], s1);
-                s2 = fma(res[j], res[j], s2);
-                s3 = fma(fj[j], fj[j], s3);
-            }
-        }
     });
-    if (STEP && part != nullptr) {
-        block_sum3_store(s1, s2, s3, part);
-        close_sums3(part, gridDim.x, done, dv, hist);
-    }
-    if (!STEP) reset_exponent(emax_p, reset);
+    reset_exponent(emax_p, reset);
 }
 
 // Binary32: same decomposition, float arithmetic.  NV vectors of VPL columns
 // per lane, 32 * VPL columns apart, so rows whose length only allows narrow
 // vectors still keep as many bytes in flight.
-template <int VPL, int NV, bool RED>
+template <int VPL, int NV>
 __global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
                                                    const float* w_old, int64_t Dup, int64_t Ddn, UpGrid g,
                                                    const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
                                                    const uint32_t* __restrict__ list, const uint32_t* __restrict__ su,
-                                                   const uint32_t* __restrict__ sd, float mt, float U, float mbeta,
-                                                   double* part, unsigned* done, LzDev* dv, double* hist) {
+                                                   const uint32_t* __restrict__ sd, float mt, float U, float mbeta) {
     extern __shared__ __align__(16) unsigned char smem_raw[];
     grid_dep_wait();
-    if (dv != nullptr && dv->stall) return;
-    FFAcc s1, s2, s3;
-    if (dv != nullptr) mbeta = (float)-dv->beta;          // device-resident step: beta_j on the device
     using V = typename F32Vec<VPL>::T;
     const int lane = threadIdx.x & 31;
     constexpr int CC = 32 * VPL * NV;
@@ -893,8 +975,14 @@ __global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, 
                 }
 #pragma unroll
             for (int i = 0; i < NV; ++i) {
-                if (neg) addf(N[i], x[i][0], x[i][1], x[i][2], x[i][3]);
-                else addf(P[i], x[i][0], x[i][1], x[i][2], x[i][3]);
+                V& A = neg ? N[i] : P[i];
+                if constexpr (full.value == 4) {
+                    addf(A, x[i][0], x[i][1], x[i][2], x[i][3]);
+                } else {
+                    addf(A, x[i][0]);
+                    addf(A, x[i][1]);
+                    addf(A, x[i][2]);
+                }
             }
         });
         const uint32_t su_u = st[r];
@@ -912,20 +1000,8 @@ __global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, 
             if constexpr (VPL == 4) __stcs(reinterpret_cast<float4*>(w + J), make_float4(res[0], res[1], res[2], res[3]));
             else if constexpr (VPL == 2) __stcs(reinterpret_cast<float2*>(w + J), make_float2(res[0], res[1]));
             else __stcs(w + J, res[0]);
-            if constexpr (RED) {
-#pragma unroll
-                for (int j = 0; j < VPL; ++j) {
-                    s1.add_product(res[j], comp(xo[i], j));
-                    s2.add_product(res[j], res[j]);
-                    s3.add_product(comp(xo[i], j), comp(xo[i], j));
-                }
-            }
         }
     });
-    if constexpr (RED) {
-        block_sum3_store(s1.value(), s2.value(), s3.value(), part);
-        close_sums3(part, gridDim.x, done, dv, hist);
-    }
 }
 
 // ---------------------------------------------------------------------------
@@ -1082,16 +1158,17 @@ void allow_smem() {
     (void)once;
 }
 
-// Which binary64 up phase takes a sector with rows of even length (odd ones
-// always take the resident-row kernel):
+// Which binary64 up phase forms a product or a replayed step of a sector with rows
+// of even length (odd ones always take the resident-row kernel):
 //   up to kUpSmall elements: work items dealt over all CTAs -- a CTA has one or
-//     two, and staging lists would only lengthen its chain (ring 12 (6,6) step
-//     52.8 us, 57.2 with resident rows; ring 14 (7,7) 322 against 320);
-//   above: resident rows (4x4 (5,5) product 414 -> 376 us, step 600 -> 524 us;
-//     4x4 (8,8) step 5.35 -> 5.24 ms), except
+//     two, and staging lists would only lengthen its chain;
+//   above: resident rows (4x4 (5,5) product 414 -> 376 us), except
 //   standalone products of more than kUpHbm bytes a vector (4x4 (8,8) 3.80 ms
 //     with items, 4.11 with resident rows; 4x4 (7,7) 2.87, 2.95; ring 16 (6,6),
 //     513 MB: 1.10, 1.05).
+// A Lanczos step has items of one shape at every size (kUpRows).  On more than
+// kUpSmall elements its kernel and the item product take the rest of a hop list
+// one by one (4x4 (8,8) product 3.80 ms, 4.49 with padded groups).
 constexpr int64_t kUpSmall = 2500000, kUpHbm = 600ll << 20;
 // Kernels of a sector start while the one before drains (launch_on) when its
 // vectors stay in L2 (ring 12 product 29.9 -> 26.1 us, step 55.9 -> 44.3 us); on
@@ -1102,6 +1179,11 @@ constexpr int64_t kPdlBytes = 100ll << 20;
 // (ring 8 (4,4) product: two kernels instead of a memset and three)
 constexpr int64_t kScanElems = 16384;
 constexpr int64_t kMaxRow = (1ll << 29) - 1;       // row pitch in bytes held in 32 bits
+
+// items of a Lanczos step's up phase (k_up_step_f64x, k_up_step_f32)
+int64_t up_step_items(int vpl, int64_t Dup, int64_t Ddn) {
+    return (Ddn + 32 * vpl - 1) / (32 * vpl) * ((Dup + kUpRows - 1) / kUpRows);
+}
 
 // a grid of at most `full` CTAs and no more than the work items
 int grid_cap(int full, int64_t items) { return (int)std::max<int64_t>(1, std::min<int64_t>(full, items)); }
@@ -1236,20 +1318,38 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         const EpiParams ep = make_epilogue(H->t, H->U, H->ns, w_old ? beta : 0.0, H->host[0].W + H->host[1].W);
         // columns per lane in the up phase: 2 when Ddn is even (16-byte loads)
         const int vpl = ((Ddn & 1) == 0 && H->vec_cols != 1) ? 2 : 1;
-        const bool step = part != nullptr || w_old != nullptr;
         unsigned* reset = self_reset ? done : nullptr;
+        const bool tail = H->D <= kUpSmall;
         int up_grid = 0;
-        if (vpl == 1 || ysplit || (H->D > kUpSmall && (step || H->D * 8 <= kUpHbm))) {
-            const bool three = step || (H->ctas_cols == 2 && !ysplit);
+        if (part != nullptr) {                            // a Lanczos step
+            const int64_t items = up_step_items(vpl, Dup, Ddn);
+            up_grid = grid_cap(sms() * 3, items);
+#define UPS64(V, F, T, YS, NT)                                                                              \
+    launch_on(pdl, k_up_step_f64x<V, F, T, YS, NT>, up_grid, NT, 0, s, Xg, Y, (double*)w, (const double*)w_old, Dup, \
+        Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax, (const double*)v, part, \
+        done, dv, hist)
+#define UPS64_T(V, F)                                                                                      \
+    if (ysplit) { if (tail) { UPS64(V, F, true, true, 256); } else { UPS64(V, F, false, true, 256); } }    \
+    else if (items <= sms()) { UPS64(V, F, true, false, 512); }                                            \
+    else if (tail) { UPS64(V, F, true, false, 256); }                                                      \
+    else { UPS64(V, F, false, false, 256); }
+            if (vpl == 2) {
+                if (ep.fast) { UPS64_T(2, true) } else { UPS64_T(2, false) }
+            } else {
+                if (ep.fast) { UPS64_T(1, true) } else { UPS64_T(1, false) }
+            }
+#undef UPS64_T
+#undef UPS64
+        } else if (vpl == 1 || ysplit || (H->D > kUpSmall && (w_old != nullptr || H->D * 8 <= kUpHbm))) {
+            const bool three = w_old != nullptr || (H->ctas_cols == 2 && !ysplit);
             const UpGrid g = up_grid_for(H, (Ddn + 32 * vpl - 1) / (32 * vpl), sms() * (three ? 3 : 4));
-            up_grid = g.gx * g.gy;
-#define UPR64(V, F, ST, YS, CT)                                                                             \
-    launch_on(pdl, k_upr_f64x<V, F, ST, YS, CT>, up_grid, 256, g.smem, s, Xg, Y, (double*)w, (const double*)w_old, Dup, \
-        Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax, reset, (const double*)v, \
-        part, done, dv, hist)
+#define UPR64(V, F, OLD, YS, CT)                                                                            \
+    launch_on(pdl, k_upr_f64x<V, F, OLD, YS, CT>, g.gx * g.gy, 256, g.smem, s, Xg, Y, (double*)w,              \
+        (const double*)w_old, Dup, Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax,  \
+        fixed_emax, reset)
 #define UPR64_S(V, F)                                                                                      \
-    if (ysplit) { if (step) { UPR64(V, F, true, true, 3); } else { UPR64(V, F, false, true, 4); } }        \
-    else if (step) { UPR64(V, F, true, false, 3); }                                                        \
+    if (ysplit) { if (three) { UPR64(V, F, true, true, 3); } else { UPR64(V, F, false, true, 4); } }       \
+    else if (w_old != nullptr) { UPR64(V, F, true, false, 3); }                                            \
     else if (three) { UPR64(V, F, false, false, 3); }                                                      \
     else { UPR64(V, F, false, false, 4); }
             if (vpl == 2) {
@@ -1261,35 +1361,25 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #undef UPR64
         } else {
             const int64_t up_chunks = (Ddn + 63) / 64;
-            const int up_full = sms() * (part != nullptr ? 3 : 4);
-            const int rbr = up_rows(up_chunks, Dup, up_full);
+            const int rbr = up_rows(up_chunks, Dup, sms() * 4);
             const int64_t up_items = up_chunks * ((Dup + rbr - 1) / rbr);
-            up_grid = grid_cap(up_full, up_items);
             // standalone: request the epilogue's own element and Y before the
             // gathers (at 3 CTAs/SM for the registers) where that measured faster --
             // the 128-bit epilogue and rows staged from global memory -- unless the
             // schedule fixes it (ctas_cols 1: no, 2: yes)
             const bool pre = H->ctas_cols == 2 || (H->ctas_cols == 0 && (!ep.fast || va == 0));
-            const bool tail = H->D <= kUpSmall;
-#define UP64(K)                                                                                             \
-    launch_on(pdl, K, up_grid, 256, 0, s, Xg, Y, (double*)w, (const double*)w_old, Dup, Ddn, rbr,  \
-        up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax
-#define UP64P(F, T)                                                                                         \
-    launch_on(pdl, k_up_f64x<F, T, true, 3>, grid_cap(sms() * 3, up_items), 256, 0, s, Xg, Y, (double*)w, \
+#define UP64(CT, ...)                                                                                       \
+    launch_on(pdl, k_up_f64x<__VA_ARGS__>, grid_cap(sms() * CT, up_items), 256, 0, s, Xg, Y, (double*)w,       \
         (const double*)w_old, Dup, Ddn, rbr, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep,  \
         emax, fixed_emax, reset)
 #define UP64_T(F, T)                                                                                        \
-    if (pre) { UP64P(F, T); } else { UP64((k_up_f64x<F, T>)), reset); }
-            if (part != nullptr) {                        // a Lanczos step; a replayed one (w_old alone) goes below
-                if (ep.fast) { UP64((k_up_step_f64x<true>)), (const double*)v, part, done, dv, hist); }
-                else { UP64((k_up_step_f64x<false>)), (const double*)v, part, done, dv, hist); }
-            } else if (tail) {
+    if (pre) { UP64(3, F, T, true, 3); } else { UP64(4, F, T); }
+            if (tail) {
                 if (ep.fast) { UP64_T(true, true) } else { UP64_T(false, true) }
             } else {
                 if (ep.fast) { UP64_T(true, false) } else { UP64_T(false, false) }
             }
 #undef UP64_T
-#undef UP64P
 #undef UP64
         }
         if (part != nullptr && nparts != nullptr) *nparts = up_grid;
@@ -1320,16 +1410,25 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #undef ROWS32
 #undef ROWS32_U
     int up_grid = 0;
+    if (part != nullptr) {                                // a Lanczos step
+        up_grid = grid_cap(sms() * 4, up_step_items(vpl, Dup, Ddn));
+#define UPS32(V)                                                                                           \
+    launch_on(pdl, k_up_step_f32<V>, up_grid, 256, 0, s, (const float*)v, Y, (float*)w, (const float*)w_old, Dup, \
+        Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U, (float)-beta, \
+        part, done, dv, hist)
+        if (vpl == 4) { UPS32(4); } else if (vpl == 2) { UPS32(2); } else { UPS32(1); }
+#undef UPS32
+    } else {
 #define UP32(V, NV)                                                                                        \
     {                                                                                                      \
         const UpGrid g = up_grid_for(H, (Ddn + 32 * V * NV - 1) / (32 * V * NV), sms() * 4);               \
-        up_grid = g.gx * g.gy;                                                                             \
-        launch_on(pdl, part != nullptr ? k_up_f32<V, NV, true> : k_up_f32<V, NV, false>, up_grid, 256, g.smem, s, \
-            (const float*)v, Y, (float*)w, (const float*)w_old, Dup, Ddn, g, up.pn_ptr, up.pn_npos,         \
-            up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U, (float)-beta, part, done, dv, hist); \
+        launch_on(pdl, k_up_f32<V, NV>, g.gx * g.gy, 256, g.smem, s, (const float*)v, Y, (float*)w,         \
+            (const float*)w_old, Dup, Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states,      \
+            (float)-H->t, (float)H->U, (float)-beta);                                                      \
     }
-    if (vpl == 4) { UP32(4, 1) } else if (vpl == 2) { UP32(2, 2) } else { UP32(1, 2) }
+        if (vpl == 4) { UP32(4, 1) } else if (vpl == 2) { UP32(2, 2) } else { UP32(1, 2) }
 #undef UP32
+    }
     if (part != nullptr && nparts != nullptr) *nparts = up_grid;
     HUB_CUDA(cudaGetLastError());
     count_launches(2);
