@@ -1276,7 +1276,7 @@ static int ritz_vector(hubbard_t H, const void* v0, int v0_dtype, int dtype, con
         if (dtype == HUB_F64)
             rc = launch_psi_multi_f64((const double*)store, (int64_t)(stride / 8), k, sv.data(), H->red, psi, H->D, s);
         else
-            rc = launch_psi_multi((const float*)store, (int64_t)(stride / 4), k, sv.data(), H->red, psi, H->D, k == m, s);
+            rc = launch_psi_multi((const float*)store, (int64_t)(stride / 4), k, sv.data(), H->red, psi, H->D, s);
         if (rc) return rc;
     }
     if (k < m) {
@@ -1310,7 +1310,6 @@ static int ritz_vector(hubbard_t H, const void* v0, int v0_dtype, int dtype, con
             if ((rc = launch_axpy_scale(ru.a, ru.inv, ru.fo, f, H->D, dtype, s))) return rc;
             if ((rc = psi_accumulate(f, dtype, psi, H->D, sv[(size_t)m - 1], false, s))) return rc;
         }
-        if (dtype == HUB_F32 && (rc = launch_psi_finish(psi, H->D, s))) return rc;
     }
     double pn = 0.0;
     if ((rc = launch_dot(H, psi, psi, H->D, HUB_F64, H->red, s)) || (rc = reduce_partials_host(H->red, s, &pn))) return rc;
@@ -1491,7 +1490,7 @@ int lanczos_ground_state_refined(hubbard_t H, const void* v0, int max_iters, dou
     //    and psi are bit-identical whatever k is)
     const int k = std::min(m, store_cap);
     if (k >= 1) {
-        if ((rc = launch_psi_multi((const float*)store, (int64_t)(slot / 4), k, sv.data(), H->red, psi, H->D, k == m, s)))
+        if ((rc = launch_psi_multi((const float*)store, (int64_t)(slot / 4), k, sv.data(), H->red, psi, H->D, s)))
             return rc;
     }
     out->replayed = m - std::max(k, 1);
@@ -1531,7 +1530,6 @@ int lanczos_ground_state_refined(hubbard_t H, const void* v0, int max_iters, dou
             if ((rc = launch_axpy_scale(ru.a, ru.inv, ru.fo, ff, H->D, HUB_F32, s))) return rc;
             if ((rc = launch_psi_accumulate(ff, psi, H->D, sv[(size_t)m - 1], false, s))) return rc;
         }
-        if ((rc = launch_psi_finish(psi, H->D, s))) return rc;
     }
     double pn = 0.0;
     if ((rc = launch_dot(H, psi, psi, H->D, HUB_F64, H->red, s)) || (rc = reduce_partials_host(H->red, s, &pn))) return rc;

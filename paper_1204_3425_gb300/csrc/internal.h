@@ -257,17 +257,13 @@ int launch_scale(double a, void* y, int64_t n, int dtype, cudaStream_t s);
 int launch_copy_normalise(const void* x, void* y, int64_t n, int dtype, double inv_norm, cudaStream_t s);
 int launch_f64_to_f32_scaled(const double* x, float* y, int64_t n, double a, cudaStream_t s);
 int launch_fill_splitmix(void* v, int64_t n, unsigned long long seed, int64_t start, int dtype, cudaStream_t s);
-// psi <- (init ? 0 : psi) + s_j f; binary32 f: psi holds float-float pairs until
-// launch_psi_finish turns them into binary64
+// psi <- (init ? 0 : psi) + s_j f, in binary64
 int launch_psi_accumulate(const float* f, double* psi, int64_t n, double sj, bool init, cudaStream_t s);
-int launch_psi_finish(double* psi, int64_t n, cudaStream_t s);
 int launch_psi_accumulate_f64(const double* f, double* psi, int64_t n, double sj, bool init, cudaStream_t s);
 // psi = sum_{j<m} sv_j f_j, f_j = base + j * stride (binary32), coefficients
-// uploaded to dev (8 m bytes); bit-identical to m successive
-// launch_psi_accumulate calls, then launch_psi_finish when fin
-int launch_psi_multi(const float* base, int64_t stride, int m, const double* sv, void* dev, double* psi, int64_t n,
-                     bool fin, cudaStream_t s);
-
+// uploaded to dev (m doubles); bit-identical to m successive launch_psi_accumulate calls
+int launch_psi_multi(const float* base, int64_t stride, int m, const double* sv, double* dev, double* psi, int64_t n,
+                     cudaStream_t s);
 // the same for binary64 vectors, bit-identical to m launch_psi_accumulate_f64 calls
 int launch_psi_multi_f64(const double* base, int64_t stride, int m, const double* sv, double* dev, double* psi, int64_t n,
                          cudaStream_t s);

@@ -8,7 +8,6 @@
 // Packed hop entry: (target << 1) | (sign < 0); <target|H_sigma|src> = -t*sign.
 #include <cstdint>
 #include <mutex>
-#include <vector>
 #include <cuda_runtime.h>
 
 #include "internal.h"
@@ -329,41 +328,10 @@ __global__ void k_f64_to_f32_scaled(const double* __restrict__ x, float* __restr
         y[i] = (float)(a * x[i]);
 }
 
-// Ritz vector of binary32 Lanczos vectors: psi + s f in float-float (about 48
-// bits: the product split exactly, TwoSum), the pair (hi, lo) kept in the 8 bytes
-// of psi until k_psi_finish.  A binary64 multiply-add and the conversion of f
-// took both slots of the FP64 pipe (two lanes a clock), so combining 117 vectors
-// of 1.2e7 elements ran at 1.4 TB/s; the eleven binary32 operations leave it
-// bound by reading the vectors.  psi's error is that of the binary32 vectors,
-// 1e-6, on either route.
-struct SplitCoef {
-    float hi, lo;                                     // s = hi + lo to 2^-48
-};
-__device__ __forceinline__ void psi_add(float2& p, SplitCoef s, float f) {
-    const float q = __fmul_rn(s.hi, f);                // intrinsics: not contracted, the same bits in every kernel
-    const float e = fmaf(s.lo, f, fmaf(s.hi, f, -q));
-    const float t = __fadd_rn(p.x, q);
-    const float bb = __fsub_rn(t, p.x);
-    const float r = __fadd_rn(__fsub_rn(p.x, __fsub_rn(t, bb)), __fsub_rn(q, bb));
-    p.y = __fadd_rn(p.y, __fadd_rn(r, e));
-    p.x = t;
-}
-
-// psi <- (init ? 0 : psi) + s f
-__global__ void k_psi_acc(const float* __restrict__ f, float2* __restrict__ psi, int64_t n, SplitCoef s, int init) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        float2 p = init ? make_float2(0.0f, 0.0f) : psi[i];
-        psi_add(p, s, f[i]);
-        psi[i] = p;
-    }
-}
-
-// the pairs of k_psi_acc as binary64, in place
-__global__ void k_psi_finish(double* psi, int64_t n) {
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
-        const float2 p = reinterpret_cast<const float2*>(psi)[i];
-        psi[i] = (double)p.x + (double)p.y;
-    }
+// psi <- (init ? 0 : psi) + s * f  (binary32 f, binary64 psi)
+__global__ void k_psi_acc(const float* __restrict__ f, double* __restrict__ psi, int64_t n, double s, int init) {
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        psi[i] = init ? s * (double)f[i] : fma(s, (double)f[i], psi[i]);
 }
 
 // psi <- (init ? 0 : psi) + s * f  (binary64 f)
@@ -373,57 +341,42 @@ __global__ void k_psi_acc_f64(const double* __restrict__ f, double* __restrict__
 }
 
 // psi = sum_j s_j f_j over m stored binary32 vectors f_j = base + j * stride,
-// accumulated per element in j order with the operations of successive
-// k_psi_acc launches (so the result is bit-identical to that sequence); pairs,
-// or with fin the binary64 values.  Four elements per thread and four vectors'
-// 16-byte loads issued before their additions; base and stride must keep f_j
-// 16-byte aligned, psi 16-byte aligned.
-__global__ void __launch_bounds__(256) k_psi_multi(const float* __restrict__ base, int64_t stride, int m,
-                                                   const SplitCoef* __restrict__ s, double* __restrict__ psi,
-                                                   int64_t n, int fin) {
-    constexpr int U = 4;
-    const int64_t n4 = n / 4;
-    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n4; i += (int64_t)gridDim.x * blockDim.x) {
-        const float* p = base + 4 * i;
-        float2 a[4];
-#pragma unroll
-        for (int c = 0; c < 4; ++c) a[c] = make_float2(0.0f, 0.0f);
-        int j = 0;
+// accumulated per element in j order with the same operations as successive
+// k_psi_acc launches (so the result is bit-identical to that sequence).  Two
+// elements per thread and eight vectors' loads issued before their
+// multiply-adds (the loop is bound by the latency of m scattered streams);
+// base and stride must keep f_j 8-byte aligned, psi 16-byte aligned.
+__global__ void k_psi_multi(const float* __restrict__ base, int64_t stride, int m, const double* __restrict__ s,
+                            double* __restrict__ psi, int64_t n) {
+    constexpr int U = 8;
+    const int64_t n2 = n / 2;
+    for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n2; i += (int64_t)gridDim.x * blockDim.x) {
+        const float* p = base + 2 * i;
+        const float2 x0 = *reinterpret_cast<const float2*>(p);
+        double ax = s[0] * (double)x0.x, ay = s[0] * (double)x0.y;
+        int j = 1;
         for (; j + U <= m; j += U) {
-            float4 x[U];
+            float2 x[U];
 #pragma unroll
-            for (int q = 0; q < U; ++q) x[q] = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)(j + q) * stride));
+            for (int q = 0; q < U; ++q) x[q] = __ldcs(reinterpret_cast<const float2*>(p + (int64_t)(j + q) * stride));
 #pragma unroll
             for (int q = 0; q < U; ++q) {
-                const SplitCoef c = s[j + q];
-                psi_add(a[0], c, x[q].x);
-                psi_add(a[1], c, x[q].y);
-                psi_add(a[2], c, x[q].z);
-                psi_add(a[3], c, x[q].w);
+                ax = fma(s[j + q], (double)x[q].x, ax);
+                ay = fma(s[j + q], (double)x[q].y, ay);
             }
         }
         for (; j < m; ++j) {
-            const float4 x = __ldcs(reinterpret_cast<const float4*>(p + (int64_t)j * stride));
-            const SplitCoef c = s[j];
-            psi_add(a[0], c, x.x);
-            psi_add(a[1], c, x.y);
-            psi_add(a[2], c, x.z);
-            psi_add(a[3], c, x.w);
+            const float2 x = __ldcs(reinterpret_cast<const float2*>(p + (int64_t)j * stride));
+            ax = fma(s[j], (double)x.x, ax);
+            ay = fma(s[j], (double)x.y, ay);
         }
-        if (fin) {
-            reinterpret_cast<double2*>(psi)[2 * i] = make_double2((double)a[0].x + (double)a[0].y, (double)a[1].x + (double)a[1].y);
-            reinterpret_cast<double2*>(psi)[2 * i + 1] = make_double2((double)a[2].x + (double)a[2].y, (double)a[3].x + (double)a[3].y);
-        } else {
-            reinterpret_cast<float4*>(psi)[2 * i] = make_float4(a[0].x, a[0].y, a[1].x, a[1].y);
-            reinterpret_cast<float4*>(psi)[2 * i + 1] = make_float4(a[2].x, a[2].y, a[3].x, a[3].y);
-        }
+        reinterpret_cast<double2*>(psi)[i] = make_double2(ax, ay);
     }
-    if (blockIdx.x == 0 && threadIdx.x < (n & 3)) {
-        const int64_t i = 4 * n4 + threadIdx.x;
-        float2 a = make_float2(0.0f, 0.0f);
-        for (int j = 0; j < m; ++j) psi_add(a, s[j], __ldcs(base + (int64_t)j * stride + i));
-        if (fin) psi[i] = (double)a.x + (double)a.y;
-        else reinterpret_cast<float2*>(psi)[i] = a;
+    if ((n & 1) && blockIdx.x == 0 && threadIdx.x == 0) {
+        const int64_t i = n - 1;
+        double acc = s[0] * (double)base[i];
+        for (int j = 1; j < m; ++j) acc = fma(s[j], (double)__ldcs(base + (int64_t)j * stride + i), acc);
+        psi[i] = acc;
     }
 }
 
@@ -714,22 +667,9 @@ int launch_f64_to_f32_scaled(const double* x, float* y, int64_t n, double a, cud
     return HUB_OK;
 }
 
-static SplitCoef split_coef(double x) {
-    const float hi = (float)x;
-    return SplitCoef{hi, (float)(x - (double)hi)};
-}
-
 int launch_psi_accumulate(const float* f, double* psi, int64_t n, double sj, bool init, cudaStream_t s) {
     const int g = grid_for(n, kThreads * 8, sm_count() * 8);
-    k_psi_acc<<<g, kThreads, 0, s>>>(f, (float2*)psi, n, split_coef(sj), init ? 1 : 0);
-    HUB_CUDA(cudaGetLastError());
-    count_launches(1);
-    return HUB_OK;
-}
-
-int launch_psi_finish(double* psi, int64_t n, cudaStream_t s) {
-    const int g = grid_for(n, kThreads * 8, sm_count() * 8);
-    k_psi_finish<<<g, kThreads, 0, s>>>(psi, n);
+    k_psi_acc<<<g, kThreads, 0, s>>>(f, psi, n, sj, init ? 1 : 0);
     HUB_CUDA(cudaGetLastError());
     count_launches(1);
     return HUB_OK;
@@ -743,13 +683,11 @@ int launch_psi_accumulate_f64(const double* f, double* psi, int64_t n, double sj
     return HUB_OK;
 }
 
-int launch_psi_multi(const float* base, int64_t stride, int m, const double* sv, void* dev, double* psi, int64_t n,
-                     bool fin, cudaStream_t s) {
-    std::vector<SplitCoef> c((size_t)m);
-    for (int j = 0; j < m; ++j) c[(size_t)j] = split_coef(sv[j]);
-    HUB_CUDA(cudaMemcpyAsync(dev, c.data(), c.size() * sizeof(SplitCoef), cudaMemcpyHostToDevice, s));   // pageable: staged
-    const int g = grid_for(n, kThreads * 4, sm_count() * 8);
-    k_psi_multi<<<g, kThreads, 0, s>>>(base, stride, m, (const SplitCoef*)dev, psi, n, fin ? 1 : 0);
+int launch_psi_multi(const float* base, int64_t stride, int m, const double* sv, double* dev, double* psi, int64_t n,
+                     cudaStream_t s) {
+    HUB_CUDA(cudaMemcpyAsync(dev, sv, (size_t)m * sizeof(double), cudaMemcpyHostToDevice, s));   // pageable: staged
+    const int g = grid_for(n, kThreads * 8, sm_count() * 8);
+    k_psi_multi<<<g, kThreads, 0, s>>>(base, stride, m, dev, psi, n);
     HUB_CUDA(cudaGetLastError());
     count_launches(1);
     return HUB_OK;

@@ -66,8 +66,42 @@ def test_lanczos_scalars_are_the_recorded_ones(case):
     assert _run(*case) == want
 
 
+# binary32 vectors combined in binary64: lattice, N_up, N_dn, U
+PSI_CASES = [("sq3x3", 4, 4, 4.0), ("ring11", 5, 6, 7.3), ("ring12", 6, 6, 4.0)]
+
+
+def _psi32(lattice, nup, ndn, U, store):
+    """The Ritz vector of the refined solver (store: vectors it may keep), or of a
+    binary32 run (store None)."""
+    import paper_1204_3425_gb300 as hub
+    from workload import lattice_by_name, start_vector
+    ns, bonds = lattice_by_name(lattice)
+    H = hub.hubbard_sector_create(ns, bonds, nup, ndn, 1.0, U)
+    v = torch.from_numpy(start_vector(H.D, seed=31)).cuda()
+    psi = torch.empty_like(v)
+    if store is None:
+        r = hub.lanczos_ground_state(H, v.float(), 60, 0.0, psi_out=psi)
+    else:
+        r = hub.lanczos_ground_state_refined(H, v, 1000, 1e-10, psi_out=psi, store_vectors=store)
+    H.close()
+    return dict(energy=float(r["energy"]).hex(), psi=hashlib.sha256((psi.cpu().numpy() + 0.0).tobytes()).hexdigest())
+
+
+@pytest.mark.parametrize("case", PSI_CASES, ids=lambda c: "%s-%d-%d-%g" % c)
+def test_ritz_vectors_of_binary32_runs_are_the_recorded_ones(case):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 152:
+        pytest.skip("recorded on 152 SMs")
+    with open(GOLDEN) as f:
+        want = json.load(f)["psi32-%s-%d-%d-%g" % case]
+    assert _psi32(*case, None) == want["run"]
+    for store in (0, 1, 2, 9, 300):
+        assert _psi32(*case, store) == want["refined"], store
+
+
 if __name__ == "__main__":
     got = {"%s-%d-%d-%g-%s" % c[:5]: _run(*c) for c in CASES}
+    for c in PSI_CASES:
+        got["psi32-%s-%d-%d-%g" % c] = dict(run=_psi32(*c, None), refined=_psi32(*c, 300))
     with open(GOLDEN, "w") as f:
         json.dump(got, f, indent=0)
         f.write("\n")
