@@ -29,6 +29,7 @@
 #include "internal.h"
 #include "row_blocks.cuh"
 #include "hv_epilogue.cuh"
+#include "up_grid.h"
 
 namespace hub {
 
@@ -472,6 +473,9 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
 // thread's elements in that order (then block_sum3_store), so this division is
 // part of the result: a schedule may not change it.
 constexpr int kUpRows = 16;
+// CTAs an SM of the step kernels: their grids, and with them the partials, are at
+// most so many times the SMs
+constexpr int kStepCtas64 = 3, kStepCtas32 = 4;
 
 // Lanczos-step variant of k_up_f64x (Algorithm 1 fused with Algorithms 2, 4):
 // W = H f - beta w_old and, per CTA, the partials of <W, f>, <W, W> and
@@ -484,7 +488,7 @@ constexpr int kUpRows = 16;
 // has two rows' memory rounds in flight instead of one after the other (3x3 (4,4)
 // ground state with its vector 2.04 -> 1.92 ms).
 template <int VPL, bool FAST, bool TAIL, bool YS, int NT>
-__global__ void __launch_bounds__(NT, NT == 512 ? 1 : 3) k_up_step_f64x(
+__global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64x(
         const int2* __restrict__ X, const long long* __restrict__ Y, double* w, const double* w_old, int64_t Dup,
         int64_t Ddn, const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
         const uint32_t* __restrict__ list, const uint32_t* __restrict__ su, const uint32_t* __restrict__ sd,
@@ -623,7 +627,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : 3) k_up_step_f64x(
 // left of a hop list is requested at once on every size (4x4 (8,8) step 2.75 ->
 // 2.62 ms, ring 14 (7,7) 162 -> 146 us).
 template <int VPL>
-__global__ void __launch_bounds__(256, 4) k_up_step_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
+__global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
                                                         const float* w_old, int64_t Dup, int64_t Ddn,
                                                         const int32_t* __restrict__ ptr,
                                                         const int32_t* __restrict__ npos,
@@ -705,19 +709,6 @@ __global__ void __launch_bounds__(256, 4) k_up_step_f32(const float* __restrict_
 // requested at once.  Read per segment, the row pointer, the list and the
 // epilogue operands each added an L2 or HBM latency to the chain, and with
 // registers for 24-32 warps per SM the phase ran at that chain's pace.
-struct UpGrid {
-    int gx, gy;                      // row ranges, interleaved column chunks
-    int cap;                         // rows whose lists fit in shared memory at a time
-    int W;                           // longest hop list
-    size_t smem;
-};
-
-struct UpLists {
-    const uint32_t* list;            // [cap][W] target rows, sign +1 first
-    const int2* cnt;                 // [cap] (+1 targets, targets)
-    const uint32_t* st;              // [cap] basis words
-};
-
 __device__ __forceinline__ void stage_up_lists(unsigned char* smem, int cap, int W, int64_t r0, int nr,
                                                const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
                                                const uint32_t* __restrict__ list, const uint32_t* __restrict__ su) {
@@ -752,9 +743,6 @@ __device__ __forceinline__ void list_hops(const uint32_t* L, int np, int n, Add&
         if (q < end) add(true, L + q, std::integral_constant<int, 0>{}, end - q);
     }
 }
-
-// Cost of a row's segment in units of one hop, besides its hops.
-constexpr int kUpRowCost = 8;
 
 // First row of range i of gx: ranges of equal cost, sum of (hops + kUpRowCost).
 // The hop counts of neighbouring rows are alike (they share their upper sites),
@@ -1195,24 +1183,8 @@ int choose_vec(int req, int64_t len, int elem_bytes, int vmax, int reserve) {
     return req;
 }
 
-// Row ranges and column groups of the up phase: ranges of about 32 rows, the
-// chunks dealt to as many CTAs of each range as the device holds.  Longer ranges
-// let a list serve more segments, but the CTAs then differ more in how their
-// memory rounds add up (4x4 (5,5) binary64: 403, 385, 376, 392, 414 us with 7,
-// 14, 29, 57, 115 rows; 4x4 (8,8) binary32: 1.95, 1.91, 1.97, 2.01 ms with 21,
-// 42, 85, 169).
 UpGrid up_grid_for(const hubbard_sector* H, int64_t nchunk, int ctas) {
-    UpGrid g;
-    g.W = std::max(H->host[0].W, 1);
-    g.gy = (int)std::max<int64_t>(1, std::min<int64_t>(nchunk, (32 * (int64_t)ctas + H->Dup - 1) / H->Dup));
-    g.gx = (int)std::max<int64_t>(1, std::min<int64_t>(ctas / g.gy, (H->Dup + 7) / 8));
-    // most rows of a range: all of them without hops
-    const int64_t total = (int64_t)H->host[0].tgt.size() + kUpRowCost * H->Dup;
-    const int64_t rows = std::min<int64_t>(H->Dup, total / g.gx / kUpRowCost + 2);
-    const int64_t per_row = 12 + 4 * (int64_t)g.W;
-    g.cap = (int)std::max<int64_t>(1, std::min<int64_t>(rows, 24 * 1024 / per_row));
-    g.smem = (size_t)(g.cap * per_row);
-    return g;
+    return make_up_grid(H->Dup, (int64_t)H->host[0].tgt.size(), H->host[0].W, nchunk, ctas);
 }
 
 }  // namespace
@@ -1221,7 +1193,7 @@ UpGrid up_grid_for(const hubbard_sector* H, int64_t nchunk, int ctas) {
 // (the caller then uses the single-pass gather kernel).
 bool hv_phases_fuse(const hubbard_sector* H, int dtype) {
     if (H->Ddn > kMaxRow) return false;
-    if (sms() * 5 > kPartStride) return false;
+    if (sms() * kStepCtas32 > kPartStride) return false;   // one partial per CTA
     return dtype == HUB_F64 || choose_vec(H->vec_rows, H->Ddn, 4, 4, 0) != 0;
 }
 
@@ -1230,7 +1202,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
                      const RowUpdate* upd, LzDev* dv, double* hist) {
     if (nparts != nullptr) *nparts = 0;
     if (H->Ddn > kMaxRow) return -1;
-    if (sms() * 5 > kPartStride) part = nullptr;        // partial arrays too short: no fused reduction
+    if (sms() * kStepCtas32 > kPartStride) part = nullptr;   // partial arrays too short: no fused reduction
     const DevSpin& up = H->dev[0];
     const DevSpin& dn = H->dev[1];
     const int64_t Dup = H->Dup, Ddn = H->Ddn;
@@ -1323,7 +1295,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         int up_grid = 0;
         if (part != nullptr) {                            // a Lanczos step
             const int64_t items = up_step_items(vpl, Dup, Ddn);
-            up_grid = grid_cap(sms() * 3, items);
+            up_grid = grid_cap(sms() * kStepCtas64, items);
 #define UPS64(V, F, T, YS, NT)                                                                              \
     launch_on(pdl, k_up_step_f64x<V, F, T, YS, NT>, up_grid, NT, 0, s, Xg, Y, (double*)w, (const double*)w_old, Dup, \
         Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax, fixed_emax, (const double*)v, part, \
@@ -1411,7 +1383,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #undef ROWS32_U
     int up_grid = 0;
     if (part != nullptr) {                                // a Lanczos step
-        up_grid = grid_cap(sms() * 4, up_step_items(vpl, Dup, Ddn));
+        up_grid = grid_cap(sms() * kStepCtas32, up_step_items(vpl, Dup, Ddn));
 #define UPS32(V)                                                                                           \
     launch_on(pdl, k_up_step_f32<V>, up_grid, 256, 0, s, (const float*)v, Y, (float*)w, (const float*)w_old, Dup, \
         Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U, (float)-beta, \
