@@ -624,9 +624,10 @@ int hub::sector_create_streamed(int Ns, const int32_t* bonds, int n_bonds, int N
     H->D = H->Dup * H->Ddn;
     if (rc == HUB_OK) {
         cudaError_t e = dev_alloc((void**)&H->red, kRedSlots * sizeof(double), ms);
-        if (e == cudaSuccess) e = dev_alloc((void**)&H->status, 4 * sizeof(int), ms);
+        if (e == cudaSuccess) e = dev_alloc((void**)&H->status, (kStatusWords + kExpSlots) * sizeof(int), ms);
         if (e == cudaSuccess)
-            e = ms ? cudaMemsetAsync(H->status, 0, 4 * sizeof(int), ms) : cudaMemset(H->status, 0, 4 * sizeof(int));
+            e = ms ? cudaMemsetAsync(H->status, 0, kStatusWords * sizeof(int), ms)
+                   : cudaMemset(H->status, 0, kStatusWords * sizeof(int));
         if (e == cudaSuccess)
             e = ms ? cudaMemsetAsync(H->red, 0, kRedSlots * sizeof(double), ms)
                    : cudaMemset(H->red, 0, kRedSlots * sizeof(double));

@@ -48,6 +48,30 @@ __device__ __forceinline__ float comp(float x, int) { return x; }
 __device__ __forceinline__ float comp(float2 x, int i) { return i == 0 ? x.x : x.y; }
 __device__ __forceinline__ float comp(float4 x, int i) { return i == 0 ? x.x : (i == 1 ? x.y : (i == 2 ? x.z : x.w)); }
 
+// The exponent bound of a product, found by every CTA of its row phase: the
+// largest exponent of v itself (scan: at most kScanElems elements), or of the
+// per-CTA maxima an exponent pass left in slots[0 .. nslots).  CTA 0 hands it on to
+// the up phase in *emax_p.  Every word is written before it is read within the
+// product, so nothing has to be set back between products.
+__device__ __forceinline__ int cta_exponent(const double* v, int n, const int* slots, int nslots, int* emax_p) {
+    __shared__ int emax_s;
+    if (threadIdx.x == 0) emax_s = 1;
+    __syncthreads();
+    int m = 1;
+    if (slots != nullptr) {
+        for (int i = threadIdx.x; i < nslots; i += blockDim.x) m = max(m, slots[i]);
+    } else {
+#pragma unroll 8
+        for (int i = threadIdx.x; i < n; i += blockDim.x)
+            m = max(m, (int)(((unsigned long long)__double_as_longlong(v[i]) >> 52) & 0x7FF));
+    }
+    m = __reduce_max_sync(0xffffffffu, m);
+    if ((threadIdx.x & 31) == 0) atomicMax(&emax_s, m);
+    __syncthreads();
+    if (blockIdx.x == 0 && threadIdx.x == 0) *emax_p = emax_s;
+    return emax_s;
+}
+
 // Row phase, binary64 fixed point: Y[u, d] = sum_{(d', s) in hops_dn(d)} s X[u, d'];
 // also writes the fixed-point copy of V to Xg for the up phase.
 // UPD: the previous Lanczos step's update is applied on the way in,
@@ -60,6 +84,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
                                                      const int32_t* __restrict__ bcnt,
                                                      const EntT* __restrict__ ent,
                                                      int* emax_p, int fixed_emax, int scan,
+                                                     const int* slots, int nslots,
                                                      const double* __restrict__ fo, double ua, double uinv,
                                                      const LzDev* __restrict__ dv) {
     using S = typename FxVec<VEC>::T;
@@ -74,25 +99,8 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
     extern __shared__ __align__(16) unsigned char smem_raw[];
     S* X = reinterpret_cast<S*>(smem_raw);
     int emax = fixed_emax;
-    if (!UPD && scan) {
-        // a sector this small: every CTA finds max|v| itself (the same word from
-        // all of them), which saves the pass before this one
-        __shared__ int emax_s;
-        if (threadIdx.x == 0) emax_s = 1;
-        __syncthreads();
-        int m = 1;
-        const int n = (int)(Dup * Ddn);
-#pragma unroll 8
-        for (int i = threadIdx.x; i < n; i += blockDim.x)
-            m = max(m, (int)(((unsigned long long)__double_as_longlong(v[i]) >> 52) & 0x7FF));
-        m = __reduce_max_sync(0xffffffffu, m);
-        if ((threadIdx.x & 31) == 0) atomicMax(&emax_s, m);
-        __syncthreads();
-        emax = emax_s;
-        if (threadIdx.x == 0) *emax_p = emax;
-    } else if (fixed_emax <= 0) {
-        emax = max(*emax_p, 1);
-    }
+    if (!UPD && (scan || slots != nullptr)) emax = cta_exponent(v, (int)(Dup * Ddn), slots, nslots, emax_p);
+    else if (fixed_emax <= 0) emax = max(*emax_p, 1);
     const int lane = threadIdx.x & 31;
     const int64_t nblk = (Dup + VEC - 1) / VEC;
     const int64_t step = blockDim.x;
@@ -188,11 +196,14 @@ __global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* __re
                                                             const int64_t* __restrict__ boff,
                                                             const int32_t* __restrict__ bcnt,
                                                             const EntT* __restrict__ ent,
-                                                            const int* __restrict__ emax_p, int fixed_emax) {
+                                                            int* emax_p, int fixed_emax, const int* slots,
+                                                            int nslots) {
     grid_dep_wait();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     int* Xs = reinterpret_cast<int*>(smem_raw);
-    const int emax = fixed_emax > 0 ? fixed_emax : max(*emax_p, 1);
+    const int emax = fixed_emax > 0     ? fixed_emax
+                     : slots != nullptr ? cta_exponent(v, 0, slots, nslots, emax_p)
+                                        : max(*emax_p, 1);
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
     const int n = (int)Ddn, z0 = (int)staged_slots(Ddn) - 32;
     if (threadIdx.x < 32) Xs[z0 + threadIdx.x] = 0;
@@ -266,14 +277,6 @@ __global__ void __launch_bounds__(512) k_rows_global_f64x(const int2* __restrict
     }
 }
 
-
-// The last CTA of a kernel sets the exponent word it has read back to 0 for the
-// next product (counter: nullptr, nothing to do; it returns to 0 by itself).
-__device__ __forceinline__ void reset_exponent(int* emax_p, unsigned* counter) {
-    if (counter == nullptr || threadIdx.x != 0) return;
-    __threadfence();
-    if (atomicInc(counter, gridDim.x - 1) == gridDim.x - 1) *emax_p = 0;
-}
 
 // An item of 16 rows is two per warp; where that leaves fewer items than CTAs
 // that fit on the device, 8 rows (one per warp) spread the sector wider.
@@ -376,7 +379,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
-                                                     int* emax_p, int fixed_emax, unsigned* reset) {
+                                                     const int* __restrict__ emax_p, int fixed_emax) {
     constexpr int VPL = 2;
     using IV = int4;
     __shared__ long long Bs[33];
@@ -464,7 +467,6 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
             }
         }
     }
-    reset_exponent(emax_p, reset);
 }
 
 // Work of the Lanczos step kernels: items of 32 * VPL columns by kUpRows rows,
@@ -820,7 +822,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
-                                                     int* emax_p, int fixed_emax, unsigned* reset) {
+                                                     const int* __restrict__ emax_p, int fixed_emax) {
     grid_dep_wait();
     using IV = typename FxVec<VPL>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -911,7 +913,6 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
         if constexpr (VPL == 2) __stcs(reinterpret_cast<double2*>(w + J), make_double2(res[0], res[1]));
         else __stcs(w + J, res[0]);
     });
-    reset_exponent(emax_p, reset);
 }
 
 // Binary32: same decomposition, float arithmetic.  NV vectors of VPL columns
@@ -1207,7 +1208,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     const DevSpin& dn = H->dev[1];
     const int64_t Dup = H->Dup, Ddn = H->Ddn;
     const bool dn16 = dn.ent16 != nullptr;
-    unsigned* done = reinterpret_cast<unsigned*>(H->status + 3);
+    unsigned* done = reinterpret_cast<unsigned*>(H->status + 2);   // of the step kernels alone
     const bool pdl = H->D * (dtype == HUB_F64 ? 8 : 4) <= kPdlBytes;
     // up-phase CTAs: as many as the launch bounds keep resident (the phase is
     // bound by L2 latency, so occupancy is what counts: 4 per SM at <= 64
@@ -1216,13 +1217,16 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     // to 2 columns per lane; measured best)
     if (dtype == HUB_F64) {
         const int va = choose_vec(H->vec_rows, Ddn, 8, 2, 0);
-        // exponent word: found by the row phase itself on the smallest sectors,
-        // by a pass of its own otherwise; on sectors that launch overlapped the
-        // word is one that the last CTA of the product's up phase sets back to
-        // 0, so no memset breaks the chain of kernels
+        // exponent bound: found by the row phase itself on the smallest sectors, by a
+        // pass of its own otherwise.  On sectors that launch overlapped that pass
+        // leaves one maximum per CTA, which the row phase reduces: no memset of a
+        // word that all CTAs raise breaks the chain of kernels.
+        const bool ysplit = va == 0 && staged_slots(Ddn) * 4 <= smem_optin();
         const int scan = fixed_emax <= 0 && w_old == nullptr && va > 0 && H->D <= kScanElems;
-        const bool self_reset = fixed_emax <= 0 && w_old == nullptr && pdl && !scan;
-        int* emax = self_reset ? H->status + 2 : H->status;
+        const bool by_slots = fixed_emax <= 0 && w_old == nullptr && pdl && !scan && (va > 0 || ysplit);
+        int* emax = H->status;
+        const int* slots = by_slots ? H->status + kStatusWords : nullptr;
+        int nslots = 0;
         // the deferred update goes into the row phase when it stages rows in
         // shared memory with a fixed exponent bound; otherwise it is one pass first
         if (upd != nullptr && (va == 0 || fixed_emax <= 0)) {
@@ -1231,16 +1235,19 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
             upd = nullptr;
         }
         if (fixed_emax <= 0 && !scan) {
-            if (!self_reset) HUB_CUDA(cudaMemsetAsync(emax, 0, sizeof(int), s));
-            launch_max_exponent((const double*)v, H->D, emax, s, self_reset);
-            if (w_old != nullptr) launch_max_exponent((const double*)w_old, H->D, emax, s);
+            if (by_slots) {
+                nslots = launch_max_exponent_slots((const double*)v, H->D, H->status + kStatusWords, s);
+            } else {
+                HUB_CUDA(cudaMemsetAsync(emax, 0, sizeof(int), s));
+                launch_max_exponent((const double*)v, H->D, emax, s);
+                if (w_old != nullptr) launch_max_exponent((const double*)w_old, H->D, emax, s);
+            }
         }
         Launch LA = shape((size_t)staged_slots(Ddn) * 8 * std::max(va, 1), H->ctas_rows);
         LA.blocks = grid_cap(LA.blocks, (Dup + std::max(va, 1) - 1) / std::max(va, 1));   // no idle CTAs
         long long* Y = (long long*)ybuf;
         int2* Xg = (int2*)((char*)ybuf + (size_t)H->D * 8);
         int extra = 0;
-        const bool ysplit = va == 0 && staged_slots(Ddn) * 4 <= smem_optin();
         if (ysplit) {
             // rows of which one word per element fits in shared memory
             const size_t sm = (size_t)staged_slots(Ddn) * 4;
@@ -1250,7 +1257,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #define PLANES64(E, P)                                                                                      \
     allow_smem<k_rows_planes_f64x<E>>();                                                                    \
     launch_on(pdl, k_rows_planes_f64x<E>, blocks, 1024, sm, s, (const double*)v, (int*)Y, Xg, Dup, Ddn, \
-        dn.blk_off, dn.blk_cnt, P, emax, fixed_emax)
+        dn.blk_off, dn.blk_cnt, P, emax, fixed_emax, slots, nslots)
             if (dn16) { PLANES64(uint16_t, dn.ent16); } else { PLANES64(uint32_t, dn.ent32); }
 #undef PLANES64
         } else if (va == 0) {
@@ -1275,7 +1282,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #define ROWS64_U(V, E, P, U)                                                                                \
     allow_smem<k_rows_f64x<V, E, U>>();                                                                      \
     launch_on(pdl, k_rows_f64x<V, E, U>, LA.blocks, LA.threads, LA.smem, s, (double*)const_cast<void*>(v), Y, Xg, Dup,   \
-        Ddn, dn.blk_off, dn.blk_cnt, P, emax, fixed_emax, scan, upd ? (const double*)upd->fo : nullptr,            \
+        Ddn, dn.blk_off, dn.blk_cnt, P, emax, fixed_emax, scan, slots, nslots, upd ? (const double*)upd->fo : nullptr,            \
         upd ? upd->a : 0.0, upd ? upd->inv : 1.0, upd ? upd->dv : nullptr)
 #define ROWS64(V, E, P) if (upd) { ROWS64_U(V, E, P, true); } else { ROWS64_U(V, E, P, false); }
         if (va == 2) {
@@ -1290,7 +1297,6 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         const EpiParams ep = make_epilogue(H->t, H->U, H->ns, w_old ? beta : 0.0, H->host[0].W + H->host[1].W);
         // columns per lane in the up phase: 2 when Ddn is even (16-byte loads)
         const int vpl = ((Ddn & 1) == 0 && H->vec_cols != 1) ? 2 : 1;
-        unsigned* reset = self_reset ? done : nullptr;
         const bool tail = H->D <= kUpSmall;
         int up_grid = 0;
         if (part != nullptr) {                            // a Lanczos step
@@ -1318,7 +1324,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #define UPR64(V, F, OLD, YS, CT)                                                                            \
     launch_on(pdl, k_upr_f64x<V, F, OLD, YS, CT>, g.gx * g.gy, 256, g.smem, s, Xg, Y, (double*)w,              \
         (const double*)w_old, Dup, Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep, emax,  \
-        fixed_emax, reset)
+        fixed_emax)
 #define UPR64_S(V, F)                                                                                      \
     if (ysplit) { if (three) { UPR64(V, F, true, true, 3); } else { UPR64(V, F, false, true, 4); } }       \
     else if (w_old != nullptr) { UPR64(V, F, true, false, 3); }                                            \
@@ -1343,7 +1349,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #define UP64(CT, ...)                                                                                       \
     launch_on(pdl, k_up_f64x<__VA_ARGS__>, grid_cap(sms() * CT, up_items), 256, 0, s, Xg, Y, (double*)w,       \
         (const double*)w_old, Dup, Ddn, rbr, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, ep,  \
-        emax, fixed_emax, reset)
+        emax, fixed_emax)
 #define UP64_T(F, T)                                                                                        \
     if (pre) { UP64(3, F, T, true, 3); } else { UP64(4, F, T); }
             if (tail) {

@@ -123,7 +123,10 @@ struct hubbard_sector {
     int fixed_emax_host = 1023;      // host copy for the device word used by the fixed-scale fallback
     // small device scratch for reductions: partial sums, status words
     double* red = nullptr;           // [kRedSlots]
-    int* status = nullptr;           // [4]
+    // status words: 0 exponent bound of a product, 1 a fixed one (rows read from
+    // global memory), 2 CTAs of a Lanczos step counted (close_sums3; 0 between
+    // steps); then kExpSlots per-CTA exponents of a product
+    int* status = nullptr;           // [kStatusWords + kExpSlots]
     // device-resident Lanczos control (LzDev) and a/b history for lz_cap steps
     void* lz = nullptr;
     int lz_cap = 0;
@@ -136,6 +139,8 @@ struct hubbard_sector {
 };
 
 namespace hub {
+constexpr int kStatusWords = 32;     // a cache line of status words
+constexpr int kExpSlots = 1024;      // grid size of the exponent pass
 constexpr int kRedSlots = 4096;      // partial-sum slots for block reductions
 constexpr int kRedBlocks = 1024;     // grid size of reduction kernels (<= kRedSlots/2)
 constexpr int kPartStride = 1024;    // stride of the partial arrays of a fused three-value reduction
@@ -233,8 +238,10 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 // whether launch_hv_phases fuses the Lanczos reductions for this sector and dtype
 bool hv_phases_fuse(const hubbard_sector* H, int dtype);
 // max biased binary64 exponent of |v| folded into *emax (atomicMax; caller zeroes it)
-// (pdl: launched as launch_on)
-void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s, bool pdl = false);
+void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s);
+// max biased binary64 exponent of each CTA's part of |v|, in slots[0 .. returned count)
+// (launched as launch_on)
+int launch_max_exponent_slots(const double* v, int64_t n, int* slots, cudaStream_t s);
 // binary64 -> (lo, hi) fixed point with the exponent bound *emax (read on the device)
 void launch_to_fixed(const double* v, int64_t n, void* X, const int* emax, cudaStream_t s);
 int launch_dot(const hubbard_sector* H, const void* x, const void* y, int64_t n, int dtype,

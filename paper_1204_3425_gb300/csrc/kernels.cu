@@ -78,16 +78,33 @@ __global__ void k_hv_reference(const T* __restrict__ v, T* __restrict__ w, int64
 // |hi| <= 2^24).  A hop sum of up to 2^6 signed terms then fits two int32
 // accumulators without carries, and is exact.
 
-// max biased exponent of |v| -> *emax (atomicMax; *emax must start at 0)
-__global__ void k_max_exponent(const double* __restrict__ v, int64_t n, int* emax) {
-    grid_dep_wait();
+// max biased exponent of |v| over this thread's elements, then over its warp
+__device__ __forceinline__ int warp_max_exponent(const double* v, int64_t n) {
     int m = 0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const unsigned long long b = (unsigned long long)__double_as_longlong(v[i]);
         m = max(m, (int)((b >> 52) & 0x7FF));
     }
     for (int o = 16; o > 0; o >>= 1) m = max(m, __shfl_xor_sync(0xffffffffu, m, o));
+    return m;
+}
+// -> *emax (atomicMax; *emax must start at 0)
+__global__ void k_max_exponent(const double* __restrict__ v, int64_t n, int* emax) {
+    const int m = warp_max_exponent(v, n);
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(emax, m);
+}
+// -> slots[blockIdx.x], every CTA its own
+__global__ void k_max_exponent_slots(const double* __restrict__ v, int64_t n, int* slots) {
+    grid_dep_wait();
+    __shared__ int ws[kThreads / 32];
+    const int m = warp_max_exponent(v, n);
+    if ((threadIdx.x & 31) == 0) ws[threadIdx.x >> 5] = m;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+        int t = 0;
+        for (int i = 0; i < kThreads / 32; ++i) t = max(t, ws[i]);
+        slots[blockIdx.x] = t;
+    }
 }
 
 // rounding of one binary64 to the fixed-point grid given the exponent bound
@@ -522,9 +539,15 @@ void launch_to_fixed(const double* v, int64_t n, void* X, const int* emax, cudaS
     k_to_fixed<<<g2, kThreads, 0, s>>>(v, (int2*)X, n, emax);
 }
 
-void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s, bool pdl) {
+void launch_max_exponent(const double* v, int64_t n, int* emax, cudaStream_t s) {
     const int g2 = grid_for(n, kThreads * 8, sm_count() * 8);
-    launch_on(pdl, k_max_exponent, g2, kThreads, 0, s, v, n, emax);
+    k_max_exponent<<<g2, kThreads, 0, s>>>(v, n, emax);
+}
+
+int launch_max_exponent_slots(const double* v, int64_t n, int* slots, cudaStream_t s) {
+    const int g2 = grid_for(n, kThreads * 8, kExpSlots);
+    launch_on(true, k_max_exponent_slots, g2, kThreads, 0, s, v, n, slots);
+    return g2;
 }
 
 int launch_hv_fast(hubbard_sector* H, const void* v, void* w, int dtype, double beta, const void* w_old,
