@@ -729,21 +729,23 @@ __device__ __forceinline__ void stage_up_lists(unsigned char* smem, int cap, int
     }
 }
 
-// Sums over a staged hop list in the order of uniform_hops: windows of 32 entries,
-// in each the +1 targets and then the -1 targets.  add(neg, entries, k) sees
-// groups of four, then what is left of the sign as one group of k < 4, so that the
-// loads of a group are always requested together (a rest taken one by one is a
-// memory latency for each of its entries).
-template <typename Add>
+// Sums over a staged hop list, +1 targets then -1 targets: add(neg, entries, k)
+// sees groups of four, then what is left of the sign as one group of k < 4, so that
+// the loads of a group are always requested together (a rest taken one by one is a
+// memory latency for each of its entries).  WINDOWS: in windows of 32 entries, the
+// order of uniform_hops, for sums that round.
+template <bool WINDOWS, typename Add>
 __device__ __forceinline__ void list_hops(const uint32_t* L, int np, int n, Add&& add) {
-    for (int k0 = 0; k0 < n; k0 += 32) {
-        const int end = min(k0 + 32, n), pend = max(k0, min(end, np));
-        int q = k0;
+    int q = 0, end = n;
+    do {
+        if constexpr (WINDOWS) end = min(q + 32, n);
+        const int pend = WINDOWS ? max(q, min(end, np)) : np;
         for (; q + 4 <= pend; q += 4) add(false, L + q, std::integral_constant<int, 4>{}, 4);
         if (q < pend) add(false, L + q, std::integral_constant<int, 0>{}, pend - q);
         for (q = pend; q + 4 <= end; q += 4) add(true, L + q, std::integral_constant<int, 4>{}, 4);
         if (q < end) add(true, L + q, std::integral_constant<int, 0>{}, end - q);
-    }
+        q = end;
+    } while (WINDOWS && end < n);
 }
 
 // First row of range i of gx: ranges of equal cost, sum of (hops + kUpRowCost).
@@ -864,7 +866,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
         }
         IV A{};
         const int2 np = cnt[r];
-        list_hops(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
+        list_hops<false>(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
             IV x[4];
 #pragma unroll
             for (int q = 0; q < 4; ++q) {
@@ -953,7 +955,7 @@ __global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, 
             return __ldg(reinterpret_cast<const V*>(reinterpret_cast<const char*>(v + c[i]) + (uint64_t)t * rowb));
         };
         const int2 np = cnt[r];
-        list_hops(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
+        list_hops<true>(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
             V x[NV][4];
 #pragma unroll
             for (int q = 0; q < 4; ++q)

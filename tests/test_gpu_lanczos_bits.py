@@ -98,6 +98,22 @@ def test_ritz_vectors_of_binary32_runs_are_the_recorded_ones(case):
         assert _psi32(*case, store) == want["refined"], store
 
 
+def test_replayed_steps_sum_long_hop_lists_in_the_steps_order():
+    """36 up-hops a state: more than a window of 32.  The replay's kernel stages its hop
+    lists, the step's reads them; a psi of kept and of replayed vectors is the same."""
+    import paper_1204_3425_gb300 as hub
+    from workload import start_vector
+    H = hub.hubbard_sector_create(10, [(i, j) for i in range(10) for j in range(i)], 6, 4, 1.0, 3.0)
+    H2 = hub.hubbard_sector_create(12, [(i, j) for i in range(12) for j in range(i)], 6, 3, 1.0, 3.0)
+    for h in (H, H2):
+        v = torch.from_numpy(start_vector(h.D, seed=7)).cuda()
+        psi = [torch.empty_like(v) for _ in range(3)]
+        for p, store in zip(psi, (300, 0, 5)):
+            hub.lanczos_ground_state_refined(h, v, 60, 1e-10, psi_out=p, store_vectors=store)
+        assert torch.equal(psi[0], psi[1]) and torch.equal(psi[0], psi[2])
+        h.close()
+
+
 if __name__ == "__main__":
     got = {"%s-%d-%d-%g-%s" % c[:5]: _run(*c) for c in CASES}
     for c in PSI_CASES:
