@@ -77,7 +77,7 @@ __device__ __forceinline__ int cta_exponent(const double* v, int n, const int* s
 // UPD: the previous Lanczos step's update is applied on the way in,
 // v <- (v + ua fo) * uinv, rounded as k_axpy_scale_f64, and written back to v.
 template <int VEC, typename EntT, bool UPD>
-__global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, double*, const double*> __restrict__ v,
+__global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, double*, const double*> v,
                                                      long long* __restrict__ Y,
                                                      int2* __restrict__ Xg, int64_t Dup, int64_t Ddn,
                                                      const int64_t* __restrict__ boff,
@@ -85,8 +85,8 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
                                                      const EntT* __restrict__ ent,
                                                      int* emax_p, int fixed_emax, int scan,
                                                      const int* slots, int nslots,
-                                                     const double* __restrict__ fo, double ua, double uinv,
-                                                     const LzDev* __restrict__ dv) {
+                                                     const double* fo, double ua, double uinv,
+                                                     const LzDev* dv) {
     using S = typename FxVec<VEC>::T;
     grid_dep_wait();
     if constexpr (UPD) {
@@ -191,7 +191,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
 // the up phase joins them: joined here, each CTA would stage both words of two
 // rows instead of three planes (259 us).
 template <typename EntT>
-__global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* __restrict__ v, int* __restrict__ Ys,
+__global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* v, int* __restrict__ Ys,
                                                             int2* __restrict__ Xg, int64_t Dup, int64_t Ddn,
                                                             const int64_t* __restrict__ boff,
                                                             const int32_t* __restrict__ bcnt,
@@ -221,7 +221,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* __re
 #pragma unroll
             for (int i = 0; i < NL; ++i) {
                 const int d = d0 + i * blockDim.x;
-                x[i] = d < n ? __ldg(row + d) : 0.0;
+                x[i] = d < n ? row[d] : 0.0;
             }
 #pragma unroll
             for (int i = 0; i < NL; ++i) {
@@ -371,7 +371,7 @@ template <typename IV> struct AddFixed {
 // PRE: the epilogue's own element and Y are requested before the gathers (their
 // HBM latency then overlaps the hop sum); CT: CTAs per SM the launch bounds keep
 template <bool FAST, bool TAIL, bool PRE = false, int CT = 4>
-__global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
+__global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* X, const long long* Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
                                                      int rbr, const int32_t* __restrict__ ptr,
                                                      const int32_t* __restrict__ npos,
@@ -379,7 +379,7 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
-                                                     const int* __restrict__ emax_p, int fixed_emax) {
+                                                     const int* emax_p, int fixed_emax) {
     constexpr int VPL = 2;
     using IV = int4;
     __shared__ long long Bs[33];
@@ -416,12 +416,12 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
             [[maybe_unused]] longlong2 y2p;
             if constexpr (PRE) {
                 const int64_t J = u * Ddn + c;
-                t4p = __ldg(reinterpret_cast<const int4*>(X + J));
-                y2p = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+                t4p = *(reinterpret_cast<const int4*>(X + J));
+                y2p = ld_stream(reinterpret_cast<const longlong2*>(Y + J));
             }
             IV A{};
             uniform_hops<IV, TAIL>(list, kb, ptr[u + 1] - kb, npos[u], lane,
-                [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); },
+                [&](uint32_t t) { return *(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); },
                 AddFixed<IV>{A});
             if (act) {
                 const uint32_t su_u = su[u];
@@ -436,8 +436,8 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* __restrict__ X,
                     t4 = t4p;
                     y2 = y2p;
                 } else {
-                    t4 = __ldg(reinterpret_cast<const int4*>(X + J));
-                    y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+                    t4 = *(reinterpret_cast<const int4*>(X + J));
+                    y2 = ld_stream(reinterpret_cast<const longlong2*>(Y + J));
                 }
                 xo[0] = make_int2(t4.x, t4.y);
                 xo[1] = make_int2(t4.z, t4.w);
@@ -491,11 +491,11 @@ constexpr int kStepCtas64 = 3, kStepCtas32 = 4;
 // ground state with its vector 2.04 -> 1.92 ms).
 template <int VPL, bool FAST, bool TAIL, bool YS, int NT>
 __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64x(
-        const int2* __restrict__ X, const long long* __restrict__ Y, double* w, const double* w_old, int64_t Dup,
+        const int2* X, const long long* Y, double* w, const double* w_old, int64_t Dup,
         int64_t Ddn, const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
         const uint32_t* __restrict__ list, const uint32_t* __restrict__ su, const uint32_t* __restrict__ sd,
-        const __grid_constant__ EpiParams ep, const int* __restrict__ emax_p, int fixed_emax,
-        const double* __restrict__ fv, double* part, unsigned* done, LzDev* dv, double* hist) {
+        const __grid_constant__ EpiParams ep, const int* emax_p, int fixed_emax,
+        const double* fv, double* part, unsigned* done, LzDev* dv, double* hist) {
     grid_dep_wait();
     if (dv != nullptr && dv->stall) return;
     using IV = typename FxVec<VPL>::T;
@@ -548,24 +548,24 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
             // streamed operands of the epilogue, requested before the gathers
             double wv[VPL];
             long long yv[VPL];
-            const IV xo4 = __ldg(reinterpret_cast<const IV*>(X + J));
+            const IV xo4 = *(reinterpret_cast<const IV*>(X + J));
             if constexpr (VPL == 2) {
-                const longlong2 y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+                const longlong2 y2 = ld_stream(reinterpret_cast<const longlong2*>(Y + J));
                 yv[0] = y2.x; yv[1] = y2.y;
                 if (w_old != nullptr) {
-                    const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
+                    const double2 q = ld_stream(reinterpret_cast<const double2*>(w_old + J));
                     wv[0] = q.x; wv[1] = q.y;
                 }
-                const double2 q = __ldcs(reinterpret_cast<const double2*>(fv + J));
+                const double2 q = ld_stream(reinterpret_cast<const double2*>(fv + J));
                 fj[0] = q.x; fj[1] = q.y;
             } else {
-                yv[0] = __ldcs(Y + J);
-                if (w_old != nullptr) wv[0] = __ldcs(w_old + J);
-                fj[0] = __ldcs(fv + J);
+                yv[0] = ld_stream(Y + J);
+                if (w_old != nullptr) wv[0] = ld_stream(w_old + J);
+                fj[0] = ld_stream(fv + J);
             }
             IV A{};
             uniform_hops<IV, TAIL>(list, kb, ptr[u + 1] - kb, npos[u], lane,
-                [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (int64_t)t * Ddn)); },
+                [&](uint32_t t) { return *(reinterpret_cast<const IV*>(base + (int64_t)t * Ddn)); },
                 AddFixed<IV>{A});
             if (!act) continue;
             const uint32_t su_u = su[u];
@@ -629,7 +629,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
 // left of a hop list is requested at once on every size (4x4 (8,8) step 2.75 ->
 // 2.62 ms, ring 14 (7,7) 162 -> 146 us).
 template <int VPL>
-__global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
+__global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* v, const float* Y, float* w,
                                                         const float* w_old, int64_t Dup, int64_t Ddn,
                                                         const int32_t* __restrict__ ptr,
                                                         const int32_t* __restrict__ npos,
@@ -667,13 +667,13 @@ __global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* _
             const int32_t kb = ptr[u];
             const int64_t J = u * Ddn + c;
             // epilogue operands, requested before the gathers
-            const V xo = __ldg(reinterpret_cast<const V*>(v + J));
-            const V yv = __ldcs(reinterpret_cast<const V*>(Y + J));
+            const V xo = *(reinterpret_cast<const V*>(v + J));
+            const V yv = ld_stream(reinterpret_cast<const V*>(Y + J));
             V wv{};
-            if (w_old != nullptr) wv = __ldcs(reinterpret_cast<const V*>(w_old + J));
+            if (w_old != nullptr) wv = ld_stream(reinterpret_cast<const V*>(w_old + J));
             V P{}, N{};
             uniform_hops<V, true>(list, kb, ptr[u + 1] - kb, npos[u], lane,
-                [&](uint32_t t) { return __ldg(reinterpret_cast<const V*>(base + (int64_t)t * Ddn)); },
+                [&](uint32_t t) { return *(reinterpret_cast<const V*>(base + (int64_t)t * Ddn)); },
                 AddFloat<V>{P, N});
             if (!act) continue;
             const uint32_t su_u = su[u];
@@ -816,7 +816,7 @@ __device__ __forceinline__ void up_segments(unsigned char* smem, int64_t Dup, in
 // beta w_old.  CT: CTAs per SM the launch bounds keep.  YS: Y holds word pairs
 // (k_rows_planes_f64x).
 template <int VPL, bool FAST, bool OLD, bool YS, int CT>
-__global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X, const long long* __restrict__ Y,
+__global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* X, const long long* Y,
                                                      double* w, const double* w_old, int64_t Dup, int64_t Ddn,
                                                      UpGrid g, const int32_t* __restrict__ ptr,
                                                      const int32_t* __restrict__ npos,
@@ -824,7 +824,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
                                                      const uint32_t* __restrict__ su,
                                                      const uint32_t* __restrict__ sd,
                                                      const __grid_constant__ EpiParams ep,
-                                                     const int* __restrict__ emax_p, int fixed_emax) {
+                                                     const int* emax_p, int fixed_emax) {
     grid_dep_wait();
     using IV = typename FxVec<VPL>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -845,24 +845,24 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
         const int64_t c = act ? c_raw : Ddn - VPL;     // tail lanes read a valid column, store nothing
         const int64_t J = (r0 + r) * Ddn + c;
         const char* base = reinterpret_cast<const char*>(X + c);
-        auto load = [&](uint32_t t) { return __ldg(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); };
+        auto load = [&](uint32_t t) { return *(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); };
         // epilogue operands, requested with the gathers
-        const IV xo4 = __ldg(reinterpret_cast<const IV*>(X + J));
+        const IV xo4 = *(reinterpret_cast<const IV*>(X + J));
         long long yv[VPL];
         double wv[VPL];
         uint32_t sdc[VPL];
         if constexpr (VPL == 2) {
-            const longlong2 y2 = __ldcs(reinterpret_cast<const longlong2*>(Y + J));
+            const longlong2 y2 = ld_stream(reinterpret_cast<const longlong2*>(Y + J));
             yv[0] = y2.x;
             yv[1] = y2.y;
             if constexpr (OLD) {
-                const double2 q = __ldcs(reinterpret_cast<const double2*>(w_old + J));
+                const double2 q = ld_stream(reinterpret_cast<const double2*>(w_old + J));
                 wv[0] = q.x;
                 wv[1] = q.y;
             }
         } else {
-            yv[0] = __ldcs(Y + J);
-            if constexpr (OLD) wv[0] = __ldcs(w_old + J);
+            yv[0] = ld_stream(Y + J);
+            if constexpr (OLD) wv[0] = ld_stream(w_old + J);
         }
         IV A{};
         const int2 np = cnt[r];
@@ -921,7 +921,7 @@ __global__ void __launch_bounds__(256, CT) k_upr_f64x(const int2* __restrict__ X
 // per lane, 32 * VPL columns apart, so rows whose length only allows narrow
 // vectors still keep as many bytes in flight.
 template <int VPL, int NV>
-__global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, const float* __restrict__ Y, float* w,
+__global__ void __launch_bounds__(256, 4) k_up_f32(const float* v, const float* Y, float* w,
                                                    const float* w_old, int64_t Dup, int64_t Ddn, UpGrid g,
                                                    const int32_t* __restrict__ ptr, const int32_t* __restrict__ npos,
                                                    const uint32_t* __restrict__ list, const uint32_t* __restrict__ su,
@@ -945,14 +945,14 @@ __global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, 
             act[i] = c_raw < Ddn;
             c[i] = act[i] ? c_raw : Ddn - VPL;
             const int64_t J = (r0 + r) * Ddn + c[i];
-            xo[i] = __ldg(reinterpret_cast<const V*>(v + J));
-            yv[i] = __ldcs(reinterpret_cast<const V*>(Y + J));
-            if (w_old != nullptr) wv[i] = __ldcs(reinterpret_cast<const V*>(w_old + J));
+            xo[i] = *(reinterpret_cast<const V*>(v + J));
+            yv[i] = ld_stream(reinterpret_cast<const V*>(Y + J));
+            if (w_old != nullptr) wv[i] = ld_stream(reinterpret_cast<const V*>(w_old + J));
             P[i] = V{};
             N[i] = V{};
         }
         auto load = [&](uint32_t t, int i) {
-            return __ldg(reinterpret_cast<const V*>(reinterpret_cast<const char*>(v + c[i]) + (uint64_t)t * rowb));
+            return *(reinterpret_cast<const V*>(reinterpret_cast<const char*>(v + c[i]) + (uint64_t)t * rowb));
         };
         const int2 np = cnt[r];
         list_hops<true>(L + r * g.W, np.x, np.y, [&](bool neg, const uint32_t* t, auto full, int m) {
@@ -999,13 +999,13 @@ __global__ void __launch_bounds__(256, 4) k_up_f32(const float* __restrict__ v, 
 // binary32 variants: same structure, float arithmetic (UPD: the deferred
 // Lanczos update, rounded as k_axpy_scale_f32)
 template <int VEC, typename EntT, bool UPD>
-__global__ void __launch_bounds__(1024, 1) k_rows_f32(std::conditional_t<UPD, float*, const float*> __restrict__ v,
+__global__ void __launch_bounds__(1024, 1) k_rows_f32(std::conditional_t<UPD, float*, const float*> v,
                                                     float* __restrict__ Y, int64_t Dup,
                                                     int64_t Ddn, const int64_t* __restrict__ boff,
                                                     const int32_t* __restrict__ bcnt,
                                                     const EntT* __restrict__ ent,
-                                                    const float* __restrict__ fo, float ua, float uinv,
-                                                    const LzDev* __restrict__ dv) {
+                                                    const float* fo, float ua, float uinv,
+                                                    const LzDev* dv) {
     using S = typename F32Vec<VEC>::T;
     grid_dep_wait();
     if constexpr (UPD) {

@@ -203,10 +203,51 @@ inline cudaError_t launch_on(bool pdl, void (*kern)(KArgs...), int grid, int thr
 }
 #ifdef __CUDACC__
 // the kernel before this one on the stream has finished; and the next may begin
-// to take its places (both before any access to what kernels write)
+// to take its places (both before any access to what kernels write).  The kernel
+// before may be writing while this one is already resident, so what kernels write
+// (vectors, X and Y, exponent words, LzDev) is read by plain loads or ld_stream
+// after the wait, never through __ldg or a const __restrict__ pointer: those
+// promise data that does not change while the kernel lives.  Tables do not.
 __device__ __forceinline__ void grid_dep_wait() {
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+// loads of streamed data (evicted first), kept behind grid_dep_wait
+__device__ __forceinline__ double ld_stream(const double* p) {
+    double v;
+    asm volatile("ld.global.cs.f64 %0, [%1];" : "=d"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ double2 ld_stream(const double2* p) {
+    double2 v;
+    asm volatile("ld.global.cs.v2.f64 {%0, %1}, [%2];" : "=d"(v.x), "=d"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ long long ld_stream(const long long* p) {
+    long long v;
+    asm volatile("ld.global.cs.s64 %0, [%1];" : "=l"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ longlong2 ld_stream(const longlong2* p) {
+    longlong2 v;
+    asm volatile("ld.global.cs.v2.s64 {%0, %1}, [%2];" : "=l"(v.x), "=l"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float ld_stream(const float* p) {
+    float v;
+    asm volatile("ld.global.cs.f32 %0, [%1];" : "=f"(v) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float2 ld_stream(const float2* p) {
+    float2 v;
+    asm volatile("ld.global.cs.v2.f32 {%0, %1}, [%2];" : "=f"(v.x), "=f"(v.y) : "l"(p));
+    return v;
+}
+__device__ __forceinline__ float4 ld_stream(const float4* p) {
+    float4 v;
+    asm volatile("ld.global.cs.v4.f32 {%0, %1, %2, %3}, [%4];"
+                 : "=f"(v.x), "=f"(v.y), "=f"(v.z), "=f"(v.w) : "l"(p));
+    return v;
 }
 #endif
 

@@ -94,7 +94,7 @@ __global__ void k_max_exponent(const double* __restrict__ v, int64_t n, int* ema
     if ((threadIdx.x & 31) == 0 && m > 0) atomicMax(emax, m);
 }
 // -> slots[blockIdx.x], every CTA its own
-__global__ void k_max_exponent_slots(const double* __restrict__ v, int64_t n, int* slots) {
+__global__ void k_max_exponent_slots(const double* v, int64_t n, int* slots) {
     grid_dep_wait();
     __shared__ int ws[kThreads / 32];
     const int m = warp_max_exponent(v, n);
