@@ -273,10 +273,13 @@ int hubbard_lanczos_step(hubbard_t H, const void* f, void* g, double beta_j, int
  *              aligned, not overlapping the workspace) receiving the
  *              normalised Ritz vector psi = sum_j s_j f_j of the lowest Ritz
  *              value.  The Lanczos vectors the first pass could keep are
- *              combined in one pass: up to 1 GiB of them, taken for the call
- *              from a pool of the library's own that holds at most as much
- *              between calls (none where there is no room, or above 2.5e7
- *              elements).  The rest is replayed: the same recurrence with the
+ *              combined in one pass: up to 1 GiB of them over all calls that
+ *              run on the device, taken for the call from a pool of the
+ *              library's own (none where there is no room, or above 2.5e7
+ *              elements).  The pool keeps that memory between calls; it goes
+ *              back to the device with the device's last handle, and when an
+ *              allocation of the library finds none.  The vectors that were
+ *              not kept are replayed: the same recurrence with the
  *              recorded a_j, b_j (the kernels are deterministic, so the
  *              replayed f_j are the ones of the first pass), accumulated in
  *              j order in binary64, so psi is the same however many were

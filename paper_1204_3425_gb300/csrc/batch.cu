@@ -1503,7 +1503,7 @@ int hubbard_selftest_wait_timeout(void* stream) {
     clear_error();
     cudaStream_t s = (cudaStream_t)stream;
     char* buf = nullptr;
-    HUB_CUDA(cudaMalloc((void**)&buf, 256));
+    HUB_CUDA(dev_alloc((void**)&buf, 256));
     int err = 0;
     cudaError_t e = cudaMemsetAsync(buf, 0, 256, s);
     if (e == cudaSuccess) {
@@ -1757,7 +1757,7 @@ int pool_append(T** pool, size_t* used, size_t* capn, const T* src, size_t n, cu
     if (start + n > *capn) {
         size_t nc = std::max<size_t>(*capn * 2, start + n + align);
         T* np = nullptr;
-        if (cudaMalloc((void**)&np, nc * sizeof(T)) != cudaSuccess) return fail(HUB_ENOMEM, "queue table pool");
+        if (dev_alloc((void**)&np, nc * sizeof(T)) != cudaSuccess) return fail(HUB_ENOMEM, "queue table pool");
         if (*used > 0) HUB_CUDA(cudaMemcpyAsync(np, *pool, *used * sizeof(T), cudaMemcpyDeviceToDevice, s));
         HUB_CUDA(cudaStreamSynchronize(s));
         cudaFree(*pool);
@@ -2058,13 +2058,13 @@ int hubbard_queue_create(int capacity, int64_t max_dim, int max_iters, double to
     cudaError_t e = cudaStreamCreateWithFlags(&Q->cstream, cudaStreamNonBlocking);
     for (int w = 0; w < hubbard_queue::kWorkers && e == cudaSuccess; ++w)
         e = cudaStreamCreateWithFlags(&Q->ks[w], cudaStreamNonBlocking);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_sec, (size_t)capacity * sizeof(SectorDesc));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_f, nv * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_g, nv * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_xg, nv * sizeof(int2));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_ab, (size_t)capacity * 2 * max_iters * sizeof(double));
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_err, 256);
-    if (e == cudaSuccess) e = cudaMalloc((void**)&Q->d_claim, 256);
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_sec, (size_t)capacity * sizeof(SectorDesc));
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_f, nv * sizeof(double));
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_g, nv * sizeof(double));
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_xg, nv * sizeof(int2));
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_ab, (size_t)capacity * 2 * max_iters * sizeof(double));
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_err, 256);
+    if (e == cudaSuccess) e = dev_alloc((void**)&Q->d_claim, 256);
     if (e == cudaSuccess) e = cudaMemset(Q->d_err, 0, 256);
     if (e == cudaSuccess) e = cudaMemset(Q->d_claim, 0, 256);
     if (e == cudaSuccess) e = cudaHostAlloc((void**)&Q->h_ctl, 256, cudaHostAllocMapped);
@@ -2086,12 +2086,12 @@ int hubbard_queue_create(int capacity, int64_t max_dim, int max_iters, double to
         Q->c_bo = (size_t)1 << 18;
         Q->c_bc = (size_t)1 << 18;
         Q->c_be = (size_t)4 << 20;
-        cudaError_t e2 = cudaMalloc((void**)&Q->d_rp, Q->c_rp * sizeof(int32_t));
-        if (e2 == cudaSuccess) e2 = cudaMalloc((void**)&Q->d_ent, Q->c_ent * sizeof(uint32_t));
-        if (e2 == cudaSuccess) e2 = cudaMalloc((void**)&Q->d_st, Q->c_st * sizeof(uint32_t));
-        if (e2 == cudaSuccess) e2 = cudaMalloc((void**)&Q->d_bo, Q->c_bo * sizeof(int64_t));
-        if (e2 == cudaSuccess) e2 = cudaMalloc((void**)&Q->d_bc, Q->c_bc * sizeof(int32_t));
-        if (e2 == cudaSuccess) e2 = cudaMalloc((void**)&Q->d_be, Q->c_be * sizeof(uint16_t));
+        cudaError_t e2 = dev_alloc((void**)&Q->d_rp, Q->c_rp * sizeof(int32_t));
+        if (e2 == cudaSuccess) e2 = dev_alloc((void**)&Q->d_ent, Q->c_ent * sizeof(uint32_t));
+        if (e2 == cudaSuccess) e2 = dev_alloc((void**)&Q->d_st, Q->c_st * sizeof(uint32_t));
+        if (e2 == cudaSuccess) e2 = dev_alloc((void**)&Q->d_bo, Q->c_bo * sizeof(int64_t));
+        if (e2 == cudaSuccess) e2 = dev_alloc((void**)&Q->d_bc, Q->c_bc * sizeof(int32_t));
+        if (e2 == cudaSuccess) e2 = dev_alloc((void**)&Q->d_be, Q->c_be * sizeof(uint16_t));
         if (e2 != cudaSuccess) {
             queue_free(Q);
             return cuda_fail(e2, "queue table pools");

@@ -60,7 +60,7 @@ template <typename T>
 int upload(T** dst, const T* src, size_t n) {
     *dst = nullptr;
     size_t bytes = std::max<size_t>(n, 1) * sizeof(T);
-    cudaError_t e = cudaMalloc((void**)dst, bytes);
+    cudaError_t e = dev_alloc((void**)dst, bytes);
     if (e != cudaSuccess) return cuda_fail(e, "cudaMalloc(tables)");
     if (n > 0) HUB_CUDA(cudaMemcpy(*dst, src, n * sizeof(T), cudaMemcpyHostToDevice));
     return HUB_OK;
@@ -174,7 +174,87 @@ void lz_host_return(LzHost* p) {
     lz_host_delete(p);
 }
 
+// Device memory for Lanczos vectors a call keeps beside its workspace, one pool
+// per device, safe across threads and streams.  All calls together hold at most
+// kStoreBytes of it and the pool keeps no more than that between calls; it is
+// given back to the device when the device's last handle is destroyed, and when an
+// allocation of the library finds no memory.
+constexpr size_t kStoreBytes = 1ull << 30;
+constexpr int kStoreDevices = 64;
+struct StorePool {
+    cudaMemPool_t pool = nullptr;
+    size_t used = 0;                           // bytes of the calls that run now
+    int handles = 0;
+};
+std::mutex g_store_mu;
+StorePool g_store[kStoreDevices];
+
+// cap in: vectors wanted; out: vectors there is room for (nullptr below least)
+void* store_take(int device, size_t stride, int least, int* cap, cudaStream_t s) {
+    if (device < 0 || device >= kStoreDevices) return nullptr;
+    std::lock_guard<std::mutex> lk(g_store_mu);
+    StorePool& S = g_store[device];
+    if (S.pool == nullptr) {
+        cudaMemPoolProps props{};
+        props.allocType = cudaMemAllocationTypePinned;
+        props.location.type = cudaMemLocationTypeDevice;
+        props.location.id = device;
+        uint64_t keep = kStoreBytes;
+        if (cudaMemPoolCreate(&S.pool, &props) != cudaSuccess) S.pool = nullptr;
+        else if (cudaMemPoolSetAttribute(S.pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
+            cudaMemPoolDestroy(S.pool);
+            S.pool = nullptr;
+        }
+        if (S.pool == nullptr) {
+            cudaGetLastError();
+            return nullptr;
+        }
+    }
+    *cap = (int)std::min<size_t>((size_t)*cap, (kStoreBytes - S.used) / stride);
+    if (*cap < least) return nullptr;
+    const size_t bytes = (size_t)*cap * stride;
+    // what is kept but too small goes first, so that kept and used stay in the bound
+    uint64_t res = 0, cur = 0;
+    if (cudaMemPoolGetAttribute(S.pool, cudaMemPoolAttrReservedMemCurrent, &res) == cudaSuccess &&
+        cudaMemPoolGetAttribute(S.pool, cudaMemPoolAttrUsedMemCurrent, &cur) == cudaSuccess && res < cur + bytes)
+        cudaMemPoolTrimTo(S.pool, cur);
+    void* p = nullptr;
+    if (cudaMallocFromPoolAsync(&p, bytes, S.pool, s) != cudaSuccess) {
+        cudaGetLastError();
+        return nullptr;
+    }
+    S.used += bytes;
+    return p;
+}
+
+void store_return(int device, void* p, size_t bytes, cudaStream_t s) {
+    std::lock_guard<std::mutex> lk(g_store_mu);
+    cudaFreeAsync(p, s);
+    g_store[device].used -= bytes;
+}
+
+// handles of the device: +1 made, -1 destroyed (the last gives the pool's memory back)
+void store_handles(int device, int d) {
+    if (device < 0 || device >= kStoreDevices) return;
+    std::lock_guard<std::mutex> lk(g_store_mu);
+    StorePool& S = g_store[device];
+    S.handles += d;
+    if (S.handles == 0 && S.pool != nullptr && cudaMemPoolTrimTo(S.pool, 0) != cudaSuccess) cudaGetLastError();
+}
+
+bool store_give_back() {
+    int dev = 0;
+    if (cudaGetDevice(&dev) != cudaSuccess || dev >= kStoreDevices) return false;
+    std::lock_guard<std::mutex> lk(g_store_mu);
+    uint64_t a = 0, b = 0;
+    cudaMemPool_t pool = g_store[dev].pool;
+    return pool != nullptr && cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &a) == cudaSuccess &&
+           cudaMemPoolTrimTo(pool, 0) == cudaSuccess &&
+           cudaMemPoolGetAttribute(pool, cudaMemPoolAttrReservedMemCurrent, &b) == cudaSuccess && b < a;
+}
+
 void free_dev(hubbard_sector* H) {
+    store_handles(H->device, -1);
     host_pipe_free(H);
     lz_host_return(H->lz_host);                // no run is in flight: every run ends with its stream synchronised
     H->lz_host = nullptr;
@@ -584,6 +664,15 @@ int hubbard_sector_create(int Ns, const int32_t* bonds, int n_bonds, int Nup, in
 
 }  // extern "C"
 
+cudaError_t hub::dev_alloc(void** p, size_t bytes, cudaStream_t ms) {
+    cudaError_t e = ms ? cudaMallocAsync(p, bytes, ms) : cudaMalloc(p, bytes);
+    if (e == cudaErrorMemoryAllocation && store_give_back()) {
+        cudaGetLastError();
+        e = ms ? cudaMallocAsync(p, bytes, ms) : cudaMalloc(p, bytes);
+    }
+    return e;
+}
+
 int hub::sector_create_streamed(int Ns, const int32_t* bonds, int n_bonds, int Nup, int Ndn, double t, double U,
                                 cudaStream_t ms, hubbard_t* out) {
     clear_error();
@@ -600,6 +689,7 @@ int hub::sector_create_streamed(int Ns, const int32_t* bonds, int n_bonds, int N
         delete H;
         return fail(HUB_ECUDA, "no CUDA device");
     }
+    store_handles(H->device, 1);
     H->mem_stream = ms;
     H->ns = Ns;
     H->nup = Nup;
@@ -737,8 +827,8 @@ int hubbard_apply_host(hubbard_t H, const void* v_host, void* w_host, int dtype,
         for (int k = 0; k < 2 && e == cudaSuccess; ++k) {
             for (cudaEvent_t* ev : {&P->uploaded[k], &P->computed[k], &P->downloaded[k]})
                 if (e == cudaSuccess) e = cudaEventCreateWithFlags(ev, cudaEventDisableTiming);
-            if (e == cudaSuccess) e = cudaMalloc(&P->v[k], std::max<size_t>(bytes, 256));
-            if (e == cudaSuccess) e = cudaMalloc(&P->w[k], std::max<size_t>(bytes, 256));
+            if (e == cudaSuccess) e = dev_alloc(&P->v[k], std::max<size_t>(bytes, 256));
+            if (e == cudaSuccess) e = dev_alloc(&P->w[k], std::max<size_t>(bytes, 256));
         }
         if (e != cudaSuccess) {
             host_pipe_free(H);
@@ -867,7 +957,7 @@ static double* reduction_scratch() {
     cudaGetDevice(&cur);
     if (p == nullptr || dev != cur) {
         p = nullptr;
-        if (cudaMalloc((void**)&p, kRedSlots * sizeof(double)) != cudaSuccess) p = nullptr;
+        if (dev_alloc((void**)&p, kRedSlots * sizeof(double)) != cudaSuccess) p = nullptr;
         dev = cur;
     }
     return p;
@@ -1319,56 +1409,28 @@ static int ritz_vector(hubbard_t H, const void* v0, int v0_dtype, int dtype, con
 
 // Room for the Lanczos vectors of one lanczos_ground_state call that wants a
 // Ritz vector: replaying the recurrence doubles the H*v count, the stored
-// vectors are one pass.  Taken for the call from a pool of the library's own on
-// the call's stream (one pool per device, safe across threads and streams), at
-// most kStoreBytes; the pool keeps at most that much between calls.  nullptr
-// when there is no room: the recurrence is then replayed.
-constexpr size_t kStoreBytes = 1ull << 30;
+// vectors are one pass.  What the device's pool (StorePool) still has, at most
+// kStoreBytes; none where there is no room: the recurrence is then replayed.
 constexpr int kStoreMin = 8;                         // fewer vectors save less than they take
-
-static cudaMemPool_t store_pool(int device) {
-    static std::mutex mu;
-    static std::map<int, cudaMemPool_t> pools;
-    std::lock_guard<std::mutex> lk(mu);
-    auto it = pools.find(device);
-    if (it != pools.end()) return it->second;
-    cudaMemPoolProps props{};
-    props.allocType = cudaMemAllocationTypePinned;
-    props.location.type = cudaMemLocationTypeDevice;
-    props.location.id = device;
-    cudaMemPool_t pool = nullptr;
-    uint64_t keep = kStoreBytes;
-    if (cudaMemPoolCreate(&pool, &props) != cudaSuccess ||
-        cudaMemPoolSetAttribute(pool, cudaMemPoolAttrReleaseThreshold, &keep) != cudaSuccess) {
-        cudaGetLastError();
-        if (pool) cudaMemPoolDestroy(pool);
-        pool = nullptr;
-    }
-    pools[device] = pool;
-    return pool;
-}
 
 struct VectorStore {
     char* p = nullptr;
-    size_t stride = 0;
+    size_t stride = 0, bytes = 0;
     int cap = 0;
+    int device;
     cudaStream_t s;
-    VectorStore(hubbard_t H, int dtype, int steps, cudaStream_t st) : s(st) {
-        stride = align_up((size_t)H->D * elem_size(dtype), 256);
-        const int n = (int)std::min<size_t>((size_t)std::min(steps, kRedSlots), kStoreBytes / stride);
-        if (n < std::min(steps, kStoreMin)) return;
-        cudaMemPool_t pool = store_pool(H->device);
-        if (pool == nullptr || cudaMallocFromPoolAsync((void**)&p, (size_t)n * stride, pool, s) != cudaSuccess) {
-            cudaGetLastError();
-            p = nullptr;
-            return;
-        }
-        cap = n;
+    VectorStore(int dev, cudaStream_t st) : device(dev), s(st) {}
+    void take(int64_t D, int dtype, int steps) {
+        stride = align_up((size_t)D * elem_size(dtype), 256);
+        cap = (int)std::min<size_t>((size_t)std::min(steps, kRedSlots), kStoreBytes / stride);
+        if (cap >= std::min(steps, kStoreMin)) p = (char*)store_take(device, stride, std::min(steps, kStoreMin), &cap, s);
+        if (p == nullptr) cap = 0;
+        bytes = (size_t)cap * stride;
     }
     VectorStore(const VectorStore&) = delete;
     VectorStore& operator=(const VectorStore&) = delete;
     ~VectorStore() {
-        if (p) cudaFreeAsync(p, s);
+        if (p) store_return(device, p, bytes, s);
     }
 };
 
@@ -1401,12 +1463,10 @@ int lanczos_ground_state(hubbard_t H, const void* v0, int max_iters, double tol,
     LanczosRun R;
     // sectors with device-resident steps keep their vectors for psi where there is room
     const int steps = (int)std::min<int64_t>(max_iters, H->D);
-    std::unique_ptr<VectorStore> kept;
-    if (psi_out != nullptr && !lanczos_host_driven(H, dtype)) kept = std::make_unique<VectorStore>(H, dtype, steps, s);
-    char* store = kept ? kept->p : nullptr;
-    const size_t stride = kept ? kept->stride : 0;
-    const int cap = kept ? kept->cap : 0;
-    if ((rc = lanczos_core(H, v0, dtype, max_iters, tol, dtype, ws, ws + vec, s, R, 0.0, store, stride, cap))) return rc;
+    VectorStore kept(H->device, s);
+    if (psi_out != nullptr && !lanczos_host_driven(H, dtype)) kept.take(H->D, dtype, steps);
+    if ((rc = lanczos_core(H, v0, dtype, max_iters, tol, dtype, ws, ws + vec, s, R, 0.0, kept.p, kept.stride,
+                           kept.cap))) return rc;
     const int m = (int)R.a.size();
     if (alpha_out) std::memcpy(alpha_out, R.a.data(), m * sizeof(double));
     if (beta_out) std::memcpy(beta_out, R.b.data(), m * sizeof(double));
@@ -1415,7 +1475,8 @@ int lanczos_ground_state(hubbard_t H, const void* v0, int max_iters, double tol,
         std::vector<double> sv((size_t)m);
         double th = 0.0;
         tridiag_lowest_vector(R.a.data(), R.b.data(), m, &th, sv.data());
-        if ((rc = ritz_vector(H, v0, dtype, dtype, R, sv, ws, ws + vec, (double*)psi_out, store, stride, cap, s))) return rc;
+        if ((rc = ritz_vector(H, v0, dtype, dtype, R, sv, ws, ws + vec, (double*)psi_out, kept.p, kept.stride,
+                              kept.cap, s))) return rc;
         if (cudaStreamSynchronize(s) != cudaSuccess) return fail(HUB_ECUDA, "lanczos synchronise");
     }
     out->energy = R.theta;

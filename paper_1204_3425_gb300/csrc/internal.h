@@ -22,9 +22,7 @@ int cuda_fail(cudaError_t e, const char* what);
 // uploaded and freed in that stream's order, so releasing it does not wait for
 // the whole device (cudaFree would).  ms == nullptr: cudaMalloc / cudaMemcpy /
 // cudaFree.
-inline cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t ms) {
-    return ms ? cudaMallocAsync(p, bytes, ms) : cudaMalloc(p, bytes);
-}
+cudaError_t dev_alloc(void** p, size_t bytes, cudaStream_t ms = nullptr);
 inline void dev_free(void* p, cudaStream_t ms) {
     if (p == nullptr) return;
     if (ms) cudaFreeAsync(p, ms);

@@ -27,7 +27,8 @@ CASES = [
     ("ring12", 2, 5, 8.0, "f64", 0),       # about as many items as CTAs
     ("ring13", 5, 5, 2.0, "f64", 30),      # odd rows
     ("ring13", 6, 6, 8.0, "f64", 30),      # more than 2.5e6 elements
-    ("ring15", 5, 6, 7.3, "f64", 12),      # the same, odd rows
+    ("ring13", 6, 6, 7.3, "f64", 60),      # the same; 45 vectors kept for psi, 15 replayed
+    ("ring15", 5, 6, 7.3, "f64", 12),      # more than 2.5e6 elements, odd rows
     ("ring18", 2, 9, 7.3, "f64", 12),      # rows staged one word at a time
     ("ring16", 1, 8, 4.0, "f64", 0),       # 16 rows of 12870 elements
     ("ring10", 3, 0, 4.0, "f64", 0),       # one column
@@ -67,7 +68,8 @@ def test_lanczos_scalars_are_the_recorded_ones(case):
 
 
 # binary32 vectors combined in binary64: lattice, N_up, N_dn, U
-PSI_CASES = [("sq3x3", 4, 4, 4.0), ("ring11", 5, 6, 7.3), ("ring12", 6, 6, 4.0)]
+PSI_CASES = [("sq3x3", 4, 4, 4.0), ("ring11", 5, 6, 7.3), ("ring12", 6, 6, 4.0),
+             ("ring14", 7, 7, 4.0)]      # 22 vectors of the plain run kept for psi, 38 replayed
 
 
 def _psi32(lattice, nup, ndn, U, store):
