@@ -127,9 +127,10 @@ struct LzHost {
 
 namespace {
 
-constexpr size_t kLzPool = 64;
+constexpr int kLzPool = 64;
 std::mutex g_lz_mu;
-std::vector<LzHost*> g_lz_pool;
+LzHost* g_lz_pool[kLzPool];                    // the first g_lz_kept are set; an array, so that keeping one cannot throw
+int g_lz_kept = 0;
 
 void lz_host_delete(LzHost* p) {
     if (p->ab[0]) cudaFreeHost(p->ab[0]);
@@ -141,10 +142,10 @@ void lz_host_delete(LzHost* p) {
 LzHost* lz_host_take(int device) {
     {
         std::lock_guard<std::mutex> lk(g_lz_mu);
-        for (size_t i = 0; i < g_lz_pool.size(); ++i)
+        for (int i = 0; i < g_lz_kept; ++i)
             if (g_lz_pool[i]->device == device) {
                 LzHost* p = g_lz_pool[i];
-                g_lz_pool.erase(g_lz_pool.begin() + (ptrdiff_t)i);
+                g_lz_pool[i] = g_lz_pool[--g_lz_kept];
                 return p;
             }
     }
@@ -166,8 +167,8 @@ void lz_host_return(LzHost* p) {
     if (p == nullptr) return;
     {
         std::lock_guard<std::mutex> lk(g_lz_mu);
-        if (g_lz_pool.size() < kLzPool) {
-            g_lz_pool.push_back(p);
+        if (g_lz_kept < kLzPool) {
+            g_lz_pool[g_lz_kept++] = p;
             return;
         }
     }
