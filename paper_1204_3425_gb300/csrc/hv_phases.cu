@@ -1107,6 +1107,9 @@ int sms() {
     return n;
 }
 
+// static shared memory of the binary64 row kernels (cta_exponent)
+constexpr int kRowStatic = 16;
+
 // largest VEC in {4,2,1} (capped by vmax) whose staging buffer (with the
 // zero slots) fits
 int pick_vec(int64_t len, int elem_bytes, int vmax, int reserve) {
@@ -1218,12 +1221,12 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     // epilogue operands need the registers), 5 at <= 51 for binary32 with up
     // to 2 columns per lane; measured best)
     if (dtype == HUB_F64) {
-        const int va = choose_vec(H->vec_rows, Ddn, 8, 2, 0);
+        const int va = choose_vec(H->vec_rows, Ddn, 8, 2, kRowStatic);
         // exponent bound: found by the row phase itself on the smallest sectors, by a
         // pass of its own otherwise.  On sectors that launch overlapped that pass
         // leaves one maximum per CTA, which the row phase reduces: no memset of a
         // word that all CTAs raise breaks the chain of kernels.
-        const bool ysplit = va == 0 && staged_slots(Ddn) * 4 <= smem_optin();
+        const bool ysplit = va == 0 && staged_slots(Ddn) * 4 + kRowStatic <= smem_optin();
         const int scan = fixed_emax <= 0 && w_old == nullptr && va > 0 && H->D <= kScanElems;
         const bool by_slots = fixed_emax <= 0 && w_old == nullptr && pdl && !scan && (va > 0 || ysplit);
         int* emax = H->status;
