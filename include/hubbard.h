@@ -283,7 +283,9 @@ int hubbard_lanczos_step(hubbard_t H, const void* f, void* g, double beta_j, int
  *              recorded a_j, b_j (the kernels are deterministic, so the
  *              replayed f_j are the ones of the first pass), accumulated in
  *              j order in binary64, so psi is the same however many were
- *              kept.  NULL skips it.
+ *              kept.  Its sign makes sum_j s_j positive; where that sum is
+ *              near 0 rounding decides, so a caller who needs a sign fixes one
+ *              (a positive overlap with v0, say).  NULL skips it.
  *   alpha_out, beta_out  optional host arrays of max_iters doubles receiving
  *              a_1..a_m and b_2..b_{m+1}
  *   out        host result: energy (lowest Ritz value), residual rho,

@@ -298,7 +298,8 @@ __device__ __forceinline__ int exp_bits(double x) { return (__double2hiint(x) >>
 // p_k = (a_{k-1} - x) p_{k-1} - b_{k-2}^2 p_{k-2} (Sturm sequence).  No division;
 // both terms are rescaled by 2^-600 / 2^600 when they leave a safe range, tested
 // every fourth step while every entry is below 2^50 in magnitude (a step then
-// grows them at most 2^102 times), every step otherwise.  Signs and magnitudes
+// grows them at most 2^102 times; two steps shrink them at most by b^2, and a run
+// ends at b <= 1e-13), every step otherwise.  Signs and magnitudes
 // are read from the bits.  A zero p_k takes the sign of p_{k-1}.
 __device__ __noinline__ int warp_sturm(const double* a, const double* b, int m, double x, bool large) {
     double p0 = 1.0, p1 = a[0] - x;

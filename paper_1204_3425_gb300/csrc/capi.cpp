@@ -1699,7 +1699,7 @@ static int lanczos_core_in_store(hubbard_t H, const void* v0, int slots, char* s
 
 // A <- A + sum_j ca_j f_j, B <- B + sum_j cb_j f_j over the Lanczos vectors of a
 // finished lanczos_core run from p, by replaying its recurrence as
-// replay_ritz_vector does (same kernels and operands, hence the same f_j bit
+// ritz_vector does (same kernels and operands, hence the same f_j bit
 // for bit); the accumulation is the one launch_combine2_f64 does over stored
 // vectors, so both routes give the same A, B.
 static int replay_combine2(hubbard_t H, const void* p, const LanczosRun& R, const std::vector<double>& ca,

@@ -179,8 +179,11 @@ __device__ __forceinline__ void sub4(int2& A, int2 a) { A.x -= a.x; A.y -= a.y; 
 // thread accumulates <w, f>, <w, w> and <f, f> over its outputs in a fixed
 // order, the CTA sums its threads, and the last CTA the per-CTA partials
 // (part[b], part[kPartStride + b], part[2 kPartStride + b]), in fixed trees, so
-// the result is deterministic.  binary32 outputs use a float-float accumulator
-// (exact product split + TwoSum), as the stand-alone dot kernel does.
+// the result is deterministic.  binary32 outputs, like the stand-alone dot
+// kernels, use a float-float accumulator: each product is split exactly (p + e
+// with e = fma(x, y, -p)) and added with Knuth's TwoSum, so the FP32 pipe carries
+// some 48 bits and the binary64 pipe (two lanes a clock) is touched once per
+// thread, not per element.
 struct FFAcc {
     float hi = 0.0f, lo = 0.0f;
     __device__ __forceinline__ void add_product(float x, float y) {

@@ -180,7 +180,7 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
 }
 
 // Row phase for binary64 rows of which only one 4-byte word per element fits in
-// shared memory (28672 < D_dn <= 58000): the (lo, hi) words are staged and summed
+// shared memory (29024 < D_dn <= 58080 with 227 KB to a CTA): the (lo, hi) words are staged and summed
 // apart.  A plane is one word of one row; the 2 Dup planes, split into groups of
 // 32 columns, are dealt to the CTAs in equal contiguous ranges, so a few long
 // rows still fill the device evenly (153 rows of 48620 elements are two waves of
@@ -473,7 +473,8 @@ __global__ void __launch_bounds__(256, CT) k_up_f64x(const int2* X, const long l
 // dealt to the CTAs in turn, thread (warp, lane) of a CTA taking rows warp and
 // warp + 8 of an item and columns lane * VPL + j.  The step's sums are over a
 // thread's elements in that order (then block_sum3_store), so this division is
-// part of the result: a schedule may not change it.
+// part of the result, in the last bits of a_j and b_{j+1}: it follows the row
+// length, the SMs and a vec_cols that the caller sets, and nothing else.
 constexpr int kUpRows = 16;
 // CTAs an SM of the step kernels: their grids, and with them the partials, are at
 // most so many times the SMs
@@ -1216,10 +1217,9 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     unsigned* done = reinterpret_cast<unsigned*>(H->status + 2);   // of the step kernels alone
     const bool pdl = H->D * (dtype == HUB_F64 ? 8 : 4) <= kPdlBytes;
     // up-phase CTAs: as many as the launch bounds keep resident (the phase is
-    // bound by L2 latency, so occupancy is what counts: 4 per SM at <= 64
-    // registers for binary64 (3 for the Lanczos variant, whose prefetched
-    // epilogue operands need the registers), 5 at <= 51 for binary32 with up
-    // to 2 columns per lane; measured best)
+    // bound by L2 latency, so occupancy is what counts): 4 per SM at <= 64
+    // registers, 3 where binary64 requests its epilogue's operands before the
+    // gathers (the Lanczos step, replayed steps, pre below)
     if (dtype == HUB_F64) {
         const int va = choose_vec(H->vec_rows, Ddn, 8, 2, kRowStatic);
         // exponent bound: found by the row phase itself on the smallest sectors, by a

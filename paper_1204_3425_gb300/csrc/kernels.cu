@@ -202,23 +202,6 @@ __device__ __forceinline__ double block_sum(double s) {
     return s;
 }
 
-// Per-thread float-float accumulator for binary32 vectors: each product x*y
-// is split exactly (p + e with e = fma(x, y, -p)) and added with Knuth's
-// TwoSum, so the FP32 pipe carries ~48 bits and the binary64 pipe (1.7
-// op/clk/SM here) is touched once per thread, not per element.
-struct FF {
-    float hi = 0.0f, lo = 0.0f;
-    __device__ __forceinline__ void add_product(float x, float y) {
-        const float p = x * y;
-        const float e = fmaf(x, y, -p);
-        const float s = hi + p;
-        const float bb = s - hi;
-        lo += ((hi - (s - bb)) + (p - bb)) + e;
-        hi = s;
-    }
-    __device__ __forceinline__ double value() const { return (double)hi + (double)lo; }
-};
-
 __global__ void k_dot_f64(const double* __restrict__ x, const double* __restrict__ y, int64_t n, double* partials) {
     double s = 0.0;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
@@ -228,7 +211,7 @@ __global__ void k_dot_f64(const double* __restrict__ x, const double* __restrict
 }
 
 __global__ void k_dot_f32(const float* __restrict__ x, const float* __restrict__ y, int64_t n, double* partials) {
-    FF acc;
+    FFAcc acc;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
         acc.add_product(x[i], y[i]);
     const double s = block_sum(acc.value());
@@ -250,7 +233,7 @@ __global__ void k_axpy_nrm2_f64(double a, const double* __restrict__ x, double* 
 
 __global__ void k_axpy_nrm2_f32(float a, const float* __restrict__ x, float* __restrict__ y, int64_t n,
                                 double* partials) {
-    FF acc;
+    FFAcc acc;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float r = fmaf(a, x[i], y[i]);
         y[i] = r;
@@ -313,7 +296,7 @@ __global__ void k_lz_axpy_nrm2_f32(const LzDev* __restrict__ dv, const float* __
                                    int64_t n, double* partials) {
     if (dv->fused) return;
     const float a = (float)(-dv->a);
-    FF acc;
+    FFAcc acc;
     for (int64_t i = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x) {
         const float r = fmaf(a, x[i], y[i]);
         y[i] = r;
