@@ -180,8 +180,8 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
 }
 
 // Row phase for binary64 rows of which only one 4-byte word per element fits in
-// shared memory (29024 < D_dn <= 58080 with 227 KB to a CTA): the (lo, hi) words are staged and summed
-// apart.  A plane is one word of one row; the 2 Dup planes, split into groups of
+// shared memory (29024 < D_dn <= 58080 with 227 KB to a CTA), of vectors that stay
+// in L2: the (lo, hi) words are staged and summed apart.  A plane is one word of one row; the 2 Dup planes, split into groups of
 // 32 columns, are dealt to the CTAs in equal contiguous ranges, so a few long
 // rows still fill the device evenly (153 rows of 48620 elements are two waves of
 // one row per SM).  A gather from L2 fetched a 32-byte sector at L2 latency for
@@ -189,7 +189,9 @@ __global__ void __launch_bounds__(1024, 1) k_rows_f64x(std::conditional_t<UPD, d
 // product 304 -> 236 us).  The CTA that begins a row's lo plane also writes its
 // fixed-point copy X.  Ys holds the two word sums of an element side by side and
 // the up phase joins them: joined here, each CTA would stage both words of two
-// rows instead of three planes (259 us).
+// rows instead of three planes (259 us).  On HBM-sized vectors one CTA an SM stages
+// and sums in turn and the gathers of k_rows_global_f64x overlap better (816 x 43758
+// elements: product 0.89 ms with planes, 0.85 without; 1140 x 38760: 1.23, 0.98).
 template <typename EntT>
 __global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* v, int* __restrict__ Ys,
                                                             int2* __restrict__ Xg, int64_t Dup, int64_t Ddn,
@@ -247,7 +249,8 @@ __global__ void __launch_bounds__(1024, 1) k_rows_planes_f64x(const double* v, i
     }
 }
 
-// Row phase for binary64 rows too long for shared memory: the fixed-point
+// Row phase for binary64 rows too long for shared memory (by the word, or whole on
+// HBM-sized vectors): the fixed-point
 // copy X is already in global memory (k_to_fixed) and the down-hop gathers
 // read row u of it through L1/L2.
 template <typename EntT>
@@ -1226,7 +1229,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
         // pass of its own otherwise.  On sectors that launch overlapped that pass
         // leaves one maximum per CTA, which the row phase reduces: no memset of a
         // word that all CTAs raise breaks the chain of kernels.
-        const bool ysplit = va == 0 && staged_slots(Ddn) * 4 + kRowStatic <= smem_optin();
+        const bool ysplit = va == 0 && H->D * 8 <= kPdlBytes && staged_slots(Ddn) * 4 + kRowStatic <= smem_optin();
         const int scan = fixed_emax <= 0 && w_old == nullptr && va > 0 && H->D <= kScanElems;
         const bool by_slots = fixed_emax <= 0 && w_old == nullptr && pdl && !scan && (va > 0 || ysplit);
         int* emax = H->status;
@@ -1266,7 +1269,7 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
             if (dn16) { PLANES64(uint16_t, dn.ent16); } else { PLANES64(uint32_t, dn.ent32); }
 #undef PLANES64
         } else if (va == 0) {
-            // longer rows still: fixed-point copy first, then gathers through L1/L2
+            // fixed-point copy first, then gathers through L1/L2
             int* em = emax;
             int* fixed_word = H->status + 1;
             if (fixed_emax > 0) {

@@ -16,7 +16,7 @@ pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(),
     ("ring13", 6, 6, 8.0),     # more than 2.5e6 elements
     ("ring15", 6, 5, 2.0),     # the same, odd rows
     ("ring18", 1, 9, 7.3),     # 48620 columns: two words an element
-    ("ring18", 3, 8, 4.0),     # 43758 columns, 816 rows
+    ("ring18", 3, 8, 4.0),     # 43758 columns, 816 rows: gathered from L2
     ("ring16", 0, 8, 4.0),     # one row
     ("ring16", 8, 0, 4.0),     # one column
 ])
@@ -39,13 +39,16 @@ def test_step_forms_match_the_reference_kernel(lattice, nup, ndn, U, dtype):
     beta = 1.75
     r = torch.empty_like(f)
     hub.hubbard_apply_reference(H, f, r)
+    w = torch.empty_like(f)
+    hub.hubbard_apply(H, f, w)                          # and the product of the same sector
+    eps = 2.4e-12 if dtype == "f64" else 2 * 50 * 2.0 ** -24 * max(1.0, U * min(nup, ndn))
+    assert float((w.double() - r.double()).abs().max()) <= eps * float(f.abs().max())
     w = r.double() - beta * g.double()
     f64 = f.double()
     a = float(w @ f64)
     w -= a * f64
     b = float(w.norm())
     size = max(float(f.abs().max()), beta * float(g.abs().max()))
-    eps = 2.4e-12 if dtype == "f64" else 2 * 50 * 2.0 ** -24 * max(1.0, U * min(nup, ndn))
     a1, b2 = hub.hubbard_lanczos_step(H, f, g, beta)
     assert abs(a1 - a) <= eps * max(1.0, abs(a)) and abs(b2 - b) <= eps * max(1.0, b)
     assert float((g.double() - w / b).abs().max()) <= 3 * eps * size * max(1.0, 1.0 / b)
