@@ -487,7 +487,10 @@ constexpr int kStepCtas64 = 3, kStepCtas32 = 4;
 // W = H f - beta w_old and, per CTA, the partials of <W, f>, <W, W> and
 // <f, f>, closed by the last CTA.  Its epilogue streams four arrays (own element,
 // Y, w_old, f), whose loads are issued before the gathers; the extra live
-// registers cost one CTA per SM (3 instead of 4).  YS: Y holds word pairs
+// registers cost one CTA per SM (3 instead of 4).  Items, rows and the row pitch
+// are 32-bit, and T A is always the 128-bit multiply: with 64-bit ones and mac_t's
+// two forms the 128-bit epilogue spilled (4x4 (8,8), U = 7.3: step 6.18 -> 5.28 ms,
+// U = 8: 5.01 -> 5.00).  YS: Y holds word pairs
 // (k_rows_planes_f64x).
 // NT = 512: a sector of no more items than SMs, one item a CTA and one row a
 // warp; warps 8-15 continue the sums of warps 0-7, in the order above, so a CTA
@@ -516,8 +519,8 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
     const int k = 1070 - emax;
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     constexpr int nw = NT / 32, CC = 32 * VPL;
-    const int64_t nchunk = (Ddn + CC - 1) / CC;
-    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
+    const int nchunk = (int)((Ddn + CC - 1) / CC), nrb = (int)((Dup + kUpRows - 1) / kUpRows);
+    const uint32_t rowb = (uint32_t)Ddn * 8u;             // bytes of a row (Ddn <= kMaxRow)
     double s1 = 0.0, s2 = 0.0, s3 = 0.0;
     double r[VPL], fj[VPL];                               // this thread's elements of a row
     bool have = false;                                    // NT = 512: r, fj hold its only row
@@ -530,25 +533,25 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
         }
     };
     // item = chunk * nrb + rb, advanced by gridDim.x without division
-    int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
-    const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
+    int chunk = (int)blockIdx.x / nrb, rb = (int)blockIdx.x % nrb;
+    const int dch = (int)gridDim.x / nrb, drb = (int)gridDim.x % nrb;
     for (; chunk < nchunk; chunk += dch, rb += drb) {
         if (rb >= nrb) {
             rb -= nrb;
             ++chunk;
             if (chunk >= nchunk) break;
         }
-        const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
-        const bool act = c_raw < Ddn;
-        const int64_t c = act ? c_raw : Ddn - VPL;     // tail lanes read a valid column, store nothing
+        const int c_raw = chunk * CC + lane * VPL;
+        const bool act = c_raw < (int)Ddn;
+        const int c = act ? c_raw : (int)Ddn - VPL;     // tail lanes read a valid column, store nothing
         uint32_t sdc[VPL];
 #pragma unroll
         for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
-        const int2* base = X + c;
-        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
-        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
+        const char* base = reinterpret_cast<const char*>(X + c);
+        const int uend = min(rb * kUpRows + kUpRows, (int)Dup);
+        for (int u = rb * kUpRows + warp; u < uend; u += nw) {
             const int32_t kb = ptr[u];
-            const int64_t J = u * Ddn + c;
+            const int64_t J = (int64_t)u * (int)Ddn + c;
             // streamed operands of the epilogue, requested before the gathers
             double wv[VPL];
             long long yv[VPL];
@@ -569,7 +572,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
             }
             IV A{};
             uniform_hops<IV, TAIL>(list, kb, ptr[u + 1] - kb, npos[u], lane,
-                [&](uint32_t t) { return *(reinterpret_cast<const IV*>(base + (int64_t)t * Ddn)); },
+                [&](uint32_t t) { return *(reinterpret_cast<const IV*>(base + (uint64_t)t * rowb)); },
                 AddFixed<IV>{A});
             if (!act) continue;
             const uint32_t su_u = su[u];
@@ -592,7 +595,7 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
                     if (w_old != nullptr) r[j] = fma(mbeta, wv[j], r[j]);
                 } else {
                     I128 acc{0ull, 0ll};
-                    mac_t(acc, T, ep);
+                    mac128(acc, T, ep.A);
                     mac128(acc, fx_join(xo.x, xo.y), Bs[nd]);
                     if (w_old != nullptr) {
                         int glo, ghi;
