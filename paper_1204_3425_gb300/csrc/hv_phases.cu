@@ -482,6 +482,7 @@ constexpr int kUpRows = 16;
 // CTAs an SM of the step kernels: their grids, and with them the partials, are at
 // most so many times the SMs
 constexpr int kStepCtas64 = 3, kStepCtas32 = 4;
+constexpr int up32_ctas(int vpl, bool red) { return red || vpl == 4 ? kStepCtas32 : 5; }
 
 // Lanczos-step variant of k_up_f64x (Algorithm 1 fused with Algorithms 2, 4):
 // W = H f - beta w_old and, per CTA, the partials of <W, f>, <W, W> and
@@ -635,8 +636,10 @@ __global__ void __launch_bounds__(NT, NT == 512 ? 1 : kStepCtas64) k_up_step_f64
 // Lanczos-step variant of the binary32 up phase, items and sums as above.  What is
 // left of a hop list is requested at once on every size (4x4 (8,8) step 2.75 ->
 // 2.62 ms, ring 14 (7,7) 162 -> 146 us).
-template <int VPL>
-__global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* v, const float* Y, float* w,
+// RED false: a product or a replayed step that does not take resident rows
+// (up_items32).
+template <int VPL, bool RED>
+__global__ void __launch_bounds__(256, up32_ctas(VPL, RED)) k_up_step_f32(const float* v, const float* Y, float* w,
                                                         const float* w_old, int64_t Dup, int64_t Ddn,
                                                         const int32_t* __restrict__ ptr,
                                                         const int32_t* __restrict__ npos,
@@ -646,7 +649,6 @@ __global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* v
                                                         double* part, unsigned* done, LzDev* dv, double* hist) {
     grid_dep_wait();
     if (dv != nullptr && dv->stall) return;
-    __shared__ double red[kSumSlots];
     FFAcc s1, s2, s3;
     if (dv != nullptr) mbeta = (float)-dv->beta;          // device-resident step: beta_j on the device
     using V = typename F32Vec<VPL>::T;
@@ -694,16 +696,21 @@ __global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* v
             if constexpr (VPL == 4) __stcs(reinterpret_cast<float4*>(w + J), make_float4(r[0], r[1], r[2], r[3]));
             else if constexpr (VPL == 2) __stcs(reinterpret_cast<float2*>(w + J), make_float2(r[0], r[1]));
             else __stcs(w + J, r[0]);
+            if constexpr (RED) {
 #pragma unroll
-            for (int j = 0; j < VPL; ++j) {
-                s1.add_product(r[j], comp(xo, j));
-                s2.add_product(r[j], r[j]);
-                s3.add_product(comp(xo, j), comp(xo, j));
+                for (int j = 0; j < VPL; ++j) {
+                    s1.add_product(r[j], comp(xo, j));
+                    s2.add_product(r[j], r[j]);
+                    s3.add_product(comp(xo, j), comp(xo, j));
+                }
             }
         }
     }
-    block_sum3_store(s1.value(), s2.value(), s3.value(), part, red, threadIdx.x);
-    close_sums3(part, gridDim.x, done, dv, hist, red);
+    if constexpr (RED) {
+        __shared__ double red[kSumSlots];
+        block_sum3_store(s1.value(), s2.value(), s3.value(), part, red, threadIdx.x);
+        close_sums3(part, gridDim.x, done, dv, hist, red);
+    }
 }
 
 // Up phase with resident rows: a warp builds one row segment of 32 * VPL * NV
@@ -711,7 +718,7 @@ __global__ void __launch_bounds__(256, kStepCtas32) k_up_step_f32(const float* v
 //
 // CTA (i, j) of the grid owns row range i and the column chunks j, j + gy, ...;
 // its rows' hop lists are staged in shared memory once and serve every chunk
-// (a range whose lists do not fit goes in blocks, staged again for each chunk).
+// (a range whose lists do not fit goes in blocks).
 // All CTAs sweep the chunks in the same order, so the chunk of X that the rows
 // of every CTA gather from stays in L2.  A segment is then one dependent step:
 // its gathers and its epilogue operands (own element, Y, w_old, f) are all
@@ -809,14 +816,16 @@ __device__ __forceinline__ void up_segments(unsigned char* smem, int64_t Dup, in
         }
         return;
     }
-    for (int64_t chunk = j; chunk < nchunk; chunk += g.gy)
-        for (int b = 0; b < nr; b += g.cap) {
-            const int nb = min(g.cap, nr - b);
-            __syncthreads();
-            stage_up_lists(smem, g.cap, g.W, r0 + b, nb, ptr, npos, list, su);
-            __syncthreads();
+    // so many rows that a chunk of them does not stay in L2 anyway: block by block,
+    // each staged once (22 sites (11,2) binary64 product 6.16 -> 5.68 ms)
+    for (int b = 0; b < nr; b += g.cap) {
+        const int nb = min(g.cap, nr - b);
+        __syncthreads();
+        stage_up_lists(smem, g.cap, g.W, r0 + b, nb, ptr, npos, list, su);
+        __syncthreads();
+        for (int64_t chunk = j; chunk < nchunk; chunk += g.gy)
             for (int r = warp; r < nb; r += nw) seg(r0 + b, r, chunk);
-        }
+    }
 }
 
 // Binary64 fixed point, resident rows.  OLD: a replayed Lanczos step, W = H f -
@@ -1196,6 +1205,17 @@ int choose_vec(int req, int64_t len, int elem_bytes, int vmax, int reserve) {
     return req;
 }
 
+// Whether a binary32 product or replayed step takes items: where a range's lists
+// do not fit in shared memory at a time, or serve one chunk of many rows, staging
+// them gains nothing (24 sites (8,2), 276 columns: 2.97 ms with resident rows, 2.51
+// with items; (12,0): 2.90, 2.71; 18 sites (9,1): 59, 55 us, but 16 sites (8,1),
+// 21 rows a range: 19, 21 us).  Rows of odd length keep the resident kernel's two
+// segments a lane (22 sites (11,2): 2.86, 3.61 ms).
+bool up_items32(const UpGrid& g, int vpl, int64_t nchunk) {
+    if (nchunk == 1) return g.rows > 48;
+    return vpl > 1 && g.rows > g.cap;
+}
+
 UpGrid up_grid_for(const hubbard_sector* H, int64_t nchunk, int ctas) {
     return make_up_grid(H->Dup, (int64_t)H->host[0].tgt.size(), H->host[0].W, nchunk, ctas);
 }
@@ -1399,18 +1419,22 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
 #undef ROWS32
 #undef ROWS32_U
     int up_grid = 0;
-    if (part != nullptr) {                                // a Lanczos step
-        up_grid = grid_cap(sms() * kStepCtas32, up_step_items(vpl, Dup, Ddn));
-#define UPS32(V)                                                                                           \
-    launch_on(pdl, k_up_step_f32<V>, up_grid, 256, 0, s, (const float*)v, Y, (float*)w, (const float*)w_old, Dup, \
-        Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U, (float)-beta, \
-        part, done, dv, hist)
-        if (vpl == 4) { UPS32(4); } else if (vpl == 2) { UPS32(2); } else { UPS32(1); }
+    const int cols = vpl == 1 ? 64 : 128;                 // of a resident-row segment
+    const int64_t nchunk = (Ddn + cols - 1) / cols;
+    const UpGrid g = up_grid_for(H, nchunk, sms() * 4);
+    if (part != nullptr || up_items32(g, vpl, nchunk)) {
+        up_grid = grid_cap(sms() * up32_ctas(vpl, part != nullptr), up_step_items(vpl, Dup, Ddn));
+#define UPS32(V, RED)                                                                                      \
+    launch_on(pdl, k_up_step_f32<V, RED>, up_grid, 256, 0, s, (const float*)v, Y, (float*)w, (const float*)w_old, \
+        Dup, Ddn, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U,       \
+        (float)-beta, part, done, dv, hist)
+#define UPS32_R(V) if (part != nullptr) { UPS32(V, true); } else { UPS32(V, false); }
+        if (vpl == 4) { UPS32_R(4) } else if (vpl == 2) { UPS32_R(2) } else { UPS32_R(1) }
+#undef UPS32_R
 #undef UPS32
     } else {
 #define UP32(V, NV)                                                                                        \
     {                                                                                                      \
-        const UpGrid g = up_grid_for(H, (Ddn + 32 * V * NV - 1) / (32 * V * NV), sms() * 4);               \
         launch_on(pdl, k_up_f32<V, NV>, g.gx * g.gy, 256, g.smem, s, (const float*)v, Y, (float*)w,         \
             (const float*)w_old, Dup, Ddn, g, up.pn_ptr, up.pn_npos, up.pn_list, up.states, dn.states,      \
             (float)-H->t, (float)H->U, (float)-beta);                                                      \

@@ -46,5 +46,7 @@ def test_no_more_ctas_than_asked_for(grid, ctas):
                     gx, gy, cap, w, smem = grid(Dup, hops, W, nchunk, ctas)
                     assert gx >= 1 and 1 <= gy <= nchunk and gx <= Dup
                     assert gx * gy <= ctas, (ns, nup, ndn, cols)
+                    rounds = -(-nchunk // gy)           # chunks of a CTA: dealt evenly
+                    assert gy == -(-nchunk // rounds)
                     assert 1 <= cap <= Dup and w >= max(W, 1)
                     assert smem == cap * (12 + 4 * w) and (cap == 1 or smem <= 24 * 1024)
