@@ -9,7 +9,7 @@ pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(),
 # exponent found by the row phase; by a pass of its own (even rows, odd rows, long
 # rows, more than 2.5e6 elements); by one word that a memset sets back
 SECTORS = [("ring8", 4, 4), ("sq3x3", 4, 5), ("ring12", 6, 6), ("ring13", 6, 5), ("ring18", 1, 9), ("sq4x4", 5, 5),
-           ("ring15", 7, 5)]
+           ("ring15", 7, 5), ("ring18", 3, 8)]
 
 
 def _sector(lattice, nup, ndn, U=4.0):
