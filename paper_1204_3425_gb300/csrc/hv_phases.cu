@@ -713,6 +713,79 @@ __global__ void __launch_bounds__(256, up32_ctas(VPL, RED)) k_up_step_f32(const 
     }
 }
 
+// Binary32 product or replayed step of the largest vectors (up_lean32): items as
+// above, with as few requests in flight as a row takes -- the rest of a hop list
+// one by one, epilogue operands after the sum.  On gigabytes the CTAs of faster
+// forms drift apart and their chunks no longer share L2 (18 sites (8,9), 8.5 GB a
+// vector: 24.4 ms, 27.3 with resident rows, 29.2 with items that request the rest
+// at once; (9,7) 17.9, 18.9, 21.6).  Launched alone, behind the row phase: loads
+// take the read-only path.
+__global__ void __launch_bounds__(256, kStepCtas32) k_up_lean_f32(const float* __restrict__ v, const float* __restrict__ Y,
+                                                                float* w, const float* w_old, int64_t Dup, int64_t Ddn,
+                                                                const int32_t* __restrict__ ptr,
+                                                                const int32_t* __restrict__ npos,
+                                                                const uint32_t* __restrict__ list,
+                                                                const uint32_t* __restrict__ su,
+                                                                const uint32_t* __restrict__ sd, float mt, float U,
+                                                                float mbeta) {
+    constexpr int VPL = 4, CC = 32 * VPL;
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+    const int64_t nchunk = (Ddn + CC - 1) / CC;
+    const int64_t nrb = (Dup + kUpRows - 1) / kUpRows;
+    int64_t chunk = blockIdx.x / nrb, rb = blockIdx.x % nrb;
+    const int64_t dch = gridDim.x / nrb, drb = gridDim.x % nrb;
+    for (; chunk < nchunk; chunk += dch, rb += drb) {
+        if (rb >= nrb) {
+            rb -= nrb;
+            ++chunk;
+            if (chunk >= nchunk) break;
+        }
+        const int64_t c_raw = chunk * CC + (int64_t)lane * VPL;
+        const bool act = c_raw < Ddn;
+        const int64_t c = act ? c_raw : Ddn - VPL;
+        uint32_t sdc[VPL];
+#pragma unroll
+        for (int j = 0; j < VPL; ++j) sdc[j] = sd[c + j];
+        const float* base = v + c;
+        const int64_t uend = min(rb * kUpRows + kUpRows, Dup);
+        for (int64_t u = rb * kUpRows + warp; u < uend; u += nw) {
+            const int32_t kb = ptr[u];
+            const int n = ptr[u + 1] - kb, np = npos[u];
+            const int64_t J = u * Ddn + c;
+            float4 P{}, N{};
+            for (int k0 = 0; k0 < n; k0 += 32) {          // the order of uniform_hops
+                const int nk = min(32, n - k0), pend = max(0, min(nk, np - k0));
+                const uint32_t mine = lane < nk ? __ldg(list + kb + k0 + lane) : 0u;
+                auto load = [&](int q) {
+                    const uint32_t t = __shfl_sync(0xffffffffu, mine, q);
+                    return __ldg(reinterpret_cast<const float4*>(base + (int64_t)t * Ddn));
+                };
+                auto four = [&](float4& A, int q) {
+                    const float4 a = load(q), b = load(q + 1), x = load(q + 2), y = load(q + 3);
+                    addf(A, a, b, x, y);
+                };
+                int q = 0;
+                for (; q + 4 <= pend; q += 4) four(P, q);
+                for (; q < pend; ++q) addf(P, load(q));
+                for (; q + 4 <= nk; q += 4) four(N, q);
+                for (; q < nk; ++q) addf(N, load(q));
+            }
+            if (!act) continue;
+            const uint32_t su_u = su[u];
+            const float4 xo = __ldg(reinterpret_cast<const float4*>(v + J));
+            const float4 yv = __ldcs(reinterpret_cast<const float4*>(Y + J));
+            float r[VPL];
+#pragma unroll
+            for (int j = 0; j < VPL; ++j) {
+                const float nd = (float)__popc(su_u & sdc[j]);
+                r[j] = fmaf(mt, (comp(P, j) - comp(N, j)) + comp(yv, j), U * nd * comp(xo, j));
+                if (w_old != nullptr) r[j] = fmaf(mbeta, w_old[J + j], r[j]);
+            }
+            __stcs(reinterpret_cast<float4*>(w + J), make_float4(r[0], r[1], r[2], r[3]));
+        }
+    }
+}
+
 // Up phase with resident rows: a warp builds one row segment of 32 * VPL * NV
 // columns with lanes over columns, as above, but the rows belong to the CTA.
 //
@@ -1216,6 +1289,12 @@ bool up_items32(const UpGrid& g, int vpl, int64_t nchunk) {
     return vpl > 1 && g.rows > g.cap;
 }
 
+// Whether a binary32 product or replayed step takes k_up_lean_f32: 16-byte columns
+// and vectors of more than 2 GiB (18 sites (5,9), 1.7 GB: 4.59 ms, 4.38 with resident
+// rows; (6,9), 3.6 GB: 10.16, 10.78; narrower columns gain with resident rows at any
+// size, (9,8), 8.5 GB: 28.7 ms, 32.2 with items).
+bool up_lean32(int64_t D, int vpl) { return vpl == 4 && D * 4 > (2ll << 30); }
+
 UpGrid up_grid_for(const hubbard_sector* H, int64_t nchunk, int ctas) {
     return make_up_grid(H->Dup, (int64_t)H->host[0].tgt.size(), H->host[0].W, nchunk, ctas);
 }
@@ -1422,7 +1501,11 @@ int launch_hv_phases(hubbard_sector* H, const void* v, void* w, int dtype, doubl
     const int cols = vpl == 1 ? 64 : 128;                 // of a resident-row segment
     const int64_t nchunk = (Ddn + cols - 1) / cols;
     const UpGrid g = up_grid_for(H, nchunk, sms() * 4);
-    if (part != nullptr || up_items32(g, vpl, nchunk)) {
+    if (part == nullptr && up_lean32(H->D, vpl)) {
+        up_grid = grid_cap(sms() * kStepCtas32, up_step_items(vpl, Dup, Ddn));
+        k_up_lean_f32<<<up_grid, 256, 0, s>>>((const float*)v, Y, (float*)w, (const float*)w_old, Dup, Ddn, up.pn_ptr,
+            up.pn_npos, up.pn_list, up.states, dn.states, (float)-H->t, (float)H->U, (float)-beta);
+    } else if (part != nullptr || up_items32(g, vpl, nchunk)) {
         up_grid = grid_cap(sms() * up32_ctas(vpl, part != nullptr), up_step_items(vpl, Dup, Ddn));
 #define UPS32(V, RED)                                                                                      \
     launch_on(pdl, k_up_step_f32<V, RED>, up_grid, 256, 0, s, (const float*)v, Y, (float*)w, (const float*)w_old, \
