@@ -11,7 +11,7 @@ import pytest
 torch = pytest.importorskip("torch")
 pytestmark = [pytest.mark.gpu, pytest.mark.skipif(not torch.cuda.is_available(), reason="needs a CUDA GPU")]
 GIB = 1 << 30
-SLACK = 128 << 20                                       # tables, scratch and the driver's own
+SLACK = 128 << 20                                       # tables, scratch and CUDA's own
 
 
 def _sector():
